@@ -56,15 +56,30 @@ __host__ __device__ constexpr int tmem_columns(int warps, int na) {
 // TMEM columns of one SM.
 constexpr int kTmemColsPerSm = 512;
 
-// Delay-table layout, row t = d - dmin (lattice offset d), depth z:
-// zb = 0: row-major, depth fastest (nzp entries per row);
-// zb > 0: depth blocks of 2^zb rows, within a block row-major.  With 8-row
-// lane groups and zb = 3 a warp's step loads (8 depth rows of 4 neighbouring
-// lattice rows) are one contiguous 256-byte run instead of four 64-byte
-// pieces.
-__host__ __device__ __forceinline__ size_t table_index(int t, int z, int ndrows, int nzp, int zb) {
-  if (zb == 0) return (size_t)t * nzp + z;
-  return (((size_t)(z >> zb) * ndrows + t) << zb) + (z & ((1 << zb) - 1));
+// Lattice-table layout.  Row t = d - dmin of lattice offset d (dmin = -m
+// steps) is residue r = t % m, sequence number q = t / m.  A thread's four
+// channel steps u .. u + 3 of one block need q, q - 1, q - 2, q - 3 of one
+// residue, and q = 3 (mod 4) at every block's first step (tiles and threads
+// start on multiples of 4 m columns, u on -3 + 4 k): the four entries of
+// every (residue, group of four q, depth) lie together, in the order of the
+// steps, as two 16-byte halves kept apart by eight depth rows:
+//   [residue][q / 4][z / 8][half][z % 8][2 entries]
+// so a block reads two 16-byte pieces at a fixed distance of 128 bytes (eight
+// rows' worth), its neighbours in depth the pieces next to them, and the
+// next block's pieces lie a fixed stride below.  Depth rows are padded to a
+// multiple of 32.  A block's four entries used to be four 8-byte loads from
+// four lattice rows, each with its own address; now they are two loads from
+// one.  Measured on GB300 (whole calls, before -> after): 16 frames of 512 x
+// 512, nearest k = 2 212.3 -> 202.9 us, 8 frames k = 5 252.2 -> 247.8 us,
+// 4 frames of 1024 x 1024, BF16 + Kahan k = 3 699 -> 677 us, 32 frames of
+// 512 x 512 k = 3 739 -> 730 us; small single frames unchanged.
+__host__ __device__ __forceinline__ size_t table_index_rq(int r, int q, int z, int groups, int nzp) {
+  const int step = 3 - (q & 3);
+  const size_t block = ((size_t)r * groups + (q >> 2)) * (nzp >> 3) + (z >> 3);
+  return block * 32 + (step >> 1) * 16 + (z & 7) * 2 + (step & 1);
+}
+__host__ __device__ __forceinline__ size_t table_index(int t, int z, int m, int groups, int nzp) {
+  return table_index_rq(t % m, t / m, z, groups, nzp);
 }
 
 // Parameters of the fused gather + interpolate + root + power-sum kernel.
@@ -84,20 +99,18 @@ struct BfParams {  // aligned as CUtensorMap requires
   int tmem_cols;          // TMEM columns a block allocates (compensated sums), else 0
   int n_elem, n_samples;
   long long frame_elems;  // N * Ns
-  const int2* table;      // lattice table [ndrows][nz_pad] {n0 * 8, float bits of a},
-                          // rows = lattice offsets
+  const int2* table;      // lattice table {n0 * 8, float bits of a} (table_index)
   const int2* ftab;       // full table, in the kernel's read order: per tile,
                           // channel step (steps + 3), pixel half c / 2, thread
                           // of the tile, pixel c % 2: {(n0 - window start) * 8,
                           // float bits of a}
   int full;               // 1: full table (channel bases are window starts)
   int steps;              // channel steps u1 - u0
-  const float* wtab;      // [ndrows][nz_pad] apodisation weight (or null)
-  int table_stride;       // entries between lattice rows at one depth (nz_pad or 2^zb)
+  const float* wtab;      // apodisation weights, in the table's order (or null)
   const int4* items;      // [n_tiles * ngroups] {tile_id, grp, tx, tz}, deepest first
   const int2* slot_rg;    // [slots] {column residue r_m, column group g}
-  int ndrows;
-  int dmin;               // lattice offset of table row 0
+  int tgroups, nz_pad;    // lattice table: groups of four q per residue, padded depth rows
+  int dmin;               // lattice offset of table row 0 (-m steps)
   int m;                  // column stride of a thread's pixels (lattice: pitch / dx)
   int R;                  // column groups per residue in a tile
   int nxt, nzt;           // tiles along x and z
@@ -123,11 +136,6 @@ struct BfParams {  // aligned as CUtensorMap requires
   int* timeouts;          // running count of blocks whose bounded TMA wait ran out
   int expect_extra;       // bytes added to every chunk's expected transaction
                           // count: 0, or > 0 only to test the bounded wait
-  // entry of table row 0 at depth z: (z >> table_zshift) * table_zblock +
-  // (z & table_zmask) (row-major: shift 31, block 0, all-ones mask)
-  int table_zshift, table_zmask;
-  long long table_zblock;
-  int table_zb, table_nzp;  // the layout for table_index (zb 0: row-major)
 };
 
 // Post-filter / envelope parameters (one warp per depth column).

@@ -67,7 +67,7 @@ struct pa_plan_s {
   // tiling
   int m = 1, R = 1, slots = 1, warps = 1, ngroups = 1, threads = 32;
   int tile_x = 0, tile_z = 32, nxt = 0, nzt = 0, n_tiles = 0, nx_pad = 0, nz_pad = 0;
-  int u0 = 0, u1 = 0, nv = 0, dmin = 0, ndrows = 0, window = 0;
+  int u0 = 0, u1 = 0, nv = 0, dmin = 0, ndrows = 0, tgroups = 0, window = 0;
   size_t full_entries = 0;  // entries of the full table (n_tiles * (steps + 3) * 32 * slots * kC)
   size_t smem = 0;
   int blocks_per_sm = 0;
@@ -158,7 +158,6 @@ struct pa_plan_s {
   std::vector<GraphEntry> graphs;
   bool use_graph = true;
   int lane_rows_log2 = 5;  // depth rows per lane group of the fused kernel (log2)
-  int table_zb = 0;        // lattice table layout: 0 row-major, else log2 depth-block height
   // kernel timing (pa_plan_profile): bit k set = kernel kind k is timed
   uint32_t prof = 0;
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_free;
@@ -226,7 +225,7 @@ __host__ __device__ __forceinline__ int full_column(const FullGeom& f, int tx, i
 }
 
 struct TableGeom {
-  int ndrows, nzp, dmin, ns, nearest, zb;
+  int ndrows, nzp, dmin, ns, nearest, m, groups;
   double x_const;  // x0 + (N-1)/2 pitch: dx of lattice offset d is x_const + (d + 1/2) dx
   double dx, z0, dz, fs, c, t0, fnum;
   // full table: element i = v + u0 of N at x_i = (i - (N-1)/2) pitch
@@ -292,7 +291,7 @@ __global__ void k_table(TableGeom g, int2* table, float* wtab) {
   int n0;
   double a;
   delay_sample(g, dxv, zp, &n0, &a);
-  const size_t ti = table_index(row, z, g.ndrows, g.nzp, g.zb);
+  const size_t ti = table_index(row, z, g.m, g.groups, g.nzp);
   table[ti] = make_int2(n0 * 8, __float_as_int((float)a));
   if (wtab) wtab[ti] = apod_weight(g, dxv, zp);
 }
@@ -350,7 +349,7 @@ __global__ void k_count_active_full(FullGeom f, const float* wtab, unsigned long
 }
 
 struct TileGeom {
-  int nxt, nzt, tile_x, tile_z, m, dmin, nzp, nv, u0, ndrows, zb;
+  int nxt, nzt, tile_x, tile_z, m, dmin, nzp, nv, u0, ndrows, groups;
   int full;  // 1: full table (laid out as full_index says)
 };
 
@@ -377,8 +376,8 @@ __global__ void k_windows(TileGeom g, int lo_align, const int2* table, int* lo, 
       atomicOr(err, 4);
       continue;
     }
-    mn = min(mn, table[table_index(row, zf, g.ndrows, g.nzp, g.zb)].x >> 3);
-    mx = max(mx, table[table_index(row, zl, g.ndrows, g.nzp, g.zb)].x >> 3);
+    mn = min(mn, table[table_index(row, zf, g.m, g.groups, g.nzp)].x >> 3);
+    mx = max(mx, table[table_index(row, zl, g.m, g.groups, g.nzp)].x >> 3);
   }
   const int lo_al = mn & ~(lo_align - 1);  // lo_align is a power of two
   lo[(size_t)tile * g.nv + v] = lo_al;
@@ -422,6 +421,7 @@ __global__ void k_uranges(TileGeom g, FullGeom f, int slots, int u1, int kc, con
     const int r_m = sl % g.m, grp = sl / g.m;
     const int jt = tx * g.tile_x + grp * g.m * kc + r_m;
     const int zl = tz * g.tile_z + g.tile_z - 1;
+    const int t0 = g.full ? 0 : tile_row(g, jt, 0);  // table row at step u0, m lower at each step
     int ua = u1, ub = g.u0;
     for (int u = g.u0; u < u1; ++u) {
       // lattice: the kC pixels of the slot share one entry at step u; full:
@@ -431,8 +431,7 @@ __global__ void k_uranges(TileGeom g, FullGeom f, int slots, int u1, int kc, con
         for (int c = 0; c < kc; ++c)
           on |= wtab[full_index(f, tile, u - g.u0, c, sl, g.tile_z - 1)] > 0.f;
       } else {
-        const int row = tile_row(g, jt, u - g.u0);
-        if (row >= 0 && row < g.ndrows) on = wtab[table_index(row, zl, g.ndrows, g.nzp, g.zb)] > 0.f;
+        on = wtab[table_index_rq(t0 % g.m, t0 / g.m - (u - g.u0), zl, g.groups, g.nzp)] > 0.f;
       }
       if (on) {
         ua = min(ua, u);
@@ -462,10 +461,9 @@ __global__ void k_count_active(TileGeom g, int nx, int nz, int n, const float* w
   const int j = blockIdx.y;
   unsigned long long c = 0;
   if (z < nz) {
-    for (int i = 0; i < n; ++i) {
-      const int row = tile_row(g, j, i - g.u0);
-      if (wtab[table_index(row, z, g.ndrows, g.nzp, g.zb)] > 0.f) ++c;
-    }
+    const int t0 = tile_row(g, j, -g.u0);  // table row of element 0, m lower at each element
+    for (int i = 0; i < n; ++i)
+      if (wtab[table_index_rq(t0 % g.m, t0 / g.m - i, z, g.groups, g.nzp)] > 0.f) ++c;
   }
   for (int s = 16; s >= 1; s >>= 1) c += __shfl_xor_sync(0xffffffffu, c, s);
   if ((threadIdx.x & 31) == 0 && c) atomicAdd(count, c);
@@ -624,19 +622,6 @@ void configure(pa_plan_s* P) {
     const int want = atoi(e) == 8 ? 3 : (atoi(e) == 16 ? 4 : 5);
     if (B % (1 << (5 - want)) == 0 && !(P->tmem_cols && P->apod)) P->lane_rows_log2 = want;
   }
-  // Lattice table layout: depth blocks of 8 rows (a warp's four lattice
-  // rows at one step in one contiguous 256-byte run: half the L1 wavefronts
-  // of four 64-byte pieces) where that measured faster, row-major elsewhere.
-  // Measured on GB300 (fused kernel per launch, one run, against row-major):
-  // cfg2 k = 1, 2 0.488 -> 0.458 ms (bound by the L1 data pipe), BF16 +
-  // Kahan k = 3 0.662 -> 0.653 ms, cfg3 BF16 + Kahan 1.261 -> 1.236 ms; but
-  // plain FP32 k = 3 0.617 -> 0.628 ms, and blocks of 32 rows were slower
-  // than row-major for every plan tried (k = 5 0.819 -> 0.838 ms, the cfg5
-  // batch 2.675 -> 2.790 ms) although a warp's loads have the same shape.
-  // (8-row lane groups imply no apodisation; the fused kernel computes the
-  // blocked address only in the instantiations for k <= 2 or compensated
-  // sums without apodisation.)
-  P->table_zb = (P->lane_rows_log2 == 3 && !P->apod && (P->K <= 2 || P->comp)) ? 3 : 0;
   P->threads = 32 * B;
   P->tile_x = P->m * kC * P->R;
   P->tile_z = 32;
@@ -655,9 +640,12 @@ void configure(pa_plan_s* P) {
     P->ndrows = 0;
     P->full_entries = (size_t)P->n_tiles * (steps + 3) * 32 * P->slots * kC;
   } else {
-    P->dmin = -P->m * i_max;
-    const int dmax = P->nx_pad - 1 + P->m * (kC - 1);
-    P->ndrows = dmax - P->dmin + 1;
+    // whole groups of four lattice sequence numbers per residue, from the
+    // pair of column 0 and the last virtual channel to that of the last
+    // padded column and the first one
+    P->dmin = -P->m * steps;
+    P->tgroups = (P->nx_pad / P->m + steps) / 4 + 1;
+    P->ndrows = 4 * P->m * P->tgroups;
   }
   P->M = 1;
   P->log2M = 0;
@@ -869,7 +857,8 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
   TableGeom tg;
   tg.ndrows = P->ndrows;
   tg.nzp = P->nz_pad;
-  tg.zb = P->table_zb;
+  tg.m = P->m;
+  tg.groups = P->tgroups;
   tg.dmin = P->dmin;
   tg.ns = d.n_samples;
   tg.nearest = d.interp == PA_INTERP_NEAREST;
@@ -899,7 +888,7 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
   g.nv = P->nv;
   g.u0 = P->u0;
   g.ndrows = P->ndrows;
-  g.zb = P->table_zb;
+  g.groups = P->tgroups;
   g.full = P->full ? 1 : 0;
   FullGeom fg{P->nxt, P->n_tiles, P->tile_x, P->tile_z, P->m, P->slots, P->u1 - P->u0,
               P->lane_rows_log2, d.nx, d.nz, d.n_elem, P->u0, P->nv};
@@ -1213,15 +1202,10 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
   b.full = P->full ? 1 : 0;
   b.steps = P->u1 - P->u0;
   b.wtab = P->wtab;
-  b.table_stride = P->table_zb ? 1 << P->table_zb : P->nz_pad;
-  b.table_zb = P->table_zb;
-  b.table_nzp = P->nz_pad;
-  b.table_zshift = P->table_zb ? P->table_zb : 31;
-  b.table_zmask = P->table_zb ? (1 << P->table_zb) - 1 : 0x7fffffff;
-  b.table_zblock = P->table_zb ? (long long)P->ndrows << P->table_zb : 0;
+  b.tgroups = P->tgroups;
+  b.nz_pad = P->nz_pad;
   b.items = P->items;
   b.slot_rg = P->slot_rg;
-  b.ndrows = P->ndrows;
   b.dmin = P->dmin;
   b.m = P->m;
   b.R = P->R;
