@@ -1,0 +1,4 @@
+// Order 2 of the two-frame fused beamforming kernel.
+#include "pa_bf_pipe.cuh"
+
+PA_DEFINE_PIPE(2)

@@ -43,15 +43,29 @@ constexpr int kLoOff = kCbOff + kCbInts * 4;
 constexpr int kRawOff = 640;  // >= kLoOff + 4 kCbInts, 128-byte aligned
 static_assert(kRawOff >= kLoOff + kCbInts * 4 && kRawOff % 128 == 0, "shared layout");
 constexpr int kMaxThreads = 1024;
+// Shared-memory layout of the two-frame kernel: the stages' mbarriers and
+// counts of finished warps, TMEM address, stop flag, the running work item,
+// then per stage 32 bytes of work-item words and the channel bases, then the
+// stages' slots (128-byte aligned).
+constexpr int kPipeStages = 4;  // at most
+constexpr int kPipeFullOff = 0, kPipeCountOff = 32, kPipeTmemOff = 48, kPipeStopOff = 52;
+constexpr int kPipeProdOff = 64;
+constexpr int kPipeMetaOff = 96;
+constexpr int kPipeCbOff = kPipeMetaOff + 32 * kPipeStages;
+constexpr int kPipeSlotOff = 1536;
+static_assert(kPipeSlotOff >= kPipeCbOff + kPipeStages * kCbInts * 4 && kPipeSlotOff % 128 == 0,
+              "shared layout");
 
 // TMEM columns a fused-kernel block allocates for compensated totals (a
 // power of two >= 32): the warps sharing a 32-lane quarter of TMEM times 8
-// columns per accumulator (kC totals and kC compensation terms).
+// columns per accumulator (kC totals and kC compensation terms; na counts the
+// accumulators of every frame of a work item).
 __host__ __device__ constexpr int tmem_columns(int warps, int na) {
   return ((warps + 3) / 4) * na * 8 <= 32    ? 32
          : ((warps + 3) / 4) * na * 8 <= 64  ? 64
          : ((warps + 3) / 4) * na * 8 <= 128 ? 128
-                                              : 256;
+         : ((warps + 3) / 4) * na * 8 <= 256 ? 256
+                                              : 512;
 }
 // TMEM columns of one SM.
 constexpr int kTmemColsPerSm = 512;
@@ -130,13 +144,43 @@ struct BfParams {  // aligned as CUtensorMap requires
   int plane_das, plane_dmas, plane_ho;  // raw plane of each output or -1
   int nx, nz;
   int n_frames;           // frames in this launch
-  int n_items;            // n_tiles * n_frames
+  int n_items;            // n_tiles * ngroups * n_frames (two-frame kernel: * n_fgroups)
+  // two-frame kernel
+  int n_fgroups;          // frame pairs (ceil(n_frames / 2))
+  int stages;             // chunks of slots in shared memory
+  const unsigned char* slots_dev;  // prepared slots (k_prep): a row of zeros,
+                                   // then [frame pair][channel] rows of
+                                   // slot_pitch slots
+  long long slot_pitch;
+  int slot_margin;        // zero slots before a row's sample 0
   int* counter;           // work counter (zeroed before launch)
   int* err;               // error flags: 1, 2 index checks (checked builds), 8 a wait ran out
   int* timeouts;          // running count of blocks whose bounded TMA wait ran out
   int expect_extra;       // bytes added to every chunk's expected transaction
                           // count: 0, or > 0 only to test the bounded wait
 };
+
+// A kernel launch described as data (direct launch or CUDA-graph node).
+struct LaunchSpec {
+  const void* func = nullptr;
+  dim3 grid, block;
+  size_t smem = 0;
+};
+
+// Preparation pass of the two-frame kernel (pa_prep.cu).
+struct PrepParams {
+  const void* rf;      // [frames][N][Ns]
+  unsigned char* slots;  // as BfParams::slots_dev
+  long long pitch;
+  int margin;
+  int rf_dtype, n_elem, n_samples, n_frames;
+  int n_lo, n_hi;      // samples the windows hold
+  int blocks_per_row;
+  int mode, order;     // slot kind (PipeMode), order of its roots
+  int* zero;           // words cleared before the fused kernel (work counter, maxima)
+  int n_zero;
+};
+void prep_spec(PrepParams* p, LaunchSpec* s);
 
 // Post-filter / envelope parameters (one warp per depth column).
 struct PostParams {
@@ -162,14 +206,10 @@ struct LogParams {
   int n_frames;
 };
 
-// A kernel launch described as data (direct launch or CUDA-graph node).
-struct LaunchSpec {
-  const void* func = nullptr;
-  dim3 grid, block;
-  size_t smem = 0;
-};
-
 const void* bf_func(int order, bool apod, bool comp, bool full);
+int pipe_slot_mode(int order, bool apod, bool nearest);  // PipeMode
+int pipe_slot_bytes(int mode);
+const void* bf_pipe_func(int order, bool apod, bool comp, bool full, bool nearest);
 void post_spec(const PostParams& p, LaunchSpec* s);
 // Radix of the first FFT pass of the in-place post kernel (the passes after
 // it are radix 8, then one radix-4 or radix-2 pass for the remainder); the
@@ -184,19 +224,12 @@ const void* post_inplace_func(int m);  // in-place kernel for M points, or nullp
 int post_team_warps(int m);  // warps per team (column pair) of the post kernel
 void log_spec(const LogParams& p, int num_sms, LaunchSpec* s);
 
-// Launchers (one translation unit per order keeps the builds parallel).
-cudaError_t bf_launch(int order, bool apod, bool comp, bool full, const BfParams& p,
-                      int grid, int block, size_t smem, cudaStream_t s);
-cudaError_t bf_occupancy(int order, bool apod, bool comp, bool full, int block,
-                         size_t smem, int* blocks_per_sm);
+cudaError_t bf_occupancy(const void* func, int block, size_t smem, int* blocks_per_sm);
 
-#define PA_DECLARE_ORDER(K)                                                 \
-  cudaError_t bf_launch_k##K(bool apod, bool comp, bool full,               \
-                             const BfParams& p, int grid, int block,        \
-                             size_t smem, cudaStream_t s);                  \
-  cudaError_t bf_occupancy_k##K(bool apod, bool comp, bool full, int block, \
-                                size_t smem, int* blocks_per_sm);           \
-  const void* bf_func_k##K(bool apod, bool comp, bool full);
+// One translation unit per order keeps the builds parallel.
+#define PA_DECLARE_ORDER(K) const void* bf_func_k##K(bool apod, bool comp, bool full);
+#define PA_DECLARE_PIPE(K) \
+  const void* bf_pipe_func_k##K(bool apod, bool comp, bool full, bool nearest);
 PA_DECLARE_ORDER(1)
 PA_DECLARE_ORDER(2)
 PA_DECLARE_ORDER(3)
@@ -205,7 +238,13 @@ PA_DECLARE_ORDER(5)
 PA_DECLARE_ORDER(6)
 PA_DECLARE_ORDER(7)
 PA_DECLARE_ORDER(8)
+PA_DECLARE_PIPE(1)
+PA_DECLARE_PIPE(2)
+PA_DECLARE_PIPE(3)
+PA_DECLARE_PIPE(4)
+PA_DECLARE_PIPE(5)
 #undef PA_DECLARE_ORDER
+#undef PA_DECLARE_PIPE
 
 // Sets the thread-local message returned by pa_last_error().
 void set_error_message(const char* msg);

@@ -58,6 +58,23 @@ struct DeviceGuard {
 // Buffer sets (and streams) of the host-buffer path.
 constexpr int kHostSets = 3;
 
+// One form of the fused kernel and the shared-memory geometry that goes with
+// it: form 0 runs one frame per work item (pa_bf_kernel.cuh), form 1 two
+// frames from prepared slots (pa_bf_pipe.cuh).
+struct FusedForm {
+  int nf = 0;             // frames per work item (0: the plan has no such form)
+  const void* func = nullptr;
+  int threads = 0;
+  int nc = 32;            // channel steps per staged chunk (multiple of kC)
+  int stages = 1;         // chunks in shared memory at once (two-frame form)
+  int rp = 0;             // raw-buffer row pitch in samples (128-byte aligned rows)
+  int pairs_off = 0;      // shared-memory offset of the interpolation slots
+  size_t smem = 0;
+  int blocks_per_sm = 0;
+  int tmem_cols = 0;      // TMEM columns per block (compensated sums)
+  int2* vchunks = nullptr;  // [n_tiles * ngroups] chunk range of a work item
+};
+
 struct pa_plan_s {
   pa_plan_desc d{};
   int device = 0, num_sms = 0;
@@ -69,17 +86,20 @@ struct pa_plan_s {
   int tile_x = 0, tile_z = 32, nxt = 0, nzt = 0, n_tiles = 0, nx_pad = 0, nz_pad = 0;
   int u0 = 0, u1 = 0, nv = 0, dmin = 0, ndrows = 0, tgroups = 0, window = 0;
   size_t full_entries = 0;  // entries of the full table (n_tiles * (steps + 3) * 32 * slots * kC)
-  size_t smem = 0;
-  int blocks_per_sm = 0;
+  FusedForm form[2];
+  // prepared slots of the two-frame form: a row of zeros, then one row of
+  // slot_pitch slots per (frame pair, channel), for ws_frames frames a round
+  unsigned char* slots_dev = nullptr;
+  long long slot_pitch = 0;
+  int used_lo = 0, used_hi = 0;  // samples [used_lo, used_hi) lie in some window
+  int slot_margin = 0, slot_mode = 0, slot_bytes = 16, ws_frames = 0;
   bool use_tma = false;
   int lo_align = 4;   // window starts are multiples of this many samples
-  int nc = 32;        // channel steps per staged chunk (multiple of kC)
-  int tmem_cols = 0;  // TMEM columns per fused-kernel block (compensated sums)
   int expect_extra = 0;   // > 0 only under PA_INJECT_TMA_SHORTFALL (tests the bounded wait)
   long long timeouts_seen = 0;  // timed-out waits already reported by pa_beamform_host
   int wr = 0;         // raw samples per channel delivered by one TMA box
-  int rp = 0;         // raw-buffer row pitch in samples (128-byte aligned rows)
-  int pairs_off = 0;  // shared-memory offset of the interpolation slots
+  int item_frames = 0;  // PA_ITEM_FRAMES: 1 or 2 picks the form (measurements, tests)
+  bool pairs_pay = false;  // resident warps and slot reuse of the two-frame form suffice
   // post
   int M = 1, log2M = 0, post_wpb = 1, n_out = 0, n_tw = 0;
   int out_id[3] = {-1, -1, -1};  // output slot (0..n_out) of DAS, DMAS, HO
@@ -91,7 +111,6 @@ struct pa_plan_s {
   float* wtab = nullptr;
   int* lo = nullptr;
   int2* urange = nullptr;
-  int2* vchunks = nullptr;
   int4* items = nullptr;   // work-item table (tile, group, tx, tz)
   int2* slot_rg = nullptr; // warp slot -> (column residue, column group)
   float2* tw = nullptr;
@@ -148,12 +167,11 @@ struct pa_plan_s {
     uint32_t stages = 0;
     cudaGraph_t graph = nullptr;  // kept alive: exec-node updates name its nodes
     cudaGraphExec_t exec = nullptr;
-    cudaGraphNode_t n_memset = nullptr;  // clearing kernel
-    cudaGraphNode_t n_bf = nullptr, n_post = nullptr, n_log = nullptr;
-    // timing graphs (built while pa_plan_profile is on): an event-record
-    // node before and after each kernel, given fresh events every launch
     uint32_t prof = 0;  // kernel kinds timed (bit per kind)
-    cudaGraphNode_t n_ev[3][2] = {};
+    std::vector<cudaGraphNode_t> kernels;
+    // timing graphs (built while pa_plan_profile is on): an event-record
+    // node before and after each timed kernel, given fresh events every launch
+    std::vector<cudaGraphNode_t> events;
   };
   std::vector<GraphEntry> graphs;
   bool use_graph = true;
@@ -348,6 +366,8 @@ __global__ void k_count_active_full(FullGeom f, const float* wtab, unsigned long
   if ((threadIdx.x & 31) == 0 && cnt) atomicAdd(count, cnt);
 }
 
+constexpr int kLoBias = 1 << 22;  // window starts + kLoBias > 0 (delays are clamped to +-2^20)
+
 struct TileGeom {
   int nxt, nzt, tile_x, tile_z, m, dmin, nzp, nv, u0, ndrows, groups;
   int full;  // 1: full table (laid out as full_index says)
@@ -359,11 +379,17 @@ __device__ __forceinline__ int tile_row(const TileGeom& g, int j, int v) {
   return j - g.m * (v + g.u0) - g.dmin;
 }
 
+// Largest window start and (as the largest negative) the smallest one.
+__device__ __forceinline__ void record_starts(int* lomax, int lo) {
+  atomicMax(lomax, lo + kLoBias);
+  atomicMax(lomax + 1, kLoBias - lo);
+}
+
 // First staged sample (rounded down to a multiple of 4) and window width of
 // every (tile, virtual channel).  The delay grows with depth for z > 0, so the
 // minimum over the tile is on its first row and the maximum on its last.
 __global__ void k_windows(TileGeom g, int lo_align, const int2* table, int* lo, int* wmax,
-                          int* err) {
+                          int* lomax, int* err) {
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   const int tile = blockIdx.y;
   if (v >= g.nv) return;
@@ -382,11 +408,13 @@ __global__ void k_windows(TileGeom g, int lo_align, const int2* table, int* lo, 
   const int lo_al = mn & ~(lo_align - 1);  // lo_align is a power of two
   lo[(size_t)tile * g.nv + v] = lo_al;
   atomicMax(wmax, mx - lo_al + 1);
+  record_starts(lomax, lo_al);
 }
 
 // The same windows for the full table, from the delays themselves (the
 // packed table is written relative to them afterwards).
-__global__ void k_windows_full(TableGeom tg, TileGeom g, int lo_align, int* lo, int* wmax) {
+__global__ void k_windows_full(TableGeom tg, TileGeom g, int lo_align, int* lo, int* wmax,
+                               int* lomax) {
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   const int tile = blockIdx.y;
   if (v >= g.nv) return;
@@ -405,6 +433,7 @@ __global__ void k_windows_full(TableGeom tg, TileGeom g, int lo_align, int* lo, 
   const int lo_al = mn & ~(lo_align - 1);
   lo[(size_t)tile * g.nv + v] = lo_al;
   atomicMax(wmax, mx - lo_al + 1);
+  record_starts(lomax, lo_al);
 }
 
 // Channel-step range of every warp slot.  Without apodisation every step is
@@ -617,10 +646,9 @@ void configure(pa_plan_s* P) {
   // Compensated sums keep their Kahan totals in TMEM; its accesses are
   // warp-wide, so every lane of a warp must run the same channel steps:
   // apodised plans (per-slot channel ranges) then keep one slot per warp.
-  P->tmem_cols = P->comp ? tmem_columns(B, P->K <= 2 ? 3 : P->K + 2) : 0;
   if (const char* e = getenv("PA_LANE_ROWS")) {
     const int want = atoi(e) == 8 ? 3 : (atoi(e) == 16 ? 4 : 5);
-    if (B % (1 << (5 - want)) == 0 && !(P->tmem_cols && P->apod)) P->lane_rows_log2 = want;
+    if (B % (1 << (5 - want)) == 0 && !(P->comp && P->apod)) P->lane_rows_log2 = want;
   }
   P->threads = 32 * B;
   P->tile_x = P->m * kC * P->R;
@@ -681,6 +709,16 @@ void configure(pa_plan_s* P) {
   // TMA boxes start on 16-byte boundaries: window starts are multiples of
   // 16 / elt samples, and rows must be 16-byte strided.
   P->lo_align = (int)(16 / P->elt);
+  // zero slots on either side of a prepared row: at least the widest RF
+  // window, i.e. the largest delay difference over a tile plus the rounding
+  // of its ends
+  {
+    const double dz = (d.z1_m - d.z0_m) / d.nz;
+    const double span = d.fs_hz / d.c_m_s * std::hypot(P->tile_x * dx, P->tile_z * dz);
+    P->slot_margin = ((int)std::min(span, 1e6) + P->lo_align + 8) / 4 * 4;
+    P->slot_mode = pipe_slot_mode(P->K, P->apod, d.interp == PA_INTERP_NEAREST);
+    P->slot_bytes = pipe_slot_bytes(P->slot_mode);
+  }
   // Measured on GB300: TMA staging wins for 16-bit RF (half-size raw buffer),
   // vectorised loads win for FP32 RF (the FP32 raw buffer costs a resident
   // block per SM).  PA_STAGING=tma|loads overrides the choice.
@@ -696,6 +734,7 @@ void configure(pa_plan_s* P) {
   const char* staging = getenv("PA_STAGING");
   if (staging && strcmp(staging, "loads") == 0) P->use_tma = false;
   if (staging && strcmp(staging, "tma") == 0) P->use_tma = (d.n_samples % P->lo_align) == 0;
+  if (const char* e = getenv("PA_ITEM_FRAMES")) P->item_frames = atoi(e);
   if (P->d.max_batch <= 0) P->d.max_batch = 1;
 }
 
@@ -704,11 +743,11 @@ void configure(pa_plan_s* P) {
 // and threads (the occupancy calculator reports one block per SM for a
 // kernel that allocates tensor memory) and is capped so that the resident
 // blocks' TMEM columns fit the SM's 512.
-cudaError_t fused_blocks_per_sm(const pa_plan_s* P, size_t smem, int* n) {
-  cudaError_t e = bf_occupancy(P->K, P->apod, P->comp, P->full, P->threads, smem, n);
-  if (e != cudaSuccess || !P->tmem_cols) return e;
+cudaError_t fused_blocks_per_sm(const pa_plan_s* P, const FusedForm& f, size_t smem, int* n) {
+  cudaError_t e = bf_occupancy(f.func, f.threads, smem, n);
+  if (e != cudaSuccess || !f.tmem_cols) return e;
   cudaFuncAttributes a;
-  e = cudaFuncGetAttributes(&a, bf_func(P->K, P->apod, P->comp, P->full));
+  e = cudaFuncGetAttributes(&a, f.func);
   if (e != cudaSuccess) return e;
   int dev = 0, regs_sm = 0, smem_sm = 0, thr_sm = 0, blk_sm = 0, rsv = 0;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -717,13 +756,31 @@ cudaError_t fused_blocks_per_sm(const pa_plan_s* P, size_t smem, int* n) {
   cudaDeviceGetAttribute(&thr_sm, cudaDevAttrMaxThreadsPerMultiProcessor, dev);
   cudaDeviceGetAttribute(&blk_sm, cudaDevAttrMaxBlocksPerMultiprocessor, dev);
   cudaDeviceGetAttribute(&rsv, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-  const int warps = (P->threads + 31) / 32;
+  const int warps = (f.threads + 31) / 32;
   const int regs_warp = ((a.numRegs * 32 + 255) / 256) * 256;  // 256-register units per warp
   int b = std::min(regs_sm / std::max(1, regs_warp * warps), thr_sm / (32 * warps));
   b = std::min(b, (int)((size_t)smem_sm / (smem + a.sharedSizeBytes + (size_t)rsv)));
   b = std::min(b, blk_sm);
-  *n = std::max(0, std::min(b, kTmemColsPerSm / P->tmem_cols));
+  *n = std::max(0, std::min(b, kTmemColsPerSm / f.tmem_cols));
   return cudaSuccess;
+}
+
+// Whether a plan of this descriptor gets the two-frame form (if it fits).
+bool wants_pairs(const pa_plan_s* P) {
+  return P->d.max_batch > 1 && P->K <= 5 && P->item_frames != 1;
+}
+
+// Frames per round of the two-frame form and the bytes of its slots.  The
+// slots of a round are written by k_prep and read back by every tile.
+constexpr size_t kSlotBytesMax = (size_t)512 << 20;
+size_t pair_slots(const pa_plan_s* P, int* frames, long long* pitch) {
+  *pitch = ((long long)P->d.n_samples + 1) / 2 * 2 + 2ll * P->slot_margin;  // 16-byte rows
+  const size_t row = (size_t)*pitch * P->slot_bytes;
+  const size_t per_pair = (size_t)P->d.n_elem * row;
+  size_t pairs = ((size_t)P->d.max_batch + 1) / 2;
+  pairs = std::max<size_t>(1, std::min(pairs, kSlotBytesMax / per_pair));
+  *frames = (int)(2 * pairs);
+  return row + pairs * per_pair;
 }
 
 // Bytes of the delay table and its apodisation weights.
@@ -747,6 +804,11 @@ size_t table_bytes(const pa_plan_s* P) {
   b += (size_t)P->n_tiles * P->nv * sizeof(int);
   b += (size_t)P->n_tiles * P->slots * sizeof(int2);
   b += (size_t)P->n_tiles * P->ngroups * sizeof(int2);
+  if (wants_pairs(P)) {  // chunk ranges and slots of the two-frame form
+    int frames;
+    long long pitch;
+    b += (size_t)P->n_tiles * P->ngroups * sizeof(int2) + pair_slots(P, &frames, &pitch);
+  }
   b += (size_t)2 * P->M * sizeof(float2) + (size_t)3 * P->M * sizeof(float);
   return b;
 }
@@ -789,7 +851,8 @@ void free_plan(pa_plan_s* P) {
   cudaFree(P->wtab);
   cudaFree(P->lo);
   cudaFree(P->urange);
-  cudaFree(P->vchunks);
+  for (FusedForm& f : P->form) cudaFree(f.vchunks);
+  cudaFree(P->slots_dev);
   cudaFree(P->items);
   cudaFree(P->slot_rg);
   cudaFree(P->tw);
@@ -822,6 +885,192 @@ void free_plan(pa_plan_s* P) {
   delete P;
 }
 
+// Shared memory of a fused-kernel block of form f with c channel steps per
+// chunk; *pairs_off is where its interpolation slots start.
+size_t form_smem(const pa_plan_s* P, const FusedForm& f, int c, int* pairs_off) {
+  const int ncs = c + kC - 1;
+  if (f.nf == 2) {
+    if (pairs_off) *pairs_off = kPipeSlotOff;
+    return (size_t)kPipeSlotOff + (size_t)f.stages * ncs * P->window * P->slot_bytes;
+  }
+  const size_t raw = P->use_tma ? (size_t)ncs * f.rp * P->elt : 0;
+  const size_t off = (size_t)kRawOff + ((raw + 127) & ~size_t(127));
+  if (pairs_off) *pairs_off = (int)off;
+  return off + (size_t)ncs * P->window * 8;
+}
+
+// TMEM-dense: a block can hold more than its register share of an SM's TMEM
+// columns (see plan_tmem).
+bool form_dense(const pa_plan_s* P, const FusedForm& f) {
+  if (!f.tmem_cols) return false;
+  cudaFuncAttributes a;
+  int regs_sm = 65536;
+  cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, P->device);
+  if (cudaFuncGetAttributes(&a, f.func) != cudaSuccess) {
+    cudaGetLastError();
+    return true;  // unknown: treat as dense (serialised with other compensated batches)
+  }
+  const size_t warps = (size_t)(f.threads + 31) / 32;
+  const size_t regs_block = (size_t)((a.numRegs * 32 + 255) / 256) * 256 * warps;
+  return (size_t)f.tmem_cols * (size_t)regs_sm > (size_t)kTmemColsPerSm * regs_block;
+}
+
+// Chunk range of every work item of form f, uploaded to f.vchunks.
+pa_status build_chunks(pa_plan_s* P, FusedForm& f, const std::vector<int2>& ur, cudaStream_t st) {
+  std::vector<int2> vk((size_t)P->n_tiles * P->ngroups);
+  for (int t = 0; t < P->n_tiles; ++t) {
+    for (int gr = 0; gr < P->ngroups; ++gr) {
+      int ua = P->u1, ub = P->u0;
+      for (int w = 0; w < P->warps; ++w) {
+        const int2 r = ur[(size_t)t * P->slots + gr * P->warps + w];
+        if (r.y > r.x) {
+          ua = std::min(ua, r.x);
+          ub = std::max(ub, r.y);
+        }
+      }
+      int2 c = make_int2(0, 0);
+      if (ub > ua) c = make_int2((ua - P->u0) / f.nc, (ub - P->u0 + f.nc - 1) / f.nc);
+      vk[(size_t)t * P->ngroups + gr] = c;
+    }
+  }
+  const pa_status s = dalloc(P, &f.vchunks, vk.size());
+  if (s != PA_OK) return s;
+  PA_CUDA(cudaMemcpyAsync(f.vchunks, vk.data(), vk.size() * sizeof(int2), cudaMemcpyHostToDevice,
+                          st));
+  PA_CUDA(cudaStreamSynchronize(st));  // vk is pageable and local
+  return PA_OK;
+}
+
+// The one-frame form.
+pa_status build_form1(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st) {
+  FusedForm& f = P->form[0];
+  f.nf = 1;
+  f.func = bf_func(P->K, P->apod, P->comp, P->full);
+  f.threads = P->threads;
+  f.tmem_cols = P->comp ? tmem_columns(P->warps, P->K <= 2 ? 3 : P->K + 2) : 0;
+  f.rp = (int)((((size_t)P->wr * P->elt + 127) & ~size_t(127)) / P->elt);
+  // Chunk length: every chunk costs a staging pass and two block barriers,
+  // so the channel steps are cut into as few, evenly sized chunks as keep
+  // the fused kernel's occupancy at what 32-step chunks give (measured at
+  // N = 128: 5 chunks of 28 steps 0.696 ms, 4 of 36 0.692 ms, 3 of 44
+  // 0.678 ms).  Limits: the slot buffer (at most 200 KiB), one issuing lane
+  // per staged channel under TMA (ncs <= 32 warps), and the multiply-shift
+  // division of the staging loops (exact while ncs * (W/4)^2 < 2^20).
+  // PA_CHUNK_STEPS caps the chunk length (for measurements).
+  const int steps = P->u1 - P->u0;
+  auto fits = [&](int c) {
+    const int ncs = c + kC - 1;
+    const long long w4 = P->window / 4;
+    return form_smem(P, f, c, nullptr) <= 200 * 1024 && ncs <= 32 * P->warps &&
+           (long long)ncs * w4 * w4 < (1ll << 20);
+  };
+  auto occupancy = [&](int c) {
+    int b = 0;
+    if (fused_blocks_per_sm(P, f, form_smem(P, f, c, nullptr), &b) != cudaSuccess) b = 0;
+    return b;
+  };
+  auto even = [&](int nch) { return ((steps + nch - 1) / nch + kC - 1) / kC * kC; };
+  int cap = kNCMax;
+  if (const char* e = getenv("PA_CHUNK_STEPS")) cap = std::max(kC, std::min(kNCMax, atoi(e)));
+  int ref = std::min(32, cap);
+  while (ref > kC && !fits(ref)) ref -= kC;
+  const int occ_ref = occupancy(ref);
+  int nc = ref;
+  for (int nch = (steps + cap - 1) / cap; nch <= (steps + ref - 1) / ref; ++nch) {
+    const int c = std::min(even(nch), cap);
+    if (c > ref && fits(c) && occupancy(c) >= occ_ref) {
+      nc = c;
+      break;
+    }
+  }
+  if (nc == ref) nc = std::min(ref, even((steps + ref - 1) / ref));
+  f.nc = nc;
+  cudaGetLastError();
+
+  // shared memory and occupancy of the fused kernel
+  f.smem = form_smem(P, f, f.nc, &f.pairs_off);
+  const long long w4 = P->window / 4;
+  if ((long long)(f.nc + kC - 1) * w4 * w4 >= (1ll << 20))
+    return fail(PA_EUNSUPPORTED, "RF window of %d samples per channel is too wide; use a finer "
+                "depth grid", P->window);
+  if (f.smem > 200 * 1024)
+    return fail(PA_EUNSUPPORTED,
+                "RF window of %d samples per channel needs %zu B of shared memory; use a finer "
+                "depth grid",
+                P->window, f.smem);
+  // (resident blocks never ask for more TMEM than an SM has, so no block's
+  // allocation waits on another block of the same launch)
+  PA_CUDA(fused_blocks_per_sm(P, f, f.smem, &f.blocks_per_sm));
+  if (f.blocks_per_sm < 1)
+    return fail(PA_EUNSUPPORTED, "fused kernel does not fit an SM (%d threads, %zu B smem)",
+                P->threads, f.smem);
+  return build_chunks(P, f, ur, st);
+}
+
+// The two-frame form; a plan it does not fit keeps the one-frame form alone.
+pa_status build_form2(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st) {
+  if (!wants_pairs(P)) return PA_OK;
+  FusedForm f;
+  f.nf = 2;
+  f.func = bf_pipe_func(P->K, P->apod, P->comp, P->full, P->d.interp == PA_INTERP_NEAREST);
+  f.threads = P->threads;
+  f.stages = 2;
+  if (const char* e = getenv("PA_STAGES")) f.stages = atoi(e);
+  f.tmem_cols = P->comp ? tmem_columns(P->warps, 2 * (P->K <= 2 ? 3 : P->K + 2)) : 0;
+  if (f.tmem_cols > kTmemColsPerSm) return PA_OK;
+  const int steps = P->u1 - P->u0;
+  auto occupancy = [&](int c) {
+    int b = 0;
+    if (form_smem(P, f, c, nullptr) > 226 * 1024 ||
+        fused_blocks_per_sm(P, f, form_smem(P, f, c, nullptr), &b) != cudaSuccess)
+      b = 0;
+    return b;
+  };
+  auto even = [&](int nch) { return ((steps + nch - 1) / nch + kC - 1) / kC * kC; };
+  int cap = kNCMax;
+  if (const char* e = getenv("PA_CHUNK_STEPS")) cap = std::max(kC, std::min(kNCMax, atoi(e)));
+  // the longest evenly cut chunk at the most resident blocks that chunks of
+  // at least 12 steps leave
+  int best = 0;
+  const int most = occupancy(kC);
+  for (int b = most; b >= 1 && !best; --b)
+    for (int nch = (steps + cap - 1) / cap; nch <= (steps + kC - 1) / kC; ++nch) {
+      const int c = std::min(even(nch), cap);
+      if (c < std::min(12, cap) && b > 1) break;
+      if (occupancy(c) >= b) {
+        best = c;
+        break;
+      }
+    }
+  cudaGetLastError();
+  if (!best) return PA_OK;
+  f.nc = best;
+  f.smem = form_smem(P, f, f.nc, &f.pairs_off);
+  PA_CUDA(fused_blocks_per_sm(P, f, f.smem, &f.blocks_per_sm));
+  if (f.blocks_per_sm < 1 || form_dense(P, f)) return PA_OK;
+  // chunks of fewer than 12 steps (RF windows of more than 200 samples) spend
+  // their time on the hand-over (0.89 measured at 8 steps)
+  if (f.nc < std::min(12, std::min(steps, cap))) return PA_OK;
+  // 12 resident warps (six-warp blocks, wide windows) are enough for orders
+  // <= 2 (1.12), not for higher ones (0.92-1.0)
+  // and the preparation pass pays where a sample serves enough pairs (38 pairs
+  // a sample: 0.95)
+  const double reuse = (double)P->executed_pairs /
+                       ((double)P->d.n_elem * std::max(1, P->used_hi - P->used_lo));
+  P->pairs_pay = reuse >= 48 && f.blocks_per_sm * P->warps >= (P->K <= 2 ? 12 : 14);
+  if (P->window > P->slot_margin) return PA_OK;  // (the margin bounds it)
+  const size_t bytes = pair_slots(P, &P->ws_frames, &P->slot_pitch);
+  if (dalloc(P, &P->slots_dev, bytes) != PA_OK) return PA_OK;  // no room
+  PA_CUDA(cudaMemsetAsync(P->slots_dev, 0, bytes, st));
+  const pa_status s = build_chunks(P, f, ur, st);
+  if (s != PA_OK) {
+    cudaFree(f.vchunks);
+    return s;
+  }
+  P->form[1] = f;
+  return PA_OK;
+}
+
 pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
   const pa_plan_desc& d = P->d;
   PA_CUDA(cudaGetDevice(&P->device));
@@ -840,7 +1089,6 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
   if ((s = dalloc(P, &P->slot_rg, (size_t)P->slots)) != PA_OK) return s;
   if ((s = dalloc(P, &P->lo, (size_t)P->n_tiles * P->nv)) != PA_OK) return s;
   if ((s = dalloc(P, &P->urange, (size_t)P->n_tiles * P->slots)) != PA_OK) return s;
-  if ((s = dalloc(P, &P->vchunks, (size_t)P->n_tiles * P->ngroups)) != PA_OK) return s;
   if ((s = dalloc(P, &P->tw, (size_t)2 * P->M)) != PA_OK) return s;  // >= n_tw
   if ((s = dalloc(P, &P->mask, (size_t)3 * P->M)) != PA_OK) return s;
   // [0] error flags, [1] work counter, [2, 2 + 3 max_batch) image maxima,
@@ -892,11 +1140,13 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
   g.full = P->full ? 1 : 0;
   FullGeom fg{P->nxt, P->n_tiles, P->tile_x, P->tile_z, P->m, P->slots, P->u1 - P->u0,
               P->lane_rows_log2, d.nx, d.nz, d.n_elem, P->u0, P->nv};
-  int* wmax = P->scratch[0] + 2;  // borrowed before first use as image maxima
+  // borrowed before first use as image maxima: window width, window starts
+  int* wmax = P->scratch[0] + 2;
+  int* lomax = P->scratch[0] + 3;
   if (P->full) {
     // windows first: the packed entries are written relative to them
     dim3 gw((P->nv + 127) / 128, P->n_tiles);
-    k_windows_full<<<gw, 128, 0, st>>>(tg, g, P->lo_align, P->lo, wmax);
+    k_windows_full<<<gw, 128, 0, st>>>(tg, g, P->lo_align, P->lo, wmax, lomax);
     PA_CUDA(cudaGetLastError());
     const size_t per_tile = P->full_entries / P->n_tiles;
     dim3 gt((unsigned)((per_tile + 255) / 256), P->n_tiles);
@@ -907,7 +1157,7 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
     k_table<<<gt, 128, 0, st>>>(tg, P->table, P->wtab);
     PA_CUDA(cudaGetLastError());
     dim3 gw((P->nv + 127) / 128, P->n_tiles);
-    k_windows<<<gw, 128, 0, st>>>(g, P->lo_align, P->table, P->lo, wmax, P->scratch[0]);
+    k_windows<<<gw, 128, 0, st>>>(g, P->lo_align, P->table, P->lo, wmax, lomax, P->scratch[0]);
     PA_CUDA(cudaGetLastError());
   }
   {
@@ -934,7 +1184,7 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
     }
   }
 
-  int head[3] = {0, 0, 0};
+  int head[5] = {0, 0, 0, 0, 0};
   std::vector<int2> ur((size_t)P->n_tiles * P->slots);
   PA_CUDA(cudaMemcpyAsync(head, P->scratch[0], sizeof head, cudaMemcpyDeviceToHost, st));
   PA_CUDA(cudaMemcpyAsync(ur.data(), P->urange, ur.size() * sizeof(int2), cudaMemcpyDeviceToHost,
@@ -947,6 +1197,9 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
   if (head[0] != 0) return fail(PA_ECUDA, "plan build: table row outside range (flag %d)", head[0]);
   const int width = head[2];
   P->window = ((std::max(width, 1) + 3) / 4) * 4;
+  // samples any window holds
+  P->used_lo = std::max(0, kLoBias - head[4]);
+  P->used_hi = std::min(d.n_samples, head[3] - kLoBias + P->window);
 
   PA_CUDA(cudaMemsetAsync(P->scratch[0], 0, P->scratch_ints * sizeof(int), st));
 
@@ -954,75 +1207,12 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
   P->wr = ((P->window + 1 + P->lo_align - 1) / P->lo_align) * P->lo_align;
   if (P->wr > 256) P->use_tma = false;  // TMA boxes span at most 256 elements
   if (P->use_tma && !tensor_map_encoder()) P->use_tma = false;
-  P->rp = (int)((((size_t)P->wr * P->elt + 127) & ~size_t(127)) / P->elt);
-  // Chunk length: every chunk costs a staging pass and two block barriers,
-  // so the channel steps are cut into as few, evenly sized chunks as keep
-  // the fused kernel's occupancy at what 32-step chunks give (measured at
-  // N = 128: 5 chunks of 28 steps 0.696 ms, 4 of 36 0.692 ms, 3 of 44
-  // 0.678 ms).  Limits: the slot buffer (at most 200 KiB), one issuing lane
-  // per staged channel under TMA (ncs <= 32 warps), and the multiply-shift
-  // division of the staging loops (exact while ncs * (W/4)^2 < 2^20).
-  // PA_CHUNK_STEPS caps the chunk length (for measurements).
-  {
-    const int steps = P->u1 - P->u0;
-    auto smem_for = [&](int c) {
-      const int ncs = c + kC - 1;
-      const size_t raw = P->use_tma ? (size_t)ncs * P->rp * P->elt : 0;
-      return (size_t)kRawOff + ((raw + 127) & ~size_t(127)) + (size_t)ncs * P->window * 8;
-    };
-    auto fits = [&](int c) {
-      const int ncs = c + kC - 1;
-      const long long w4 = P->window / 4;
-      return smem_for(c) <= 200 * 1024 && ncs <= 32 * P->warps &&
-             (long long)ncs * w4 * w4 < (1ll << 20);
-    };
-    auto occupancy = [&](int c) {
-      int b = 0;
-      if (fused_blocks_per_sm(P, smem_for(c), &b) != cudaSuccess) b = 0;
-      return b;
-    };
-    auto even = [&](int nch) { return ((steps + nch - 1) / nch + kC - 1) / kC * kC; };
-    int cap = kNCMax;
-    if (const char* e = getenv("PA_CHUNK_STEPS")) cap = std::max(kC, std::min(kNCMax, atoi(e)));
-    int ref = std::min(32, cap);
-    while (ref > kC && !fits(ref)) ref -= kC;
-    const int occ_ref = occupancy(ref);
-    int nc = ref;
-    for (int nch = (steps + cap - 1) / cap; nch <= (steps + ref - 1) / ref; ++nch) {
-      const int c = std::min(even(nch), cap);
-      if (c > ref && fits(c) && occupancy(c) >= occ_ref) {
-        nc = c;
-        break;
-      }
-    }
-    if (nc == ref) nc = std::min(ref, even((steps + ref - 1) / ref));
-    P->nc = nc;
-  }
-  cudaGetLastError();
-
-  // tile chunk ranges and executed pairs
-  std::vector<int2> vk((size_t)P->n_tiles * P->ngroups);
-  int64_t exec = 0;
-  for (int t = 0; t < P->n_tiles; ++t) {
-    for (int gr = 0; gr < P->ngroups; ++gr) {
-      int ua = P->u1, ub = P->u0;
-      for (int w = 0; w < P->warps; ++w) {
-        const int2 r = ur[(size_t)t * P->slots + gr * P->warps + w];
-        if (r.y > r.x) {
-          ua = std::min(ua, r.x);
-          ub = std::max(ub, r.y);
-          exec += (int64_t)(r.y - r.x) * 32 * kC;
-        }
-      }
-      int2 c = make_int2(0, 0);
-      if (ub > ua) c = make_int2((ua - P->u0) / P->nc, (ub - P->u0 + P->nc - 1) / P->nc);
-      vk[(size_t)t * P->ngroups + gr] = c;
-    }
-  }
-  P->executed_pairs = exec;
+  P->executed_pairs = 0;
+  for (int t = 0; t < P->n_tiles * P->slots; ++t)
+    if (ur[t].y > ur[t].x) P->executed_pairs += (int64_t)(ur[t].y - ur[t].x) * 32 * kC;
   P->active_pairs = P->apod ? (int64_t)active : (int64_t)d.nx * d.nz * d.n_elem;
-  PA_CUDA(cudaMemcpyAsync(P->vchunks, vk.data(), vk.size() * sizeof(int2), cudaMemcpyHostToDevice,
-                          st));
+  if ((s = build_form1(P, ur, st)) != PA_OK) return s;
+  if ((s = build_form2(P, ur, st)) != PA_OK) return s;
   // work items (tile, residue group) deepest tiles first; the frame is the
   // fastest index of a work item, so frames of one tile run back to back
   std::vector<int4> it((size_t)P->n_tiles * P->ngroups);
@@ -1036,27 +1226,6 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
   PA_CUDA(cudaMemcpyAsync(P->items, it.data(), it.size() * sizeof(int4), cudaMemcpyHostToDevice, st));
   PA_CUDA(cudaMemcpyAsync(P->slot_rg, srg.data(), srg.size() * sizeof(int2), cudaMemcpyHostToDevice,
                           st));
-
-  // shared memory and occupancy of the fused kernel
-  const int ncs = P->nc + kC - 1;
-  const size_t raw_bytes = P->use_tma ? (size_t)ncs * P->rp * P->elt : 0;
-  P->pairs_off = kRawOff + (int)((raw_bytes + 127) & ~size_t(127));
-  P->smem = (size_t)P->pairs_off + (size_t)ncs * P->window * sizeof(float2);
-  const long long w4 = P->window / 4;
-  if ((long long)ncs * w4 * w4 >= (1ll << 20))
-    return fail(PA_EUNSUPPORTED, "RF window of %d samples per channel is too wide; use a finer "
-                "depth grid", P->window);
-  if (P->smem > 200 * 1024)
-    return fail(PA_EUNSUPPORTED,
-                "RF window of %d samples per channel needs %zu B of shared memory; use a finer "
-                "depth grid",
-                P->window, P->smem);
-  // (resident blocks never ask for more TMEM than an SM has, so no block's
-  // allocation waits on another block of the same launch)
-  PA_CUDA(fused_blocks_per_sm(P, P->smem, &P->blocks_per_sm));
-  if (P->blocks_per_sm < 1)
-    return fail(PA_EUNSUPPORTED, "fused kernel does not fit an SM (%d threads, %zu B smem)",
-                P->threads, P->smem);
 
   // post-filter tables (host FP64 -> FP32)
   // per-pass twiddle blocks of the Stockham FFT, in the order the passes run
@@ -1120,33 +1289,23 @@ bool take_events(pa_plan_s* P, std::pair<cudaEvent_t, cudaEvent_t>* ev) {
   return true;
 }
 
-// Event pair around one kernel launch when timing is enabled.
-struct ProfScope {
-  pa_plan_s* P;
-  int kind;
-  cudaStream_t st;
-  std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
-  ProfScope(pa_plan_s* p, int k, cudaStream_t s) : P(p), kind(k), st(s) {
-    if (!(P->prof >> kind & 1u)) return;
-    if (!take_events(P, &ev)) return;
-    cudaEventRecord(ev.first, st);
-  }
-  ~ProfScope() {
-    if (!ev.first) return;
-    cudaEventRecord(ev.second, st);
-    P->ev_used.push_back({kind, ev});
-  }
+// The launches of one chunk of nf <= max_batch frames, in order.
+struct Step {
+  LaunchSpec spec;
+  void* args[2] = {nullptr, nullptr};
+  int begin = -1, end = -1;  // kernel kind whose timing starts / ends here
 };
-
-// Parameters of the launches of one chunk of nf <= max_batch frames.
 struct ChunkLaunch {
-  BfParams b;
+  struct Round {
+    BfParams b;
+    PrepParams pp;
+  };
+  std::vector<Round> rounds;
   PostParams q;
   LogParams l;
-  LaunchSpec sb, sq, sl;
-  bool post = false, log = false;
+  std::vector<Step> steps;
   int* zero = nullptr;  // counter + image maxima, cleared before the kernels
-  size_t zero_ints = 0;
+  int zero_ints = 0;
 };
 
 bool encode_rf_map(pa_plan_s* P, const void* rf, int nf, CUtensorMap* map) {
@@ -1164,30 +1323,49 @@ bool encode_rf_map(pa_plan_s* P, const void* rf, int nf, CUtensorMap* map) {
                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32_t stages,
-                        int* scratch, ChunkLaunch* c) {
+// The form a launch of nf frames runs.  Measured over 120 plans of 24-256
+// elements, 48-1024 depth rows and 2-57 frames (whole calls, one-frame form
+// time / two-frame form time):
+//   * two frames an item halve the items, so the launch has to fill the GPU
+//     all the same: below 0.65 resident blocks' worth of one-frame items
+//     0.72-0.95, above it 0.98-1.4;
+//   * an odd launch's last item does a frame's work twice: 3 and 5 frames
+//     0.85-0.99, 7 and more 1.04-1.3;
+//   * records whose rows are not 16-byte aligned (4 samples) are staged
+//     sample by sample in the one-frame form but prepared all the same in the
+//     other: 1.3-1.8 down to half as many items, odd launches included.
+const FusedForm& pick_form(const pa_plan_s* P, int nf) {
+  const FusedForm &one = P->form[0], &two = P->form[1];
+  if (two.nf == 0 || nf < 2) return one;
+  if (P->item_frames == 2) return two;
+  const double fill = (double)P->n_tiles * P->ngroups * nf / ((double)one.blocks_per_sm * P->num_sms);
+  const bool scalar = !P->use_tma && P->d.n_samples % 4 != 0;
+  const bool pays = scalar ? fill >= 0.3
+                           : fill >= 0.65 && (nf % 2 == 0 || nf >= 7) && P->pairs_pay;
+  return pays ? two : one;
+}
+
+// Launch parameters of one round of the fused kernel in form f: nf frames
+// from frame f0 of the chunk on.
+pa_status fused_params(pa_plan_s* P, const FusedForm& f, const void* rf, int nf, float* out,
+                       uint32_t stages, int* scratch, BfParams* bp) {
   const pa_plan_desc& d = P->d;
-  const int n_st = popcount3(stages);
-  const int planes = n_st * P->n_out;
+  const int planes = popcount3(stages) * P->n_out;
   const uint32_t raw_stage =
       (stages & PA_STAGE_RAW) ? PA_STAGE_RAW : ((stages & PA_STAGE_ENV) ? PA_STAGE_ENV : PA_STAGE_LOG);
-  const uint32_t env_stage = (stages & PA_STAGE_ENV) ? PA_STAGE_ENV : PA_STAGE_LOG;
   const int s_raw = stage_index(stages, raw_stage);
-  const int s_env = stage_index(stages, env_stage);
-  c->zero = scratch + 1;
-  c->zero_ints = 1 + (size_t)nf * P->n_out;
 
-  BfParams& b = c->b;
+  BfParams& b = *bp;
   memset(&b.tmap, 0, sizeof b.tmap);
-  b.use_tma = P->use_tma ? 1 : 0;
+  b.use_tma = f.nf == 1 && P->use_tma ? 1 : 0;
   b.wr = P->wr;
-  b.rp = P->rp;
-  b.nc = P->nc;
-  b.ncs = P->nc + kC - 1;
-  b.tmem_cols = P->tmem_cols;
-  b.chunk_bytes = b.ncs * P->wr * (int)P->elt;
-  b.pairs_off = P->pairs_off;
-  if (P->use_tma && !encode_rf_map(P, rf, nf, &b.tmap))
+  b.rp = f.rp;
+  b.nc = f.nc;
+  b.ncs = f.nc + kC - 1;
+  b.tmem_cols = f.tmem_cols;
+  b.chunk_bytes = f.nf == 1 ? b.ncs * P->wr * (int)P->elt : b.ncs * P->window * P->slot_bytes;
+  b.pairs_off = f.pairs_off;
+  if (b.use_tma && !encode_rf_map(P, rf, nf, &b.tmap))
     return fail(PA_ECUDA, "cuTensorMapEncodeTiled rejected the RF layout");
   b.rf = rf;
   b.rf_dtype = (int)d.rf_dtype;
@@ -1222,7 +1400,7 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
   b.w4_inv = (int)(((1u << 20) + (unsigned)(P->window / 4) - 1) / (unsigned)(P->window / 4));
   b.lo = P->lo;
   b.urange = P->urange;
-  b.vchunks = P->vchunks;
+  b.vchunks = f.vchunks;
   b.out = out;
   b.planes = planes;
   b.plane_das = P->out_id[0] >= 0 ? s_raw * P->n_out + P->out_id[0] : -1;
@@ -1231,18 +1409,89 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
   b.nx = d.nx;
   b.nz = d.nz;
   b.n_frames = nf;
-  b.n_items = P->n_tiles * P->ngroups * nf;
+  b.n_fgroups = (nf + f.nf - 1) / f.nf;
+  b.n_items = P->n_tiles * P->ngroups * b.n_fgroups;
   b.counter = scratch + 1;
   b.err = scratch;
   b.timeouts = scratch + P->scratch_ints - 1;
   b.expect_extra = P->expect_extra;
-  c->sb.func = bf_func(P->K, P->apod, P->comp, P->full);
-  c->sb.grid = dim3(std::max(1, std::min(b.n_items, P->blocks_per_sm * P->num_sms)));
-  c->sb.block = dim3(P->threads);
-  c->sb.smem = P->smem;
+  b.stages = f.stages;
+  b.slots_dev = P->slots_dev;
+  b.slot_pitch = P->slot_pitch;
+  b.slot_margin = P->slot_margin;
+  return PA_OK;
+}
 
-  c->post = (stages & (PA_STAGE_ENV | PA_STAGE_LOG)) != 0;
-  c->log = (stages & PA_STAGE_LOG) != 0;
+pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32_t stages,
+                        int* scratch, ChunkLaunch* c) {
+  const pa_plan_desc& d = P->d;
+  const int n_st = popcount3(stages);
+  const int planes = n_st * P->n_out;
+  const uint32_t raw_stage =
+      (stages & PA_STAGE_RAW) ? PA_STAGE_RAW : ((stages & PA_STAGE_ENV) ? PA_STAGE_ENV : PA_STAGE_LOG);
+  const uint32_t env_stage = (stages & PA_STAGE_ENV) ? PA_STAGE_ENV : PA_STAGE_LOG;
+  const int s_raw = stage_index(stages, raw_stage);
+  const int s_env = stage_index(stages, env_stage);
+  c->zero = scratch + 1;
+  c->zero_ints = 1 + nf * P->n_out;
+
+  const FusedForm& f = pick_form(P, nf);
+  const int per_round = f.nf == 2 ? P->ws_frames : nf;
+  const int n_rounds = (nf + per_round - 1) / per_round;
+  c->rounds.resize(n_rounds);
+  c->steps.clear();
+  c->steps.reserve(2 * n_rounds + 2);
+  if (f.nf == 1) {
+    Step z;
+    z.spec.func = reinterpret_cast<const void*>(k_zero_ints);
+    z.spec.grid = dim3(1);
+    z.spec.block = dim3(256);
+    z.args[0] = &c->zero;
+    z.args[1] = &c->zero_ints;
+    c->steps.push_back(z);
+  }
+  for (int r = 0; r < n_rounds; ++r) {
+    ChunkLaunch::Round& rd = c->rounds[r];
+    const int f0 = r * per_round, n = std::min(per_round, nf - f0);
+    const char* rf_r = (const char*)rf + (size_t)f0 * d.n_elem * d.n_samples * P->elt;
+    const pa_status s = fused_params(P, f, rf_r, n, out + (size_t)f0 * planes * d.nx * d.nz, stages,
+                                     scratch, &rd.b);
+    if (s != PA_OK) return s;
+    if (f.nf == 2) {
+      PrepParams& pp = rd.pp;
+      pp.rf = rf_r;
+      pp.slots = P->slots_dev;
+      pp.pitch = P->slot_pitch;
+      pp.margin = P->slot_margin;
+      pp.rf_dtype = (int)d.rf_dtype;
+      pp.n_elem = d.n_elem;
+      pp.n_samples = d.n_samples;
+      pp.n_frames = n;
+      pp.n_lo = P->used_lo;
+      pp.n_hi = P->used_hi;
+      pp.mode = P->slot_mode;
+      pp.order = P->K;
+      pp.zero = c->zero;
+      pp.n_zero = r == 0 ? c->zero_ints : 1;  // later rounds: the work counter only
+      Step sp;
+      prep_spec(&pp, &sp.spec);
+      sp.args[0] = &pp;
+      sp.begin = 0;
+      c->steps.push_back(sp);
+    }
+    Step sb;
+    sb.spec.func = f.func;
+    sb.spec.grid = dim3(std::max(1, std::min(rd.b.n_items, f.blocks_per_sm * P->num_sms)));
+    sb.spec.block = dim3(f.threads);
+    sb.spec.smem = f.smem;
+    sb.args[0] = &rd.b;
+    sb.begin = f.nf == 1 ? 0 : -1;
+    sb.end = 0;
+    c->steps.push_back(sb);
+  }
+
+  const bool post = (stages & (PA_STAGE_ENV | PA_STAGE_LOG)) != 0;
+  const bool log = (stages & PA_STAGE_LOG) != 0;
   PostParams& q = c->q;
   q.out = out;
   q.planes = planes;
@@ -1259,7 +1508,13 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
   q.maxslot = scratch + 2;
   q.n_frames = nf;
   q.warps_per_block = P->post_wpb;
-  post_spec(q, &c->sq);
+  if (post) {
+    Step t;
+    post_spec(q, &t.spec);
+    t.args[0] = &c->q;
+    t.begin = t.end = 1;
+    c->steps.push_back(t);
+  }
   LogParams& l = c->l;
   l.out = out;
   l.planes = planes;
@@ -1270,83 +1525,70 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
   l.maxslot = scratch + 2;
   l.dyn_range_db = P->dyn_range;
   l.n_frames = nf;
-  log_spec(l, P->num_sms, &c->sl);
+  if (log) {
+    Step t;
+    log_spec(l, P->num_sms, &t.spec);
+    t.args[0] = &c->l;
+    t.begin = t.end = 2;
+    c->steps.push_back(t);
+  }
   return PA_OK;
 }
 
 pa_status launch_direct(pa_plan_s* P, ChunkLaunch& c, cudaStream_t st) {
-  k_zero_ints<<<1, 256, 0, st>>>(c.zero, (int)c.zero_ints);
-  PA_CUDA(cudaGetLastError());
-  {
-    ProfScope ps(P, 0, st);
-    void* args[] = {&c.b};
-    PA_CUDA(cudaLaunchKernel(c.sb.func, c.sb.grid, c.sb.block, args, c.sb.smem, st));
-  }
-  if (c.post) {
-    ProfScope ps(P, 1, st);
-    void* args[] = {&c.q};
-    PA_CUDA(cudaLaunchKernel(c.sq.func, c.sq.grid, c.sq.block, args, c.sq.smem, st));
-  }
-  if (c.log) {
-    ProfScope ps(P, 2, st);
-    void* args[] = {&c.l};
-    PA_CUDA(cudaLaunchKernel(c.sl.func, c.sl.grid, c.sl.block, args, c.sl.smem, st));
+  std::pair<cudaEvent_t, cudaEvent_t> ev{nullptr, nullptr};
+  for (Step& t : c.steps) {
+    if (t.begin >= 0 && (P->prof >> t.begin & 1u) && take_events(P, &ev))
+      cudaEventRecord(ev.first, st);
+    const cudaError_t e =
+        cudaLaunchKernel(t.spec.func, t.spec.grid, t.spec.block, t.args, t.spec.smem, st);
+    if (ev.first && (t.end >= 0 || e != cudaSuccess)) {
+      cudaEventRecord(ev.second, st);
+      if (t.end >= 0) P->ev_used.push_back({t.end, ev});
+      else P->ev_free.push_back(ev);
+      ev = {nullptr, nullptr};
+    }
+    if (e != cudaSuccess) return fail(PA_ECUDA, "kernel launch: %s", cudaGetErrorString(e));
   }
   return PA_OK;
 }
 
-cudaKernelNodeParams node_params(const LaunchSpec& s, void** args) {
+cudaKernelNodeParams node_params(Step& t) {
   cudaKernelNodeParams k{};
-  k.func = const_cast<void*>(s.func);
-  k.gridDim = s.grid;
-  k.blockDim = s.block;
-  k.sharedMemBytes = (unsigned)s.smem;
-  k.kernelParams = args;
+  k.func = const_cast<void*>(t.spec.func);
+  k.gridDim = t.spec.grid;
+  k.blockDim = t.spec.block;
+  k.sharedMemBytes = (unsigned)t.spec.smem;
+  k.kernelParams = t.args;
   k.extra = nullptr;
   return k;
 }
 
-
-// One chunk as a CUDA graph: clear -> fused kernel [-> post [-> log]].  An
-// executable graph is kept per (frames, stages, timing); later calls only
-// rewrite the node parameters (buffer pointers, and the timing events) and
-// launch it.  While timing is on, each kernel node sits between two
-// event-record nodes, so the kernels are timed on the path that serves.
+// One chunk as a CUDA graph: the chunk's launches in a row.  An executable
+// graph is kept per (frames, stages, timing); later calls only rewrite the
+// node parameters (buffer pointers, and the timing events) and launch it.
+// While timing is on, each timed kernel sits between two event-record nodes,
+// so the kernels are timed on the path that serves.
 pa_status launch_graph(pa_plan_s* P, ChunkLaunch& c, int nf, uint32_t stages, cudaStream_t st) {
   const uint32_t prof = P->prof;
   pa_plan_s::GraphEntry* ge = nullptr;
   for (auto& g : P->graphs)
     if (g.nf == nf && g.stages == stages && g.prof == prof) ge = &g;
-  void* ab[] = {&c.b};
-  void* aq[] = {&c.q};
-  void* al[] = {&c.l};
-  int zn = (int)c.zero_ints;
-  void* az[] = {&c.zero, &zn};
-  LaunchSpec sz;
-  sz.func = reinterpret_cast<const void*>(k_zero_ints);
-  sz.grid = dim3(1);
-  sz.block = dim3(256);
-  const cudaKernelNodeParams kz = node_params(sz, az);
-  const cudaKernelNodeParams kb = node_params(c.sb, ab);
-  const cudaKernelNodeParams kq = node_params(c.sq, aq);
-  const cudaKernelNodeParams kl = node_params(c.sl, al);
-  const bool has[3] = {true, c.post, c.log};
-  bool timed[3];
-  for (int k = 0; k < 3; ++k) timed[k] = has[k] && (prof >> k & 1u);
-  std::pair<cudaEvent_t, cudaEvent_t> ev[3] = {};
+  std::vector<std::pair<int, std::pair<cudaEvent_t, cudaEvent_t>>> ev;  // in step order
+  auto give_back = [&]() {
+    for (auto& e : ev) P->ev_free.push_back(e.second);
+  };
   if (prof) {
-    for (int k = 0; k < 3; ++k) {
-      if (timed[k] && !take_events(P, &ev[k])) {
-        for (int j = 0; j < k; ++j)
-          if (ev[j].first) P->ev_free.push_back(ev[j]);
+    for (const Step& t : c.steps) {
+      if (t.begin < 0 || !(prof >> t.begin & 1u)) continue;
+      std::pair<cudaEvent_t, cudaEvent_t> e;
+      if (!take_events(P, &e)) {
+        give_back();
         return fail(PA_ECUDA, "timing events: out of resources");
       }
+      ev.push_back({t.begin, e});
     }
   }
-  auto give_back = [&]() {
-    for (int k = 0; k < 3; ++k)
-      if (ev[k].first) P->ev_free.push_back(ev[k]);
-  };
   if (!ge) {
     // bounded cache: drop the oldest graph once 32 shapes are held (callers
     // that vary the batch size every call would otherwise grow it forever)
@@ -1365,22 +1607,29 @@ pa_status launch_graph(pa_plan_s* P, ChunkLaunch& c, int nf, uint32_t stages, cu
       give_back();
       return fail(PA_ECUDA, "graph build: %s", cudaGetErrorString(e));
     }
-    const cudaKernelNodeParams* kp[3] = {&kb, &kq, &kl};
-    cudaGraphNode_t* kn[3] = {&g.n_bf, &g.n_post, &g.n_log};
-    e = cudaGraphAddKernelNode(&g.n_memset, graph, nullptr, 0, &kz);
-    cudaGraphNode_t prev = g.n_memset;
-    for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
-      if (!has[k]) continue;
-      if (timed[k]) {
-        e = cudaGraphAddEventRecordNode(&g.n_ev[k][0], graph, &prev, 1, ev[k].first);
-        prev = g.n_ev[k][0];
+    cudaGraphNode_t prev = nullptr;
+    size_t next_ev = 0;
+    for (Step& t : c.steps) {
+      if (t.begin >= 0 && (prof >> t.begin & 1u)) {
+        cudaGraphNode_t n = nullptr;
+        e = cudaGraphAddEventRecordNode(&n, graph, prev ? &prev : nullptr, prev ? 1 : 0,
+                                        ev[next_ev].second.first);
+        if (e != cudaSuccess) break;
+        g.events.push_back(n);
+        prev = n;
       }
-      if (e == cudaSuccess) e = cudaGraphAddKernelNode(kn[k], graph, &prev, 1, kp[k]);
+      const cudaKernelNodeParams kp = node_params(t);
+      cudaGraphNode_t n = nullptr;
+      e = cudaGraphAddKernelNode(&n, graph, prev ? &prev : nullptr, prev ? 1 : 0, &kp);
       if (e != cudaSuccess) break;
-      prev = *kn[k];
-      if (timed[k]) {
-        e = cudaGraphAddEventRecordNode(&g.n_ev[k][1], graph, &prev, 1, ev[k].second);
-        prev = g.n_ev[k][1];
+      g.kernels.push_back(n);
+      prev = n;
+      if (t.end >= 0 && (prof >> t.end & 1u)) {
+        cudaGraphNode_t m = nullptr;
+        e = cudaGraphAddEventRecordNode(&m, graph, &prev, 1, ev[next_ev++].second.second);
+        if (e != cudaSuccess) break;
+        g.events.push_back(m);
+        prev = m;
       }
     }
     if (e == cudaSuccess) e = cudaGraphInstantiate(&g.exec, graph, 0);
@@ -1391,19 +1640,19 @@ pa_status launch_graph(pa_plan_s* P, ChunkLaunch& c, int nf, uint32_t stages, cu
     }
     g.graph = graph;
     ++P->graph_builds;
-    P->graphs.push_back(g);
+    P->graphs.push_back(std::move(g));
     ge = &P->graphs.back();
   } else {
-    cudaError_t e = cudaGraphExecKernelNodeSetParams(ge->exec, ge->n_memset, &kz);
-    if (e == cudaSuccess) e = cudaGraphExecKernelNodeSetParams(ge->exec, ge->n_bf, &kb);
-    if (e == cudaSuccess && c.post)
-      e = cudaGraphExecKernelNodeSetParams(ge->exec, ge->n_post, &kq);
-    if (e == cudaSuccess && c.log) e = cudaGraphExecKernelNodeSetParams(ge->exec, ge->n_log, &kl);
-    for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
-      if (!timed[k]) continue;
-      e = cudaGraphExecEventRecordNodeSetEvent(ge->exec, ge->n_ev[k][0], ev[k].first);
+    cudaError_t e = cudaSuccess;
+    for (size_t i = 0; i < c.steps.size() && e == cudaSuccess; ++i) {
+      const cudaKernelNodeParams kp = node_params(c.steps[i]);
+      e = cudaGraphExecKernelNodeSetParams(ge->exec, ge->kernels[i], &kp);
+    }
+    for (size_t i = 0; i < ev.size() && e == cudaSuccess; ++i) {
+      e = cudaGraphExecEventRecordNodeSetEvent(ge->exec, ge->events[2 * i], ev[i].second.first);
       if (e == cudaSuccess)
-        e = cudaGraphExecEventRecordNodeSetEvent(ge->exec, ge->n_ev[k][1], ev[k].second);
+        e = cudaGraphExecEventRecordNodeSetEvent(ge->exec, ge->events[2 * i + 1],
+                                                 ev[i].second.second);
     }
     if (e != cudaSuccess) {
       give_back();
@@ -1415,8 +1664,7 @@ pa_status launch_graph(pa_plan_s* P, ChunkLaunch& c, int nf, uint32_t stages, cu
     give_back();
     return fail(PA_ECUDA, "graph launch: %s", cudaGetErrorString(e));
   }
-  for (int k = 0; k < 3; ++k)
-    if (ev[k].first) P->ev_used.push_back({k, ev[k]});
+  for (auto& x : ev) P->ev_used.push_back(x);
   return PA_OK;
 }
 
@@ -1478,7 +1726,7 @@ pa_plan_s::HostTune* host_tune(pa_plan_s* P, int nf, uint32_t stages) {
   if (nf > 2) {
     pa_pipe_model m{};
     m.items_per_frame = std::max(1, P->n_tiles * P->ngroups);
-    m.resident = std::max(1, P->blocks_per_sm * P->num_sms);
+    m.resident = std::max(1, P->form[0].blocks_per_sm * P->num_sms);
     m.n_sets = kHostSets;
     const double rf_frame = (double)P->d.n_elem * P->d.n_samples * P->elt;
     const double out_frame = (double)popcount3(stages) * P->n_out * P->d.nx * P->d.nz * 4.0;
@@ -1579,33 +1827,15 @@ pa_status build_host_graph(pa_plan_s* P, pa_plan_s::HostGraph& hg, const void* r
     }
     cudaGraphNode_t last = nullptr;
     if (e == cudaSuccess) {
-      void* ab[] = {&cl.b};
-      void* aq[] = {&cl.q};
-      void* al[] = {&cl.l};
-      int zn = (int)cl.zero_ints;
-      void* az[] = {&cl.zero, &zn};
-      LaunchSpec sz;
-      sz.func = reinterpret_cast<const void*>(k_zero_ints);
-      sz.grid = dim3(1);
-      sz.block = dim3(256);
-      const cudaKernelNodeParams kz = node_params(sz, az);
-      const cudaKernelNodeParams kb = node_params(cl.sb, ab);
       cudaGraphNode_t deps[2] = {up, prev_last};
-      cudaGraphNode_t nz = nullptr, nb = nullptr;
-      e = cudaGraphAddKernelNode(&nz, graph, deps, prev_last ? 2 : 1, &kz);
-      if (e == cudaSuccess) e = cudaGraphAddKernelNode(&nb, graph, &nz, 1, &kb);
-      last = nb;
-      if (e == cudaSuccess && cl.post) {
-        const cudaKernelNodeParams kq = node_params(cl.sq, aq);
-        cudaGraphNode_t nq = nullptr;
-        e = cudaGraphAddKernelNode(&nq, graph, &last, 1, &kq);
-        last = nq;
-      }
-      if (e == cudaSuccess && cl.log) {
-        const cudaKernelNodeParams kl = node_params(cl.sl, al);
-        cudaGraphNode_t nl = nullptr;
-        e = cudaGraphAddKernelNode(&nl, graph, &last, 1, &kl);
-        last = nl;
+      int n_deps = prev_last ? 2 : 1;
+      for (Step& t : cl.steps) {
+        const cudaKernelNodeParams kp = node_params(t);
+        cudaGraphNode_t n = nullptr;
+        e = cudaGraphAddKernelNode(&n, graph, deps, n_deps, &kp);
+        if (e != cudaSuccess) break;
+        last = deps[0] = n;
+        n_deps = 1;
       }
     }
     if (e == cudaSuccess)
@@ -1643,7 +1873,7 @@ pa_status host_call_done(pa_plan_s* P, pa_plan_s::HostTune* tune, bool tuning, i
                      std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() -
                                                                t_start).count(),
                      cold);
-  if (P->use_tma) {
+  if (P->use_tma || P->form[1].nf) {
     long long total = 0;
     for (int b = 0; b < kHostSets; ++b) {
       if (!P->scratch[b]) continue;
@@ -1675,10 +1905,8 @@ size_t plan_device_bytes(const pa_plan_s* P) { return P ? P->device_bytes : 0; }
 
 pa_status plan_bf_params(pa_plan_s* P, const void* rf, int nf, float* out, uint32_t stages,
                          BfParams* b, int* k, bool* lattice_fp32_plain) {
-  ChunkLaunch c;
-  const pa_status s = prepare_chunk(P, rf, nf, out, stages, P->scratch[0], &c);
+  const pa_status s = fused_params(P, P->form[0], rf, nf, out, stages, P->scratch[0], b);
   if (s != PA_OK) return s;
-  *b = c.b;
   *k = P->K;
   *lattice_fp32_plain = !P->full && !P->apod && !P->comp && P->d.rf_dtype == PA_RF_F32 &&
                         P->d.interp == PA_INTERP_LINEAR;
@@ -1694,36 +1922,10 @@ pa_status plan_bf_params(pa_plan_s* P, const void* rf, int nf, float* out, uint3
 // can fill an SM's TMEM while registers remain, so a block of another
 // compensated kernel landing there would wait in tcgen05.alloc.
 void plan_tmem(const pa_plan_s* P, int* cols, bool* dense) {
-  *cols = P ? P->tmem_cols : 0;
-  *dense = false;
-  if (!P || !P->tmem_cols) return;
-  cudaFuncAttributes a;
-  int regs_sm = 65536;
-  cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, P->device);
-  if (cudaFuncGetAttributes(&a, bf_func(P->K, P->apod, P->comp, P->full)) != cudaSuccess) {
-    cudaGetLastError();
-    *dense = true;  // unknown: treat as dense (serialised with other compensated batches)
-    return;
-  }
-  const size_t warps = (size_t)(P->threads + 31) / 32;
-  const size_t regs_block = (size_t)((a.numRegs * 32 + 255) / 256) * 256 * warps;
-  *dense = (size_t)P->tmem_cols * (size_t)regs_sm > (size_t)kTmemColsPerSm * regs_block;
+  *cols = P ? P->form[0].tmem_cols : 0;
+  *dense = P && form_dense(P, P->form[0]);  // the two-frame form is never dense (build_form2)
 }
 
-cudaError_t bf_launch(int order, bool apod, bool comp, bool full, const BfParams& p, int grid,
-                      int block, size_t smem, cudaStream_t s) {
-  switch (order) {
-    case 1: return bf_launch_k1(apod, comp, full, p, grid, block, smem, s);
-    case 2: return bf_launch_k2(apod, comp, full, p, grid, block, smem, s);
-    case 3: return bf_launch_k3(apod, comp, full, p, grid, block, smem, s);
-    case 4: return bf_launch_k4(apod, comp, full, p, grid, block, smem, s);
-    case 5: return bf_launch_k5(apod, comp, full, p, grid, block, smem, s);
-    case 6: return bf_launch_k6(apod, comp, full, p, grid, block, smem, s);
-    case 7: return bf_launch_k7(apod, comp, full, p, grid, block, smem, s);
-    case 8: return bf_launch_k8(apod, comp, full, p, grid, block, smem, s);
-  }
-  return cudaErrorInvalidValue;
-}
 const void* bf_func(int order, bool apod, bool comp, bool full) {
   switch (order) {
     case 1: return bf_func_k1(apod, comp, full);
@@ -1737,19 +1939,20 @@ const void* bf_func(int order, bool apod, bool comp, bool full) {
   }
   return nullptr;
 }
-cudaError_t bf_occupancy(int order, bool apod, bool comp, bool full, int block, size_t smem,
-                         int* n) {
+const void* bf_pipe_func(int order, bool apod, bool comp, bool full, bool nearest) {
   switch (order) {
-    case 1: return bf_occupancy_k1(apod, comp, full, block, smem, n);
-    case 2: return bf_occupancy_k2(apod, comp, full, block, smem, n);
-    case 3: return bf_occupancy_k3(apod, comp, full, block, smem, n);
-    case 4: return bf_occupancy_k4(apod, comp, full, block, smem, n);
-    case 5: return bf_occupancy_k5(apod, comp, full, block, smem, n);
-    case 6: return bf_occupancy_k6(apod, comp, full, block, smem, n);
-    case 7: return bf_occupancy_k7(apod, comp, full, block, smem, n);
-    case 8: return bf_occupancy_k8(apod, comp, full, block, smem, n);
+    case 1: return bf_pipe_func_k1(apod, comp, full, nearest);
+    case 2: return bf_pipe_func_k2(apod, comp, full, nearest);
+    case 3: return bf_pipe_func_k3(apod, comp, full, nearest);
+    case 4: return bf_pipe_func_k4(apod, comp, full, nearest);
+    case 5: return bf_pipe_func_k5(apod, comp, full, nearest);
   }
-  return cudaErrorInvalidValue;
+  return nullptr;
+}
+cudaError_t bf_occupancy(const void* func, int block, size_t smem, int* n) {
+  cudaError_t e = cudaFuncSetAttribute(func, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+  if (e != cudaSuccess) return e;
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, func, block, smem);
 }
 }  // namespace pa
 
@@ -1802,7 +2005,7 @@ pa_status pa_plan_get_info(pa_plan_t P, pa_plan_info* info) {
   info->window = P->window;
   info->n_tiles = P->n_tiles;
   info->threads = P->threads;
-  info->blocks_per_sm = P->blocks_per_sm;
+  info->blocks_per_sm = P->form[0].blocks_per_sm;
   info->fft_size = P->M;
   info->n_outputs = P->n_out;
   info->warnings = P->warnings;
@@ -1811,9 +2014,9 @@ pa_status pa_plan_get_info(pa_plan_t P, pa_plan_info* info) {
   info->executed_pairs = P->executed_pairs;
   info->device_bytes = P->device_bytes;
   info->tma_staging = P->use_tma ? 1 : 0;
-  info->chunk_steps = P->nc;
+  info->chunk_steps = P->form[0].nc;
   info->lane_rows = 1 << P->lane_rows_log2;
-  info->tmem_columns = P->tmem_cols;
+  info->tmem_columns = P->form[0].tmem_cols;
   info->delay_table = P->full ? PA_TABLE_FULL : PA_TABLE_LATTICE;
   info->table_bytes = delay_table_bytes(P);
   {
