@@ -382,8 +382,7 @@ __global__ void __launch_bounds__(256, 2) k_bf_pipe(const __grid_constant__ BfPa
     for (;;) {
       if (!__all_sync(0xffffffffu, mbar_wait_bounded(full_bar(stage), phase))) {
         if (lane == 0) {
-          atomicOr(p.err, 8);
-          if (atomicExch(reinterpret_cast<int*>(smem + kPipeStopOff), 1) == 0) atomicAdd(p.timeouts, 1);
+          if (atomicExch(reinterpret_cast<int*>(smem + kPipeStopOff), 1) == 0) report_timeout(p);
         }
         break;
       }

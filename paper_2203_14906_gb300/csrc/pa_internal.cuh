@@ -156,6 +156,8 @@ struct BfParams {  // aligned as CUtensorMap requires
   int* counter;           // work counter (zeroed before launch)
   int* err;               // error flags: 1, 2 index checks (checked builds), 8 a wait ran out
   int* timeouts;          // running count of blocks whose bounded TMA wait ran out
+  int* host_flag;         // pinned host word set when one did (null before the
+                          // plan's first host-path call)
   int expect_extra;       // bytes added to every chunk's expected transaction
                           // count: 0, or > 0 only to test the bounded wait
 };

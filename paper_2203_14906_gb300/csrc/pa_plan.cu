@@ -97,6 +97,7 @@ struct pa_plan_s {
   int lo_align = 4;   // window starts are multiples of this many samples
   int expect_extra = 0;   // > 0 only under PA_INJECT_TMA_SHORTFALL (tests the bounded wait)
   long long timeouts_seen = 0;  // timed-out waits already reported by pa_beamform_host
+  int* host_flag = nullptr;  // pinned word a timed-out wait sets (host path)
   int wr = 0;         // raw samples per channel delivered by one TMA box
   int item_frames = 0;  // PA_ITEM_FRAMES: 1 or 2 picks the form (measurements, tests)
   bool pairs_pay = false;  // resident warps and slot reuse of the two-frame form suffice
@@ -862,6 +863,7 @@ void free_plan(pa_plan_s* P) {
   cudaFree(P->h_out);
   for (int s = 0; s < kHostSets; ++s)
     if (P->hs[s]) cudaStreamDestroy(P->hs[s]);
+  if (P->host_flag) cudaFreeHost(P->host_flag);
   if (P->h_ev) cudaEventDestroy(P->h_ev);
   for (int s = 0; s < kHostSets; ++s)
     if (P->h_done[s]) cudaEventDestroy(P->h_done[s]);
@@ -1414,6 +1416,7 @@ pa_status fused_params(pa_plan_s* P, const FusedForm& f, const void* rf, int nf,
   b.counter = scratch + 1;
   b.err = scratch;
   b.timeouts = scratch + P->scratch_ints - 1;
+  b.host_flag = P->host_flag;
   b.expect_extra = P->expect_extra;
   b.stages = f.stages;
   b.slots_dev = P->slots_dev;
@@ -1873,7 +1876,11 @@ pa_status host_call_done(pa_plan_s* P, pa_plan_s::HostTune* tune, bool tuning, i
                      std::chrono::duration<double, std::milli>(std::chrono::steady_clock::now() -
                                                                t_start).count(),
                      cold);
-  if (P->use_tma || P->form[1].nf) {
+  // (the counts are read only after some wait has run out: a blocking copy a
+  // buffer set costs about 10 us; an earlier launch of the plan may have run
+  // out before the word existed, so it starts out set)
+  if (*reinterpret_cast<volatile int*>(P->host_flag)) {
+    *reinterpret_cast<volatile int*>(P->host_flag) = 0;
     long long total = 0;
     for (int b = 0; b < kHostSets; ++b) {
       if (!P->scratch[b]) continue;
@@ -2112,6 +2119,10 @@ pa_status pa_beamform_host(pa_plan_t P, const void* rf_host, int32_t n_frames, f
     PA_CUDA(cudaMalloc(&P->h_out, need_out));
     P->h_out_bytes = need_out;
     P->device_bytes += need_out;
+  }
+  if (!P->host_flag) {
+    PA_CUDA(cudaHostAlloc((void**)&P->host_flag, sizeof(int), cudaHostAllocMapped));
+    *P->host_flag = 1;
   }
   if (!P->h_ev) PA_CUDA(cudaEventCreateWithFlags(&P->h_ev, cudaEventDisableTiming));
   for (int b = 0; b < nsets; ++b) {
