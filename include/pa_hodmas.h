@@ -125,8 +125,9 @@ typedef struct pa_plan_s* pa_plan_t;
 /* Read-only facts about a plan (for tests, benchmarks and admission).
  * blocks_per_sm, tma_staging, chunk_steps and tmem_columns describe the
  * one-frame form of the fused kernel; launches of two and more frames may run
- * its two-frame form (orders <= 5), which reads RF through slots prepared in
- * device memory of the plan.  Results do not depend on the form. */
+ * its two-frame form (orders <= 5) and small launches its fine-grained form,
+ * which read RF through slots prepared in device memory of the plan.  Results
+ * do not depend on the form. */
 typedef struct {
   int32_t lattice_m;          /* pitch / lateral pixel pitch (lattice table;
                                  0 with the full table)                    */
@@ -188,9 +189,10 @@ typedef struct {
  * on these): PA_STAGING=tma|loads picks the RF staging path (TMA
  * boxes need Ns to be a multiple of the window alignment), PA_CHUNK_STEPS=n
  * caps the channel steps per staged chunk, PA_LANE_ROWS=32|16|8 sets the
- * depth rows per lane group of the fused kernel, PA_ITEM_FRAMES=1|2 the
- * frames per work item of launches of two and more frames (orders <= 5).  In
- * the checked build only
+ * depth rows per lane group of the fused kernel, PA_ITEM_FRAMES the form of
+ * the fused kernel (1: one frame per work item, 2: two where the launch and the
+ * order allow it, 3: one pixel per thread where the launch allows it).  In the
+ * checked build only
  * (device bounds checks, PA_CHECK_BOUNDS), PA_INJECT_TMA_SHORTFALL makes
  * every TMA chunk expect 16 bytes more than it receives, so each block's
  * bounded wait runs out (failure-detection tests); the release build ignores

@@ -1,0 +1,4 @@
+// Order 2 of the fine-grained fused beamforming kernel.
+#include "pa_bf_fine.cuh"
+
+PA_DEFINE_FINE(2)

@@ -1,0 +1,4 @@
+// Order 3 of the fine-grained fused beamforming kernel.
+#include "pa_bf_fine.cuh"
+
+PA_DEFINE_FINE(3)

@@ -234,7 +234,11 @@ __device__ __forceinline__ void final_tmem2(float (&acc)[2][kC][NA], uint32_t tm
 // The running item and chunk live in shared memory; calls follow one another
 // (each is made by the last warp to finish the stage's previous chunk, and
 // that warp finishes no later chunk before it returns).
-template <bool FULL, int SB>
+// NF frames per item.  With one (pa_bf_fine.cuh) an item is a share of a tile's
+// warps, its chunks cover the whole tile, and the channel bases are written
+// kC times, shifted by 0 .. kC - 1 channels, so that a warp whose first pixel
+// pairs with channel u + c reads aligned fours.
+template <bool FULL, int SB, int NF>
 __device__ __forceinline__ void produce(const BfParams& p, unsigned char* smem, uint32_t sbase,
                                      int stage, int lane) {
   int4* prod = reinterpret_cast<int4*>(smem + kPipeProdOff);
@@ -257,18 +261,27 @@ __device__ __forceinline__ void produce(const BfParams& p, unsigned char* smem, 
       return;
     }
     const int tg = item / p.n_fgroups;
-    it = __ldg(p.items + tg);
-    const int2 vk = __ldg(p.vchunks + (size_t)it.x * p.ngroups + it.y);
+    int2 vk;
+    if constexpr (NF == 2) {
+      it = __ldg(p.items + tg);
+      vk = __ldg(p.vchunks + (size_t)it.x * p.ngroups + it.y);
+    } else {
+      it = __ldg(p.items + (size_t)(tg / p.splits) * p.ngroups);
+      it.y = tg % p.splits;
+      vk = __ldg(p.vchunks + it.x);
+    }
     run = make_int4(item - tg * p.n_fgroups, vk.x, vk.y, 1);
     first = true;
   }
   const bool data = run.z > run.y;  // an item without pairs still stores its zeros
   const bool last = run.y + 1 >= run.z;
   const int W = p.window, k = run.y;
-  const uint32_t slots = sbase + kPipeSlotOff + stage * (p.ncs * W * SB);
-  int* s_cb = reinterpret_cast<int*>(smem + kPipeCbOff + stage * kCbInts * 4);
+  const uint32_t slots =
+      sbase + (NF == 2 ? kPipeSlotOff : kFineSlotOff) + stage * (p.ncs * W * SB);
+  constexpr int CB = NF == 2 ? 1 : kC;  // copies of the channel bases
+  int* s_cb = reinterpret_cast<int*>(smem + kPipeCbOff + stage * CB * kCbInts * 4);
   if (lane == 0) {
-    meta[0] = make_int4(it.x, run.x * 2, it.y, k);
+    meta[0] = make_int4(it.x, run.x * NF, it.y, k);
     meta[1] = make_int4(it.z, it.w, (first ? 1 : 0) | (last ? 2 : 0) | (data ? 0 : 4), 0);
     prod[0] = it;
     prod[1] = make_int4(run.x, k + 1, run.z, last ? 0 : 1);
@@ -287,7 +300,12 @@ __device__ __forceinline__ void produce(const BfParams& p, unsigned char* smem, 
 #pragma unroll
   for (int q = 0; q < 3; ++q) {
     const int cv = lane + 32 * q;
-    if (cv < p.ncs) s_cb[cv] = (int)slots + (cv * W - (FULL ? 0 : lo[q])) * SB;
+    if (cv >= p.ncs) continue;
+    const int cb = (int)slots + (cv * W - (FULL ? 0 : lo[q])) * SB;
+    s_cb[cv] = cb;
+#pragma unroll
+    for (int c = 1; c < CB; ++c)
+      if (cv >= c) s_cb[c * kCbInts + cv - c] = cb;
   }
   __syncwarp();
   if (lane == 0) mbar_expect(bar, p.chunk_bytes + p.expect_extra);
@@ -334,7 +352,7 @@ __global__ void __launch_bounds__(256, 2) k_bf_pipe(const __grid_constant__ BfPa
   int stage = 0, phase = 0;
   if (warp == 0)
     for (int s = 0; s < p.stages; ++s) {
-      produce<FULL, SB>(p, smem, sbase, s, lane);
+      produce<FULL, SB, 2>(p, smem, sbase, s, lane);
       __syncwarp();
     }
   {
@@ -582,7 +600,7 @@ __global__ void __launch_bounds__(256, 2) k_bf_pipe(const __grid_constant__ BfPa
       if (lane == 0) before = count_arrival(sbase + kPipeCountOff + 4 * stage);
       if (__shfl_sync(0xffffffffu, before, 0) == nwarps - 1) {
         if (lane == 0) reinterpret_cast<int*>(smem + kPipeCountOff)[stage] = 0;
-        produce<FULL, SB>(p, smem, sbase, stage, lane);
+        produce<FULL, SB, 2>(p, smem, sbase, stage, lane);
         __syncwarp();
       }
       if (++stage == p.stages) {

@@ -56,6 +56,11 @@ constexpr int kPipeSlotOff = 1536;
 static_assert(kPipeSlotOff >= kPipeCbOff + kPipeStages * kCbInts * 4 && kPipeSlotOff % 128 == 0,
               "shared layout");
 
+// The fine-grained kernel keeps kC shifted copies of the channel bases.
+constexpr int kFineSlotOff = kPipeCbOff + 2 * kC * kCbInts * 4 + 128;
+constexpr int kFineStages = 2;
+static_assert(kFineSlotOff % 16 == 0, "shared layout");
+
 // TMEM columns a fused-kernel block allocates for compensated totals (a
 // power of two >= 32): the warps sharing a 32-lane quarter of TMEM times 8
 // columns per accumulator (kC totals and kC compensation terms; na counts the
@@ -146,7 +151,8 @@ struct BfParams {  // aligned as CUtensorMap requires
   int n_frames;           // frames in this launch
   int n_items;            // n_tiles * ngroups * n_frames (two-frame kernel: * n_fgroups)
   // two-frame kernel
-  int n_fgroups;          // frame pairs (ceil(n_frames / 2))
+  int n_fgroups;          // frame pairs (ceil(n_frames / 2)); fine kernel: frames
+  int splits;             // fine kernel: items per tile
   int stages;             // chunks of slots in shared memory
   const unsigned char* slots_dev;  // prepared slots (k_prep): a row of zeros,
                                    // then [frame pair][channel] rows of
@@ -178,6 +184,7 @@ struct PrepParams {
   int rf_dtype, n_elem, n_samples, n_frames;
   int n_lo, n_hi;      // samples the windows hold
   int blocks_per_row;
+  int nf;              // frames per slot: 2, or 1 ({r, d} slots of the fine kernel)
   int mode, order;     // slot kind (PipeMode), order of its roots
   int* zero;           // words cleared before the fused kernel (work counter, maxima)
   int n_zero;
@@ -209,6 +216,7 @@ struct LogParams {
 };
 
 const void* bf_func(int order, bool apod, bool comp, bool full);
+const void* bf_fine_func(int order, bool apod, bool comp, bool full, int px);
 int pipe_slot_mode(int order, bool apod, bool nearest);  // PipeMode
 int pipe_slot_bytes(int mode);
 const void* bf_pipe_func(int order, bool apod, bool comp, bool full, bool nearest);
@@ -245,6 +253,17 @@ PA_DECLARE_PIPE(2)
 PA_DECLARE_PIPE(3)
 PA_DECLARE_PIPE(4)
 PA_DECLARE_PIPE(5)
+#define PA_DECLARE_FINE(K) \
+  const void* bf_fine_func_k##K(bool apod, bool comp, bool full, int px);
+PA_DECLARE_FINE(1)
+PA_DECLARE_FINE(2)
+PA_DECLARE_FINE(3)
+PA_DECLARE_FINE(4)
+PA_DECLARE_FINE(5)
+PA_DECLARE_FINE(6)
+PA_DECLARE_FINE(7)
+PA_DECLARE_FINE(8)
+#undef PA_DECLARE_FINE
 #undef PA_DECLARE_ORDER
 #undef PA_DECLARE_PIPE
 

@@ -60,19 +60,27 @@ constexpr int kHostSets = 3;
 
 // One form of the fused kernel and the shared-memory geometry that goes with
 // it: form 0 runs one frame per work item (pa_bf_kernel.cuh), form 1 two
-// frames from prepared slots (pa_bf_pipe.cuh).
+// frames from prepared slots (pa_bf_pipe.cuh), forms 2 and 3 one and two of a
+// thread's four pixels, for small launches (pa_bf_fine.cuh).
 struct FusedForm {
   int nf = 0;             // frames per work item (0: the plan has no such form)
   const void* func = nullptr;
   int threads = 0;
   int nc = 32;            // channel steps per staged chunk (multiple of kC)
-  int stages = 1;         // chunks in shared memory at once (two-frame form)
+  int stages = 1;         // chunks in shared memory at once (forms 1-3)
   int rp = 0;             // raw-buffer row pitch in samples (128-byte aligned rows)
   int pairs_off = 0;      // shared-memory offset of the interpolation slots
   size_t smem = 0;
   int blocks_per_sm = 0;
   int tmem_cols = 0;      // TMEM columns per block (compensated sums)
-  int2* vchunks = nullptr;  // [n_tiles * ngroups] chunk range of a work item
+  int splits = 1;         // work items per tile (forms 2, 3)
+  int2* vchunks = nullptr;  // chunk range of a work item (forms 2, 3: of a tile)
+  // prepared slots: a row of zeros, then one row of slot_pitch slots per
+  // (frames of an item, channel), for max_frames frames a round (forms 2 and
+  // 3: at most that many frames a launch)
+  int slot_bytes = 0;
+  unsigned char* slots = nullptr;
+  int max_frames = 0;
 };
 
 struct pa_plan_s {
@@ -86,13 +94,11 @@ struct pa_plan_s {
   int tile_x = 0, tile_z = 32, nxt = 0, nzt = 0, n_tiles = 0, nx_pad = 0, nz_pad = 0;
   int u0 = 0, u1 = 0, nv = 0, dmin = 0, ndrows = 0, tgroups = 0, window = 0;
   size_t full_entries = 0;  // entries of the full table (n_tiles * (steps + 3) * 32 * slots * kC)
-  FusedForm form[2];
-  // prepared slots of the two-frame form: a row of zeros, then one row of
-  // slot_pitch slots per (frame pair, channel), for ws_frames frames a round
-  unsigned char* slots_dev = nullptr;
+  FusedForm form[4];
+  unsigned char* fine_slots = nullptr;  // prepared slots of forms 2 and 3
   long long slot_pitch = 0;
   int used_lo = 0, used_hi = 0;  // samples [used_lo, used_hi) lie in some window
-  int slot_margin = 0, slot_mode = 0, slot_bytes = 16, ws_frames = 0;
+  int slot_margin = 0, slot_mode = 0;
   bool use_tma = false;
   int lo_align = 4;   // window starts are multiples of this many samples
   int expect_extra = 0;   // > 0 only under PA_INJECT_TMA_SHORTFALL (tests the bounded wait)
@@ -100,6 +106,7 @@ struct pa_plan_s {
   int* host_flag = nullptr;  // pinned word a timed-out wait sets (host path)
   int wr = 0;         // raw samples per channel delivered by one TMA box
   int item_frames = 0;  // PA_ITEM_FRAMES: 1 or 2 picks the form (measurements, tests)
+  double steps_per_pixel = 0;  // channel steps evaluated per pixel, mean
   bool pairs_pay = false;  // resident warps and slot reuse of the two-frame form suffice
   // post
   int M = 1, log2M = 0, post_wpb = 1, n_out = 0, n_tw = 0;
@@ -718,7 +725,8 @@ void configure(pa_plan_s* P) {
     const double span = d.fs_hz / d.c_m_s * std::hypot(P->tile_x * dx, P->tile_z * dz);
     P->slot_margin = ((int)std::min(span, 1e6) + P->lo_align + 8) / 4 * 4;
     P->slot_mode = pipe_slot_mode(P->K, P->apod, d.interp == PA_INTERP_NEAREST);
-    P->slot_bytes = pipe_slot_bytes(P->slot_mode);
+    // 16-byte rows
+    P->slot_pitch = ((long long)d.n_samples + 1) / 2 * 2 + 2ll * P->slot_margin;
   }
   // Measured on GB300: TMA staging wins for 16-bit RF (half-size raw buffer),
   // vectorised loads win for FP32 RF (the FP32 raw buffer costs a resident
@@ -768,20 +776,43 @@ cudaError_t fused_blocks_per_sm(const pa_plan_s* P, const FusedForm& f, size_t s
 
 // Whether a plan of this descriptor gets the two-frame form (if it fits).
 bool wants_pairs(const pa_plan_s* P) {
-  return P->d.max_batch > 1 && P->K <= 5 && P->item_frames != 1;
+  return P->d.max_batch > 1 && P->K <= 5 && P->item_frames != 1 && P->item_frames != 3;
 }
 
-// Frames per round of the two-frame form and the bytes of its slots.  The
-// slots of a round are written by k_prep and read back by every tile.
+// Largest launch, in warps of 4-pixel threads, of the fine-grained forms
+// (pick_form says where the lines lie): one pixel a thread, and two.  They
+// reach further where the one-frame form is slow for its size: compensated
+// sums, the full table, records staged sample by sample.
+struct FineLimits {
+  int px1, px2;
+};
+FineLimits fine_limits(const pa_plan_s* P) {
+  if (P->item_frames == 3) return {1 << 20, 1 << 20};  // tests
+  if (P->item_frames != 0) return {0, 0};
+  const bool scalar = !P->use_tma && P->d.n_samples % 4 != 0;
+  return P->comp || P->full || scalar ? FineLimits{1100, 2400} : FineLimits{600, 0};
+}
+// Warps of 4-pixel threads of one frame.
+int64_t frame_warps(const pa_plan_s* P) { return (int64_t)P->n_tiles * P->slots; }
+
+// Frames per round of form 1 (of a launch of forms 2 and 3) and the bytes of
+// their slots; 0 frames: no such form.  The slots
+// of a round are written by the preparation pass and read back by every tile.
 constexpr size_t kSlotBytesMax = (size_t)512 << 20;
-size_t pair_slots(const pa_plan_s* P, int* frames, long long* pitch) {
-  *pitch = ((long long)P->d.n_samples + 1) / 2 * 2 + 2ll * P->slot_margin;  // 16-byte rows
-  const size_t row = (size_t)*pitch * P->slot_bytes;
-  const size_t per_pair = (size_t)P->d.n_elem * row;
-  size_t pairs = ((size_t)P->d.max_batch + 1) / 2;
-  pairs = std::max<size_t>(1, std::min(pairs, kSlotBytesMax / per_pair));
-  *frames = (int)(2 * pairs);
-  return row + pairs * per_pair;
+size_t slots_size(const pa_plan_s* P, int form, int* frames) {
+  const int item = form == 1 ? 2 : 1;
+  const FineLimits lim = fine_limits(P);
+  *frames = 0;
+  if (form > 1 && frame_warps(P) > std::max(lim.px1, lim.px2)) return 0;
+  const size_t sb = form == 1 ? pipe_slot_bytes(P->slot_mode) : sizeof(float2);
+  const size_t row = (size_t)P->slot_pitch * sb;
+  const size_t per_item = (size_t)P->d.n_elem * row;
+  size_t items = ((size_t)P->d.max_batch + item - 1) / item;
+  if (form > 1)
+    items = std::min<size_t>(items, std::max<int64_t>(1, std::max(lim.px1, lim.px2) / frame_warps(P)));
+  items = std::max<size_t>(1, std::min(items, kSlotBytesMax / per_item));
+  *frames = (int)(item * items);
+  return row + items * per_item;
 }
 
 // Bytes of the delay table and its apodisation weights.
@@ -805,11 +836,12 @@ size_t table_bytes(const pa_plan_s* P) {
   b += (size_t)P->n_tiles * P->nv * sizeof(int);
   b += (size_t)P->n_tiles * P->slots * sizeof(int2);
   b += (size_t)P->n_tiles * P->ngroups * sizeof(int2);
-  if (wants_pairs(P)) {  // chunk ranges and slots of the two-frame form
-    int frames;
-    long long pitch;
-    b += (size_t)P->n_tiles * P->ngroups * sizeof(int2) + pair_slots(P, &frames, &pitch);
-  }
+  // chunk ranges and slots of the other forms
+  int frames;
+  if (wants_pairs(P))
+    b += (size_t)P->n_tiles * P->ngroups * sizeof(int2) + slots_size(P, 1, &frames);
+  const size_t fine = slots_size(P, 2, &frames);
+  if (frames) b += fine + 2 * (size_t)P->n_tiles * sizeof(int2);
   b += (size_t)2 * P->M * sizeof(float2) + (size_t)3 * P->M * sizeof(float);
   return b;
 }
@@ -853,7 +885,8 @@ void free_plan(pa_plan_s* P) {
   cudaFree(P->lo);
   cudaFree(P->urange);
   for (FusedForm& f : P->form) cudaFree(f.vchunks);
-  cudaFree(P->slots_dev);
+  cudaFree(P->form[1].slots);
+  cudaFree(P->fine_slots);
   cudaFree(P->items);
   cudaFree(P->slot_rg);
   cudaFree(P->tw);
@@ -891,9 +924,10 @@ void free_plan(pa_plan_s* P) {
 // chunk; *pairs_off is where its interpolation slots start.
 size_t form_smem(const pa_plan_s* P, const FusedForm& f, int c, int* pairs_off) {
   const int ncs = c + kC - 1;
-  if (f.nf == 2) {
-    if (pairs_off) *pairs_off = kPipeSlotOff;
-    return (size_t)kPipeSlotOff + (size_t)f.stages * ncs * P->window * P->slot_bytes;
+  if (f.slot_bytes) {
+    const int off = f.nf == 2 ? kPipeSlotOff : kFineSlotOff;
+    if (pairs_off) *pairs_off = off;
+    return (size_t)off + (size_t)f.stages * ncs * P->window * f.slot_bytes;
   }
   const size_t raw = P->use_tma ? (size_t)ncs * f.rp * P->elt : 0;
   const size_t off = (size_t)kRawOff + ((raw + 127) & ~size_t(127));
@@ -917,14 +951,17 @@ bool form_dense(const pa_plan_s* P, const FusedForm& f) {
   return (size_t)f.tmem_cols * (size_t)regs_sm > (size_t)kTmemColsPerSm * regs_block;
 }
 
-// Chunk range of every work item of form f, uploaded to f.vchunks.
-pa_status build_chunks(pa_plan_s* P, FusedForm& f, const std::vector<int2>& ur, cudaStream_t st) {
-  std::vector<int2> vk((size_t)P->n_tiles * P->ngroups);
+// Chunk range of every (tile, share of its slots) of form f, uploaded to
+// f.vchunks: per residue group, or (form 2) of whole tiles.
+pa_status build_chunks(pa_plan_s* P, FusedForm& f, int groups, const std::vector<int2>& ur,
+                       cudaStream_t st) {
+  const int per = P->slots / groups;
+  std::vector<int2> vk((size_t)P->n_tiles * groups);
   for (int t = 0; t < P->n_tiles; ++t) {
-    for (int gr = 0; gr < P->ngroups; ++gr) {
+    for (int gr = 0; gr < groups; ++gr) {
       int ua = P->u1, ub = P->u0;
-      for (int w = 0; w < P->warps; ++w) {
-        const int2 r = ur[(size_t)t * P->slots + gr * P->warps + w];
+      for (int w = 0; w < per; ++w) {
+        const int2 r = ur[(size_t)t * P->slots + gr * per + w];
         if (r.y > r.x) {
           ua = std::min(ua, r.x);
           ub = std::max(ub, r.y);
@@ -932,7 +969,7 @@ pa_status build_chunks(pa_plan_s* P, FusedForm& f, const std::vector<int2>& ur, 
       }
       int2 c = make_int2(0, 0);
       if (ub > ua) c = make_int2((ua - P->u0) / f.nc, (ub - P->u0 + f.nc - 1) / f.nc);
-      vk[(size_t)t * P->ngroups + gr] = c;
+      vk[(size_t)t * groups + gr] = c;
     }
   }
   const pa_status s = dalloc(P, &f.vchunks, vk.size());
@@ -1006,7 +1043,28 @@ pa_status build_form1(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st
   if (f.blocks_per_sm < 1)
     return fail(PA_EUNSUPPORTED, "fused kernel does not fit an SM (%d threads, %zu B smem)",
                 P->threads, f.smem);
-  return build_chunks(P, f, ur, st);
+  return build_chunks(P, f, P->ngroups, ur, st);
+}
+
+// Slots and chunk ranges of form i, which the plan then has; without room for
+// its slots the plan does without it.
+pa_status finish_form(pa_plan_s* P, int i, FusedForm& f, int groups, const std::vector<int2>& ur,
+                      cudaStream_t st) {
+  const size_t bytes = slots_size(P, i, &f.max_frames);
+  if (f.max_frames == 0) return PA_OK;
+  unsigned char** slots = i == 1 ? &f.slots : &P->fine_slots;
+  if (!*slots) {
+    if (dalloc(P, slots, bytes) != PA_OK) return PA_OK;
+    const cudaError_t e = cudaMemsetAsync(*slots, 0, bytes, st);
+    if (e != cudaSuccess) {
+      if (i == 1) cudaFree(f.slots);
+      return fail(PA_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
+    }
+  }
+  f.slots = *slots;
+  const pa_status s = build_chunks(P, f, groups, ur, st);
+  P->form[i] = f;  // (a failed plan is freed whole)
+  return s;
 }
 
 // The two-frame form; a plan it does not fit keeps the one-frame form alone.
@@ -1014,6 +1072,7 @@ pa_status build_form2(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st
   if (!wants_pairs(P)) return PA_OK;
   FusedForm f;
   f.nf = 2;
+  f.slot_bytes = pipe_slot_bytes(P->slot_mode);
   f.func = bf_pipe_func(P->K, P->apod, P->comp, P->full, P->d.interp == PA_INTERP_NEAREST);
   f.threads = P->threads;
   f.stages = 2;
@@ -1061,16 +1120,52 @@ pa_status build_form2(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st
                        ((double)P->d.n_elem * std::max(1, P->used_hi - P->used_lo));
   P->pairs_pay = reuse >= 48 && f.blocks_per_sm * P->warps >= (P->K <= 2 ? 12 : 14);
   if (P->window > P->slot_margin) return PA_OK;  // (the margin bounds it)
-  const size_t bytes = pair_slots(P, &P->ws_frames, &P->slot_pitch);
-  if (dalloc(P, &P->slots_dev, bytes) != PA_OK) return PA_OK;  // no room
-  PA_CUDA(cudaMemsetAsync(P->slots_dev, 0, bytes, st));
-  const pa_status s = build_chunks(P, f, ur, st);
-  if (s != PA_OK) {
-    cudaFree(f.vchunks);
-    return s;
+  return finish_form(P, 1, f, P->ngroups, ur, st);
+}
+
+// The fine-grained forms: a tile's pixels at px of a thread's four per thread,
+// in blocks of at most 16 warps.
+pa_status build_form3(pa_plan_s* P, int px, const std::vector<int2>& ur, cudaStream_t st) {
+  const FineLimits lim = fine_limits(P);
+  if (frame_warps(P) > (px == 1 ? lim.px1 : lim.px2) || P->window > P->slot_margin) return PA_OK;
+  FusedForm f;
+  f.nf = 1;
+  f.slot_bytes = sizeof(float2);
+  f.stages = kFineStages;
+  const int tile_warps = P->slots * kC / px;
+  int nw = 1;
+  for (int w = 1; w <= 16; ++w)
+    if (tile_warps % w == 0) nw = w;
+  f.splits = tile_warps / nw;
+  f.threads = 32 * nw;
+  f.func = bf_fine_func(P->K, P->apod, P->comp, P->full, px);
+  const int steps = P->u1 - P->u0;
+  auto occupancy = [&](int c) {
+    int b = 0;
+    if (form_smem(P, f, c, nullptr) > 226 * 1024 ||
+        fused_blocks_per_sm(P, f, form_smem(P, f, c, nullptr), &b) != cudaSuccess)
+      b = 0;
+    return b;
+  };
+  // the longest evenly cut chunk that leaves 32 warps an SM (or as many as
+  // registers allow)
+  auto even = [&](int nch) { return ((steps + nch - 1) / nch + kC - 1) / kC * kC; };
+  int cap = kNCMax;
+  if (const char* e = getenv("PA_CHUNK_STEPS")) cap = std::max(kC, std::min(kNCMax, atoi(e)));
+  const int most = occupancy(kC);
+  int best = 0;
+  for (int nch = (steps + cap - 1) / cap; nch <= (steps + kC - 1) / kC && !best; ++nch) {
+    const int c = std::min(even(nch), cap);
+    const int b = occupancy(c);
+    if (b >= 1 && b * nw >= std::min(most * nw, 32)) best = c;
   }
-  P->form[1] = f;
-  return PA_OK;
+  cudaGetLastError();
+  if (!best) return PA_OK;
+  f.nc = best;
+  f.smem = form_smem(P, f, f.nc, &f.pairs_off);
+  PA_CUDA(fused_blocks_per_sm(P, f, f.smem, &f.blocks_per_sm));
+  if (f.blocks_per_sm < 1) return PA_OK;
+  return finish_form(P, px + 1, f, 1, ur, st);
 }
 
 pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
@@ -1212,9 +1307,12 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
   P->executed_pairs = 0;
   for (int t = 0; t < P->n_tiles * P->slots; ++t)
     if (ur[t].y > ur[t].x) P->executed_pairs += (int64_t)(ur[t].y - ur[t].x) * 32 * kC;
+  P->steps_per_pixel = (double)P->executed_pairs / ((double)P->nx_pad * P->nz_pad);
   P->active_pairs = P->apod ? (int64_t)active : (int64_t)d.nx * d.nz * d.n_elem;
   if ((s = build_form1(P, ur, st)) != PA_OK) return s;
   if ((s = build_form2(P, ur, st)) != PA_OK) return s;
+  if ((s = build_form3(P, 1, ur, st)) != PA_OK) return s;
+  if ((s = build_form3(P, 2, ur, st)) != PA_OK) return s;
   // work items (tile, residue group) deepest tiles first; the frame is the
   // fastest index of a work item, so frames of one tile run back to back
   std::vector<int4> it((size_t)P->n_tiles * P->ngroups);
@@ -1336,8 +1434,23 @@ bool encode_rf_map(pa_plan_s* P, const void* rf, int nf, CUtensorMap* map) {
 //   * records whose rows are not 16-byte aligned (4 samples) are staged
 //     sample by sample in the one-frame form but prepared all the same in the
 //     other: 1.3-1.8 down to half as many items, odd launches included.
+// Small launches (110 plans, 1-6 frames) leave most of the GPU idle with
+// 4-pixel threads: at one pixel a thread 1.0-2.0 up to 600 warps of 4-pixel
+// threads (1100 for the plans fine_limits names), where the launch fills the
+// GPU on its own; two pixels a thread 1.04-1.55 from there to 2400 for the
+// same plans (plain FP32 0.84-1.0).  Pixels of fewer than 28 channel steps
+// (50 from 1100 warps on) do not repay the preparation pass (0.84-1.0).
 const FusedForm& pick_form(const pa_plan_s* P, int nf) {
   const FusedForm &one = P->form[0], &two = P->form[1];
+  const FineLimits lim = fine_limits(P);
+  const int64_t warps = frame_warps(P) * nf;
+  const double steps = P->item_frames == 3 ? 1e9 : P->steps_per_pixel;
+  for (int px = 1; px <= 2; ++px) {
+    const FusedForm& f = P->form[px + 1];
+    if (f.nf && nf <= f.max_frames && warps <= (px == 1 ? lim.px1 : lim.px2) &&
+        steps >= (px == 1 ? 28 : 50))
+      return f;
+  }
   if (two.nf == 0 || nf < 2) return one;
   if (P->item_frames == 2) return two;
   const double fill = (double)P->n_tiles * P->ngroups * nf / ((double)one.blocks_per_sm * P->num_sms);
@@ -1359,13 +1472,13 @@ pa_status fused_params(pa_plan_s* P, const FusedForm& f, const void* rf, int nf,
 
   BfParams& b = *bp;
   memset(&b.tmap, 0, sizeof b.tmap);
-  b.use_tma = f.nf == 1 && P->use_tma ? 1 : 0;
+  b.use_tma = !f.slots && P->use_tma ? 1 : 0;
   b.wr = P->wr;
   b.rp = f.rp;
   b.nc = f.nc;
   b.ncs = f.nc + kC - 1;
   b.tmem_cols = f.tmem_cols;
-  b.chunk_bytes = f.nf == 1 ? b.ncs * P->wr * (int)P->elt : b.ncs * P->window * P->slot_bytes;
+  b.chunk_bytes = f.slots ? b.ncs * P->window * f.slot_bytes : b.ncs * P->wr * (int)P->elt;
   b.pairs_off = f.pairs_off;
   if (b.use_tma && !encode_rf_map(P, rf, nf, &b.tmap))
     return fail(PA_ECUDA, "cuTensorMapEncodeTiled rejected the RF layout");
@@ -1412,14 +1525,15 @@ pa_status fused_params(pa_plan_s* P, const FusedForm& f, const void* rf, int nf,
   b.nz = d.nz;
   b.n_frames = nf;
   b.n_fgroups = (nf + f.nf - 1) / f.nf;
-  b.n_items = P->n_tiles * P->ngroups * b.n_fgroups;
+  b.splits = f.splits;
+  b.n_items = P->n_tiles * (f.slots && f.nf == 1 ? f.splits : P->ngroups) * b.n_fgroups;
   b.counter = scratch + 1;
   b.err = scratch;
   b.timeouts = scratch + P->scratch_ints - 1;
   b.host_flag = P->host_flag;
   b.expect_extra = P->expect_extra;
   b.stages = f.stages;
-  b.slots_dev = P->slots_dev;
+  b.slots_dev = f.slots;
   b.slot_pitch = P->slot_pitch;
   b.slot_margin = P->slot_margin;
   return PA_OK;
@@ -1439,12 +1553,12 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
   c->zero_ints = 1 + nf * P->n_out;
 
   const FusedForm& f = pick_form(P, nf);
-  const int per_round = f.nf == 2 ? P->ws_frames : nf;
+  const int per_round = f.slots ? f.max_frames : nf;
   const int n_rounds = (nf + per_round - 1) / per_round;
   c->rounds.resize(n_rounds);
   c->steps.clear();
   c->steps.reserve(2 * n_rounds + 2);
-  if (f.nf == 1) {
+  if (!f.slots) {
     Step z;
     z.spec.func = reinterpret_cast<const void*>(k_zero_ints);
     z.spec.grid = dim3(1);
@@ -1460,10 +1574,11 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
     const pa_status s = fused_params(P, f, rf_r, n, out + (size_t)f0 * planes * d.nx * d.nz, stages,
                                      scratch, &rd.b);
     if (s != PA_OK) return s;
-    if (f.nf == 2) {
+    if (f.slots) {
       PrepParams& pp = rd.pp;
       pp.rf = rf_r;
-      pp.slots = P->slots_dev;
+      pp.slots = f.slots;
+      pp.nf = f.nf;
       pp.pitch = P->slot_pitch;
       pp.margin = P->slot_margin;
       pp.rf_dtype = (int)d.rf_dtype;
@@ -1488,7 +1603,7 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
     sb.spec.block = dim3(f.threads);
     sb.spec.smem = f.smem;
     sb.args[0] = &rd.b;
-    sb.begin = f.nf == 1 ? 0 : -1;
+    sb.begin = f.slots ? -1 : 0;
     sb.end = 0;
     c->steps.push_back(sb);
   }
@@ -1953,6 +2068,19 @@ const void* bf_pipe_func(int order, bool apod, bool comp, bool full, bool neares
     case 3: return bf_pipe_func_k3(apod, comp, full, nearest);
     case 4: return bf_pipe_func_k4(apod, comp, full, nearest);
     case 5: return bf_pipe_func_k5(apod, comp, full, nearest);
+  }
+  return nullptr;
+}
+const void* bf_fine_func(int order, bool apod, bool comp, bool full, int px) {
+  switch (order) {
+    case 1: return bf_fine_func_k1(apod, comp, full, px);
+    case 2: return bf_fine_func_k2(apod, comp, full, px);
+    case 3: return bf_fine_func_k3(apod, comp, full, px);
+    case 4: return bf_fine_func_k4(apod, comp, full, px);
+    case 5: return bf_fine_func_k5(apod, comp, full, px);
+    case 6: return bf_fine_func_k6(apod, comp, full, px);
+    case 7: return bf_fine_func_k7(apod, comp, full, px);
+    case 8: return bf_fine_func_k8(apod, comp, full, px);
   }
   return nullptr;
 }

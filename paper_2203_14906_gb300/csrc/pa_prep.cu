@@ -28,6 +28,27 @@ __device__ __forceinline__ float prep_root(int order, float s) {
 
 constexpr int kPerThread = 2;
 
+// Slots of one frame each: {r[n], r[n+1] - r[n]}, or {r[n], 0} for nearest
+// samples (the same fused multiply-add then gives r[n]).
+template <int DT>
+__global__ void __launch_bounds__(256) k_prep1(const PrepParams p) {
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < p.n_zero; i += blockDim.x) p.zero[i] = 0;
+  const int row = blockIdx.x / p.blocks_per_row;  // frame * N + channel
+  const int part = blockIdx.x - row * p.blocks_per_row;
+  const size_t a0 = (size_t)row * (size_t)p.n_samples;
+  float2* dst = reinterpret_cast<float2*>(p.slots) + (size_t)(1 + row) * p.pitch + p.margin;
+#pragma unroll
+  for (int q = 0; q < kPerThread; ++q) {
+    const int n = p.n_lo + (part * kPerThread + q) * 256 + threadIdx.x;
+    if (n >= p.n_hi) return;
+    const float a = rf_load<DT>(p.rf, a0 + n);
+    float d = 0.f;
+    if (p.mode == kLinear) d = (n + 1 < p.n_samples ? rf_load<DT>(p.rf, a0 + n + 1) : 0.f) - a;
+    dst[n] = make_float2(a, d);
+  }
+}
+
 template <int DT>
 __global__ void __launch_bounds__(256) k_prep(const PrepParams p) {
   if (blockIdx.x == 0)
@@ -69,6 +90,15 @@ int pipe_slot_bytes(int mode) { return slot_bytes(mode); }
 void prep_spec(PrepParams* p, LaunchSpec* s) {
   const int per_block = 256 * kPerThread;
   p->blocks_per_row = std::max(1, (p->n_hi - p->n_lo + per_block - 1) / per_block);
+  if (p->nf == 1) {
+    s->func = p->rf_dtype == PA_RF_F32    ? reinterpret_cast<const void*>(k_prep1<PA_RF_F32>)
+              : p->rf_dtype == PA_RF_BF16 ? reinterpret_cast<const void*>(k_prep1<PA_RF_BF16>)
+                                          : reinterpret_cast<const void*>(k_prep1<PA_RF_F16>);
+    s->grid = dim3((unsigned)((long long)p->n_frames * p->n_elem * p->blocks_per_row));
+    s->block = dim3(256);
+    s->smem = 0;
+    return;
+  }
   s->func = p->rf_dtype == PA_RF_F32    ? reinterpret_cast<const void*>(k_prep<PA_RF_F32>)
             : p->rf_dtype == PA_RF_BF16 ? reinterpret_cast<const void*>(k_prep<PA_RF_BF16>)
                                         : reinterpret_cast<const void*>(k_prep<PA_RF_F16>);

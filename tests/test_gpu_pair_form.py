@@ -1,6 +1,8 @@
-"""The two-frame form of the fused kernel gives the one-frame form's bits.
+"""The two-frame and fine-grained forms of the fused kernel give the one-frame
+form's bits.
 
-PA_ITEM_FRAMES picks the form; each pixel's arithmetic is the same in both, so
+PA_ITEM_FRAMES picks the form (1: one frame per work item, 2: two, 3: one pixel
+per thread); each pixel's arithmetic is the same in both, so
 images are compared bit by bit over the forms the kernel is built for: orders
 1-5, linear and nearest samples, plain and compensated sums, apodisation,
 lattice and full delay tables, the RF types, even and odd frame counts, records
@@ -48,18 +50,35 @@ def test_bits_of_the_one_frame_form(k, dtype, comp, f_number, interp, table, ns,
     wl = _wl(ns, f_number, interp, table)
     rf = np.stack([synth.make_frame(wl, 50 + f) for f in range(frames)])
     outs = {}
-    for form in ("1", "2"):
+    for form in ("1", "2", "3"):
         monkeypatch.setenv("PA_ITEM_FRAMES", form)
         outs[form], info, deq = run_gpu(wl, rf, k, rf_dtype=dtype, compensated=comp)
         assert info["device_error_flags"] == 0
-    assert np.array_equal(outs["1"], outs["2"])
+    assert np.array_equal(outs["1"], outs["2"]) and np.array_equal(outs["1"], outs["3"])
     last = frames - 1
     refs = oracle_frames(wl, deq[last:], k)
     assert_parity(compare(outs["2"][last:], refs), 1e-4, what=f"k={k} {interp} {table}")
 
 
-def test_checked_build_sees_no_access_out_of_range(monkeypatch):
-    monkeypatch.setenv("PA_ITEM_FRAMES", "2")
+def test_two_pixels_a_thread_and_high_orders():
+    """Launches between the lines of the plan's own choice: two pixels a thread
+    (compensated, 1200-2400 warps) and orders above 5 at one pixel."""
+    wl = synth.workload("cfg1", n_elem=64, nx=256, nz=256, z1_m=20e-3)  # 512 warps a frame
+    for k, frames, dtype, comp, interp in ((3, 4, "bf16", 1, "linear"), (5, 3, "f32", 1, "nearest"),
+                                           (7, 1, "f32", 0, "linear"), (8, 2, "bf16", 1, "linear")):
+        w = dict(wl, interp=interp)
+        rf = np.stack([synth.make_frame(w, 80 + f) for f in range(frames)])
+        mp = pytest.MonkeyPatch()
+        out, info, _ = run_gpu(w, rf, k, rf_dtype=dtype, compensated=comp)
+        mp.setenv("PA_ITEM_FRAMES", "1")
+        ref, _, _ = run_gpu(w, rf, k, rf_dtype=dtype, compensated=comp)
+        mp.undo()
+        assert info["device_error_flags"] == 0 and np.array_equal(out, ref), (k, frames)
+
+
+@pytest.mark.parametrize("form", ["2", "3"])
+def test_checked_build_sees_no_access_out_of_range(form, monkeypatch):
+    monkeypatch.setenv("PA_ITEM_FRAMES", form)
     for k, dtype, comp, f_number, interp, table, ns, frames in CASES[::3]:
         wl = _wl(ns, f_number, interp, table)
         rf = np.stack([synth.make_frame(wl, 50 + f) for f in range(frames)])
