@@ -191,7 +191,7 @@ struct PrepParams {
 };
 void prep_spec(PrepParams* p, LaunchSpec* s);
 
-// Post-filter / envelope parameters (one warp per depth column).
+// Post-filter / envelope parameters.
 struct PostParams {
   float* out;
   int planes;          // planes per frame
@@ -199,8 +199,11 @@ struct PostParams {
   int s_src, s_dst;    // stage index holding raw / receiving the envelope
   int nx, nz, m, log2m;
   const float2* tw;    // per-pass twiddle blocks (see twiddles() in pa_post.cu)
+  const float2* tw_reg;  // k_post_reg: e^{-2 pi i k l / M} at k L + l, k < 32, l < L = M / 32
   int n_tw;            // entries of tw
   const float* mask;   // [n_out][m] band-pass x analytic mask
+  int2 band[3];        // per output: first bin the mask keeps, rows of L bins (k_post_reg)
+  int band_rows;       // most rows of any output
   int* maxslot;        // [frames][n_out] float bits of the image maximum
   int n_frames;
   int warps_per_block;
@@ -232,6 +235,7 @@ __host__ __device__ constexpr int post_padded_len(int m) { return m + (m >> post
 int post_buffers(int m);     // M-point complex buffers per team of the post kernel
 const void* post_inplace_func(int m);  // in-place kernel for M points, or nullptr
 int post_team_warps(int m);  // warps per team (column pair) of the post kernel
+const void* post_reg_func(int m);      // register kernel for M points, or nullptr
 void log_spec(const LogParams& p, int num_sms, LaunchSpec* s);
 
 cudaError_t bf_occupancy(const void* func, int block, size_t smem, int* blocks_per_sm);

@@ -110,6 +110,8 @@ struct pa_plan_s {
   bool pairs_pay = false;  // resident warps and slot reuse of the two-frame form suffice
   // post
   int M = 1, log2M = 0, post_wpb = 1, n_out = 0, n_tw = 0;
+  int2 band[3] = {};  // bins each output keeps (PostParams)
+  int band_rows = 0;
   int out_id[3] = {-1, -1, -1};  // output slot (0..n_out) of DAS, DMAS, HO
   uint32_t warnings = 0;
   float dyn_range = 60.f;
@@ -842,7 +844,7 @@ size_t table_bytes(const pa_plan_s* P) {
     b += (size_t)P->n_tiles * P->ngroups * sizeof(int2) + slots_size(P, 1, &frames);
   const size_t fine = slots_size(P, 2, &frames);
   if (frames) b += fine + 2 * (size_t)P->n_tiles * sizeof(int2);
-  b += (size_t)2 * P->M * sizeof(float2) + (size_t)3 * P->M * sizeof(float);
+  b += (size_t)3 * P->M * sizeof(float2) + (size_t)3 * P->M * sizeof(float);
   return b;
 }
 
@@ -1186,7 +1188,7 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
   if ((s = dalloc(P, &P->slot_rg, (size_t)P->slots)) != PA_OK) return s;
   if ((s = dalloc(P, &P->lo, (size_t)P->n_tiles * P->nv)) != PA_OK) return s;
   if ((s = dalloc(P, &P->urange, (size_t)P->n_tiles * P->slots)) != PA_OK) return s;
-  if ((s = dalloc(P, &P->tw, (size_t)2 * P->M)) != PA_OK) return s;  // >= n_tw
+  if ((s = dalloc(P, &P->tw, (size_t)3 * P->M)) != PA_OK) return s;  // n_tw <= 2 M, tw_reg
   if ((s = dalloc(P, &P->mask, (size_t)3 * P->M)) != PA_OK) return s;
   // [0] error flags, [1] work counter, [2, 2 + 3 max_batch) image maxima,
   // [last] running count of timed-out waits
@@ -1351,6 +1353,15 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
     if (tw.empty()) tw.push_back(make_float2(1.f, 0.f));
   }
   P->n_tw = (int)tw.size();
+  if (post_reg_func(P->M)) {  // then the twiddles between the two levels of M = 32 L
+    const int L = P->M / 32;
+    tw.resize((size_t)2 * P->M);
+    for (int k = 0; k < 32; ++k)
+      for (int l = 0; l < L; ++l) {
+        const double ang = -2.0 * M_PI * (double)k * l / P->M;
+        tw.push_back(make_float2((float)std::cos(ang), (float)std::sin(ang)));
+      }
+  }
   std::vector<float> mk((size_t)3 * P->M, 0.f);
   const bool even_of[3] = {false, true, (P->K % 2) == 0};
   for (int o = 0; o < 3; ++o) {
@@ -1358,10 +1369,24 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
     if (build_mask(d, even_of[o], P->M, mk.data() + (size_t)P->out_id[o] * P->M))
       P->warnings |= 1u << P->out_id[o];
   }
+  // first bin each output's mask keeps and rows of L = M / 32 bins from it on
+  if (post_reg_func(P->M)) {
+    const int L = P->M / 32;
+    for (int o = 0; o < P->n_out; ++o) {
+      int first = -1, last = -1;
+      for (int b = 0; b < P->M; ++b)
+        if (mk[(size_t)o * P->M + b] != 0.f) {
+          if (first < 0) first = b;
+          last = b;
+        }
+      P->band[o] = first < 0 ? make_int2(0, 0) : make_int2(first, (last - first) / L + 1);
+      P->band_rows = std::max(P->band_rows, P->band[o].y);
+    }
+  }
   PA_CUDA(cudaMemcpyAsync(P->tw, tw.data(), tw.size() * sizeof(float2), cudaMemcpyHostToDevice, st));
   PA_CUDA(cudaMemcpyAsync(P->mask, mk.data(), mk.size() * sizeof(float), cudaMemcpyHostToDevice,
                           st));
-  // post kernel: (3 post_wpb post_padded_len(M) + M) * 8 bytes, at most 200 KiB
+  // post kernels: at most 200 KiB of shared memory a block
   PA_CUDA(post_configure((size_t)200 * 1024));
   PA_CUDA(cudaStreamSynchronize(st));
   return PA_OK;
@@ -1621,8 +1646,11 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
   q.m = P->M;
   q.log2m = P->log2M;
   q.tw = P->tw;
+  q.tw_reg = P->tw + (size_t)2 * P->M;
   q.n_tw = P->n_tw;
   q.mask = P->mask;
+  for (int o = 0; o < 3; ++o) q.band[o] = P->band[o];
+  q.band_rows = P->band_rows;
   q.maxslot = scratch + 2;
   q.n_frames = nf;
   q.warps_per_block = P->post_wpb;
