@@ -78,6 +78,7 @@ struct FusedForm {
   // prepared slots: a row of zeros, then one row of slot_pitch slots per
   // (frames of an item, channel), for max_frames frames a round (forms 2 and
   // 3: at most that many frames a launch)
+  int slots_form = 0;     // this form's index if it reads slots
   int slot_bytes = 0;
   unsigned char* slots = nullptr;
   int max_frames = 0;
@@ -95,7 +96,7 @@ struct pa_plan_s {
   int u0 = 0, u1 = 0, nv = 0, dmin = 0, ndrows = 0, tgroups = 0, window = 0;
   size_t full_entries = 0;  // entries of the full table (n_tiles * (steps + 3) * 32 * slots * kC)
   FusedForm form[4];
-  unsigned char* fine_slots = nullptr;  // prepared slots of forms 2 and 3
+  unsigned char* form_mem = nullptr;  // slots of forms 1-3 and all forms' chunk ranges
   long long slot_pitch = 0;
   int used_lo = 0, used_hi = 0;  // samples [used_lo, used_hi) lie in some window
   int slot_margin = 0, slot_mode = 0;
@@ -754,25 +755,38 @@ void configure(pa_plan_s* P) {
 // and threads (the occupancy calculator reports one block per SM for a
 // kernel that allocates tensor memory) and is capped so that the resident
 // blocks' TMEM columns fit the SM's 512.
+// (Resident blocks of form f from its kernel's attributes a: what the
+// occupancy calculator gives without tensor memory.)
+int blocks_by_attributes(const FusedForm& f, const cudaFuncAttributes& a, size_t smem) {
+  struct Limits {
+    int regs = 0, smem = 0, threads = 0, blocks = 0, reserved = 0;
+    explicit Limits(int dev) {
+      cudaDeviceGetAttribute(&regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev);
+      cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
+      cudaDeviceGetAttribute(&threads, cudaDevAttrMaxThreadsPerMultiProcessor, dev);
+      cudaDeviceGetAttribute(&blocks, cudaDevAttrMaxBlocksPerMultiprocessor, dev);
+      cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
+    }
+  };
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  const Limits lim(dev);
+  const int warps = (f.threads + 31) / 32;
+  const int regs_warp = ((a.numRegs * 32 + 255) / 256) * 256;  // 256-register units per warp
+  int b = std::min(lim.regs / std::max(1, regs_warp * warps), lim.threads / (32 * warps));
+  b = std::min(b, (int)((size_t)lim.smem / (smem + a.sharedSizeBytes + (size_t)lim.reserved)));
+  b = std::min(b, lim.blocks);
+  if (f.tmem_cols) b = std::min(b, kTmemColsPerSm / f.tmem_cols);
+  return std::max(0, b);
+}
+
 cudaError_t fused_blocks_per_sm(const pa_plan_s* P, const FusedForm& f, size_t smem, int* n) {
   cudaError_t e = bf_occupancy(f.func, f.threads, smem, n);
   if (e != cudaSuccess || !f.tmem_cols) return e;
   cudaFuncAttributes a;
   e = cudaFuncGetAttributes(&a, f.func);
   if (e != cudaSuccess) return e;
-  int dev = 0, regs_sm = 0, smem_sm = 0, thr_sm = 0, blk_sm = 0, rsv = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  cudaDeviceGetAttribute(&regs_sm, cudaDevAttrMaxRegistersPerMultiprocessor, dev);
-  cudaDeviceGetAttribute(&smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
-  cudaDeviceGetAttribute(&thr_sm, cudaDevAttrMaxThreadsPerMultiProcessor, dev);
-  cudaDeviceGetAttribute(&blk_sm, cudaDevAttrMaxBlocksPerMultiprocessor, dev);
-  cudaDeviceGetAttribute(&rsv, cudaDevAttrReservedSharedMemoryPerBlock, dev);
-  const int warps = (f.threads + 31) / 32;
-  const int regs_warp = ((a.numRegs * 32 + 255) / 256) * 256;  // 256-register units per warp
-  int b = std::min(regs_sm / std::max(1, regs_warp * warps), thr_sm / (32 * warps));
-  b = std::min(b, (int)((size_t)smem_sm / (smem + a.sharedSizeBytes + (size_t)rsv)));
-  b = std::min(b, blk_sm);
-  *n = std::max(0, std::min(b, kTmemColsPerSm / f.tmem_cols));
+  *n = blocks_by_attributes(f, a, smem);
   return cudaSuccess;
 }
 
@@ -780,6 +794,10 @@ cudaError_t fused_blocks_per_sm(const pa_plan_s* P, const FusedForm& f, size_t s
 bool wants_pairs(const pa_plan_s* P) {
   return P->d.max_batch > 1 && P->K <= 5 && P->item_frames != 1 && P->item_frames != 3;
 }
+
+// The one-frame form stages this plan's RF windows sample by sample (rows off
+// 16-byte boundaries).
+bool staged_by_samples(const pa_plan_s* P) { return !P->use_tma && P->d.n_samples % 4 != 0; }
 
 // Largest launch, in warps of 4-pixel threads, of the fine-grained forms
 // (pick_form says where the lines lie): one pixel a thread, and two.  They
@@ -791,9 +809,11 @@ struct FineLimits {
 FineLimits fine_limits(const pa_plan_s* P) {
   if (P->item_frames == 3) return {1 << 20, 1 << 20};  // tests
   if (P->item_frames != 0) return {0, 0};
-  const bool scalar = !P->use_tma && P->d.n_samples % 4 != 0;
-  return P->comp || P->full || scalar ? FineLimits{1100, 2400} : FineLimits{600, 0};
+  return P->comp || P->full || staged_by_samples(P) ? FineLimits{1100, 2400} : FineLimits{600, 0};
 }
+// Least mean channel steps per pixel of those forms.
+constexpr double kFineSteps1 = 28, kFineSteps2 = 50;
+double fine_steps(const pa_plan_s* P) { return P->item_frames == 3 ? 1e9 : P->steps_per_pixel; }
 // Warps of 4-pixel threads of one frame.
 int64_t frame_warps(const pa_plan_s* P) { return (int64_t)P->n_tiles * P->slots; }
 
@@ -886,9 +906,7 @@ void free_plan(pa_plan_s* P) {
   cudaFree(P->wtab);
   cudaFree(P->lo);
   cudaFree(P->urange);
-  for (FusedForm& f : P->form) cudaFree(f.vchunks);
-  cudaFree(P->form[1].slots);
-  cudaFree(P->fine_slots);
+  cudaFree(P->form_mem);
   cudaFree(P->items);
   cudaFree(P->slot_rg);
   cudaFree(P->tw);
@@ -953,11 +971,10 @@ bool form_dense(const pa_plan_s* P, const FusedForm& f) {
   return (size_t)f.tmem_cols * (size_t)regs_sm > (size_t)kTmemColsPerSm * regs_block;
 }
 
-// Chunk range of every (tile, share of its slots) of form f, uploaded to
-// f.vchunks: per residue group, or (form 2) of whole tiles.
-pa_status build_chunks(pa_plan_s* P, FusedForm& f, int groups, const std::vector<int2>& ur,
-                       cudaStream_t st) {
-  const int per = P->slots / groups;
+// Chunk range of every (tile, share of its slots) of form f: per residue
+// group, or (forms 2, 3) of whole tiles.
+std::vector<int2> form_chunks(const pa_plan_s* P, const FusedForm& f, const std::vector<int2>& ur) {
+  const int groups = f.slots_form > 1 ? 1 : P->ngroups, per = P->slots / groups;
   std::vector<int2> vk((size_t)P->n_tiles * groups);
   for (int t = 0; t < P->n_tiles; ++t) {
     for (int gr = 0; gr < groups; ++gr) {
@@ -974,16 +991,48 @@ pa_status build_chunks(pa_plan_s* P, FusedForm& f, int groups, const std::vector
       vk[(size_t)t * groups + gr] = c;
     }
   }
-  const pa_status s = dalloc(P, &f.vchunks, vk.size());
-  if (s != PA_OK) return s;
-  PA_CUDA(cudaMemcpyAsync(f.vchunks, vk.data(), vk.size() * sizeof(int2), cudaMemcpyHostToDevice,
-                          st));
-  PA_CUDA(cudaStreamSynchronize(st));  // vk is pageable and local
-  return PA_OK;
+  return vk;
+}
+
+// Device memory of the plan's forms, in one allocation: the slots of form 1,
+// those forms 2 and 3 share, and every form's chunk ranges.  Without room for
+// the slots the plan keeps the one-frame form alone.
+pa_status alloc_forms(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st) {
+  for (;;) {
+    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    int frames1 = 0, frames2 = 0;
+    const size_t s1 = P->form[1].nf ? up(slots_size(P, 1, &frames1)) : 0;
+    const size_t s2 = P->form[2].nf || P->form[3].nf ? up(slots_size(P, 2, &frames2)) : 0;
+    std::vector<int2> all;
+    size_t at[4] = {0, 0, 0, 0};
+    for (int i = 0; i < 4; ++i) {
+      if (!P->form[i].nf) continue;
+      at[i] = all.size();
+      const std::vector<int2> vk = form_chunks(P, P->form[i], ur);
+      all.insert(all.end(), vk.begin(), vk.end());
+    }
+    const pa_status s = dalloc(P, &P->form_mem, s1 + s2 + all.size() * sizeof(int2));
+    if (s != PA_OK) {
+      if (s1 + s2 == 0) return s;
+      for (int i = 1; i < 4; ++i) P->form[i] = FusedForm();
+      continue;
+    }
+    if (s1 + s2) PA_CUDA(cudaMemsetAsync(P->form_mem, 0, s1 + s2, st));
+    int2* vk = reinterpret_cast<int2*>(P->form_mem + s1 + s2);
+    // (pageable: the call returns once `all` has been read)
+    PA_CUDA(cudaMemcpyAsync(vk, all.data(), all.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
+    for (int i = 0; i < 4; ++i) {
+      if (!P->form[i].nf) continue;
+      P->form[i].vchunks = vk + at[i];
+      if (i) P->form[i].slots = P->form_mem + (i == 1 ? 0 : s1);
+      P->form[i].max_frames = i == 1 ? frames1 : frames2;
+    }
+    return PA_OK;
+  }
 }
 
 // The one-frame form.
-pa_status build_form1(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st) {
+pa_status build_form1(pa_plan_s* P) {
   FusedForm& f = P->form[0];
   f.nf = 1;
   f.func = bf_func(P->K, P->apod, P->comp, P->full);
@@ -1045,32 +1094,11 @@ pa_status build_form1(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st
   if (f.blocks_per_sm < 1)
     return fail(PA_EUNSUPPORTED, "fused kernel does not fit an SM (%d threads, %zu B smem)",
                 P->threads, f.smem);
-  return build_chunks(P, f, P->ngroups, ur, st);
-}
-
-// Slots and chunk ranges of form i, which the plan then has; without room for
-// its slots the plan does without it.
-pa_status finish_form(pa_plan_s* P, int i, FusedForm& f, int groups, const std::vector<int2>& ur,
-                      cudaStream_t st) {
-  const size_t bytes = slots_size(P, i, &f.max_frames);
-  if (f.max_frames == 0) return PA_OK;
-  unsigned char** slots = i == 1 ? &f.slots : &P->fine_slots;
-  if (!*slots) {
-    if (dalloc(P, slots, bytes) != PA_OK) return PA_OK;
-    const cudaError_t e = cudaMemsetAsync(*slots, 0, bytes, st);
-    if (e != cudaSuccess) {
-      if (i == 1) cudaFree(f.slots);
-      return fail(PA_ECUDA, "cudaMemsetAsync: %s", cudaGetErrorString(e));
-    }
-  }
-  f.slots = *slots;
-  const pa_status s = build_chunks(P, f, groups, ur, st);
-  P->form[i] = f;  // (a failed plan is freed whole)
-  return s;
+  return PA_OK;
 }
 
 // The two-frame form; a plan it does not fit keeps the one-frame form alone.
-pa_status build_form2(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st) {
+pa_status build_form2(pa_plan_s* P) {
   if (!wants_pairs(P)) return PA_OK;
   FusedForm f;
   f.nf = 2;
@@ -1078,16 +1106,14 @@ pa_status build_form2(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st
   f.func = bf_pipe_func(P->K, P->apod, P->comp, P->full, P->d.interp == PA_INTERP_NEAREST);
   f.threads = P->threads;
   f.stages = 2;
-  if (const char* e = getenv("PA_STAGES")) f.stages = atoi(e);
   f.tmem_cols = P->comp ? tmem_columns(P->warps, 2 * (P->K <= 2 ? 3 : P->K + 2)) : 0;
   if (f.tmem_cols > kTmemColsPerSm) return PA_OK;
   const int steps = P->u1 - P->u0;
+  cudaFuncAttributes fa;
+  PA_CUDA(cudaFuncGetAttributes(&fa, f.func));
   auto occupancy = [&](int c) {
-    int b = 0;
-    if (form_smem(P, f, c, nullptr) > 226 * 1024 ||
-        fused_blocks_per_sm(P, f, form_smem(P, f, c, nullptr), &b) != cudaSuccess)
-      b = 0;
-    return b;
+    const size_t smem = form_smem(P, f, c, nullptr);
+    return smem > 226 * 1024 ? 0 : blocks_by_attributes(f, fa, smem);
   };
   auto even = [&](int nch) { return ((steps + nch - 1) / nch + kC - 1) / kC * kC; };
   int cap = kNCMax;
@@ -1105,7 +1131,6 @@ pa_status build_form2(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st
         break;
       }
     }
-  cudaGetLastError();
   if (!best) return PA_OK;
   f.nc = best;
   f.smem = form_smem(P, f, f.nc, &f.pairs_off);
@@ -1121,15 +1146,20 @@ pa_status build_form2(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st
   const double reuse = (double)P->executed_pairs /
                        ((double)P->d.n_elem * std::max(1, P->used_hi - P->used_lo));
   P->pairs_pay = reuse >= 48 && f.blocks_per_sm * P->warps >= (P->K <= 2 ? 12 : 14);
+  // (no launch would pick the form)
+  if (!P->pairs_pay && !staged_by_samples(P) && P->item_frames != 2) return PA_OK;
   if (P->window > P->slot_margin) return PA_OK;  // (the margin bounds it)
-  return finish_form(P, 1, f, P->ngroups, ur, st);
+  f.slots_form = 1;
+  P->form[1] = f;
+  return PA_OK;
 }
 
 // The fine-grained forms: a tile's pixels at px of a thread's four per thread,
 // in blocks of at most 16 warps.
-pa_status build_form3(pa_plan_s* P, int px, const std::vector<int2>& ur, cudaStream_t st) {
+pa_status build_form3(pa_plan_s* P, int px) {
   const FineLimits lim = fine_limits(P);
   if (frame_warps(P) > (px == 1 ? lim.px1 : lim.px2) || P->window > P->slot_margin) return PA_OK;
+  if (fine_steps(P) < (px == 1 ? kFineSteps1 : kFineSteps2)) return PA_OK;
   FusedForm f;
   f.nf = 1;
   f.slot_bytes = sizeof(float2);
@@ -1142,12 +1172,11 @@ pa_status build_form3(pa_plan_s* P, int px, const std::vector<int2>& ur, cudaStr
   f.threads = 32 * nw;
   f.func = bf_fine_func(P->K, P->apod, P->comp, P->full, px);
   const int steps = P->u1 - P->u0;
+  cudaFuncAttributes fa;
+  PA_CUDA(cudaFuncGetAttributes(&fa, f.func));
   auto occupancy = [&](int c) {
-    int b = 0;
-    if (form_smem(P, f, c, nullptr) > 226 * 1024 ||
-        fused_blocks_per_sm(P, f, form_smem(P, f, c, nullptr), &b) != cudaSuccess)
-      b = 0;
-    return b;
+    const size_t smem = form_smem(P, f, c, nullptr);
+    return smem > 226 * 1024 ? 0 : blocks_by_attributes(f, fa, smem);
   };
   // the longest evenly cut chunk that leaves 32 warps an SM (or as many as
   // registers allow)
@@ -1161,13 +1190,14 @@ pa_status build_form3(pa_plan_s* P, int px, const std::vector<int2>& ur, cudaStr
     const int b = occupancy(c);
     if (b >= 1 && b * nw >= std::min(most * nw, 32)) best = c;
   }
-  cudaGetLastError();
   if (!best) return PA_OK;
   f.nc = best;
   f.smem = form_smem(P, f, f.nc, &f.pairs_off);
   PA_CUDA(fused_blocks_per_sm(P, f, f.smem, &f.blocks_per_sm));
   if (f.blocks_per_sm < 1) return PA_OK;
-  return finish_form(P, px + 1, f, 1, ur, st);
+  f.slots_form = px + 1;
+  P->form[px + 1] = f;
+  return PA_OK;
 }
 
 pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
@@ -1311,10 +1341,11 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
     if (ur[t].y > ur[t].x) P->executed_pairs += (int64_t)(ur[t].y - ur[t].x) * 32 * kC;
   P->steps_per_pixel = (double)P->executed_pairs / ((double)P->nx_pad * P->nz_pad);
   P->active_pairs = P->apod ? (int64_t)active : (int64_t)d.nx * d.nz * d.n_elem;
-  if ((s = build_form1(P, ur, st)) != PA_OK) return s;
-  if ((s = build_form2(P, ur, st)) != PA_OK) return s;
-  if ((s = build_form3(P, 1, ur, st)) != PA_OK) return s;
-  if ((s = build_form3(P, 2, ur, st)) != PA_OK) return s;
+  if ((s = build_form1(P)) != PA_OK) return s;
+  if ((s = build_form2(P)) != PA_OK) return s;
+  if ((s = build_form3(P, 1)) != PA_OK) return s;
+  if ((s = build_form3(P, 2)) != PA_OK) return s;
+  if ((s = alloc_forms(P, ur, st)) != PA_OK) return s;
   // work items (tile, residue group) deepest tiles first; the frame is the
   // fastest index of a work item, so frames of one tile run back to back
   std::vector<int4> it((size_t)P->n_tiles * P->ngroups);
@@ -1469,18 +1500,14 @@ const FusedForm& pick_form(const pa_plan_s* P, int nf) {
   const FusedForm &one = P->form[0], &two = P->form[1];
   const FineLimits lim = fine_limits(P);
   const int64_t warps = frame_warps(P) * nf;
-  const double steps = P->item_frames == 3 ? 1e9 : P->steps_per_pixel;
   for (int px = 1; px <= 2; ++px) {
     const FusedForm& f = P->form[px + 1];
-    if (f.nf && nf <= f.max_frames && warps <= (px == 1 ? lim.px1 : lim.px2) &&
-        steps >= (px == 1 ? 28 : 50))
-      return f;
+    if (f.nf && nf <= f.max_frames && warps <= (px == 1 ? lim.px1 : lim.px2)) return f;
   }
   if (two.nf == 0 || nf < 2) return one;
   if (P->item_frames == 2) return two;
   const double fill = (double)P->n_tiles * P->ngroups * nf / ((double)one.blocks_per_sm * P->num_sms);
-  const bool scalar = !P->use_tma && P->d.n_samples % 4 != 0;
-  const bool pays = scalar ? fill >= 0.3
+  const bool pays = staged_by_samples(P) ? fill >= 0.3
                            : fill >= 0.65 && (nf % 2 == 0 || nf >= 7) && P->pairs_pay;
   return pays ? two : one;
 }
