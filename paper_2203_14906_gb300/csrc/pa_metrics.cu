@@ -1,18 +1,33 @@
 // pa_metrics.cu -- image-quality metrics of Section 3 (SNR Eq. 10, CR
 // Eq. 11, gCNR Eq. 12, lateral FWHM) on device-resident images.
 //
-// Work is split into "slots": one slot is one region (target or background)
-// of one ROI pair on one image.  Each slot's bounding box of pixels is cut
-// into G chunks, one thread block per chunk, so large regions spread over the
-// whole GPU while small ones cost a block each.  Reductions are written per
-// block and summed in block order afterwards, so results do not depend on
-// scheduling.  Region membership is decided once per image column: the
-// pixels of a disc, rectangle or annulus in one column form one row interval
-// (minus an inner interval for the annulus), found by binary search with the
-// exact FP64 test, so the passes read member pixels only, warp by column with
-// coalesced loads and no per-pixel floating-point test.  Launches:
-//   ranges   per (region, column): the member row interval(s)
-// and per chunk of ROI pairs:
+// Region membership is decided once per image column: the pixels of a disc,
+// rectangle or annulus in one column form one row interval (minus an inner
+// interval for the annulus), found with the exact FP64 test, so the passes
+// read member pixels only.  Then one of two paths; results do not depend on
+// scheduling in either.
+//
+// k_m_pair, when the members of every ROI pair fit in shared memory: one
+// block per (image, ROI pair) fetches the pair's members once (4 B
+// asynchronous copies, all in flight together) and does everything else from
+// there: sums, maximum, deviations, histograms, the FWHM walk and the record.
+// The pixel indices of a region's members are listed once per call, by
+// k_m_members, so no image walks columns.  What bounds it is the chain of its
+// phases within a block, not the memory (14 KB a pair).  FP64 instructions run
+// at 2 lanes per clock and SM here, 1/64 of FP32, so the sums are kept as
+// three floats each by exact additions (72 bits, more than a double) and
+// become doubles once per region; the largest error of sigma_out against 64
+// bits fell from 3.4e-16 to 1.8e-16 of it.  Device time, this path against the
+// general one: 96 images x 10 pairs of 3600 pixels 41 against 180 us, 96 x 16
+// of 24000 199 / 604, one image and one pair of 700 pixels 19 / 53.  At the
+// limit of 51200 values the two meet for few pairs (45000 values: 50 / 72 us
+// for one pair, 127 / 373 for 512).
+//
+// The general path, for larger regions.  Work is split into "slots": one slot
+// is one region (target or background) of one ROI pair on one image.  Each
+// slot's bounding box of pixels is cut into G chunks, one thread block per
+// chunk, so large regions spread over the whole GPU.  Reductions are written
+// per block and summed in block order afterwards.  Launches:
 //   pass 1   count, sum and the largest value (with its pixel) per block
 //   reduce   per slot: count, mean, maximum
 //   pass 2   per block: sum of squared deviations from the slot's mean; the
@@ -42,18 +57,34 @@ struct MRegion {
   int shape;
   int j0, j1, l0, l1;  // bounding box of pixel indices, [j0, j1) x [l0, l1)
   long long col0;      // first entry of this region's columns in the range table
+  long long pix0;      // first entry of its members in the member list,
+  long long pix1;      // and the end of their room
   double xc, zc, a, b;
 };
 
 // Member rows of one column: [lo, hi) without [hlo, hhi).
 struct ColRange {
   int lo, hi, hlo, hhi;
+  // rows before the hole, first row behind it, rows behind it
+  __device__ __forceinline__ int before() const {
+    return max(0, (hhi > hlo ? min(hi, hlo) : hi) - lo);
+  }
+  __device__ __forceinline__ int behind_at() const { return max(lo, hhi); }
+  __device__ __forceinline__ int behind() const { return hhi > hlo ? max(0, hi - behind_at()) : 0; }
+};
+
+// Regions passed with the launch (32 x 64 B of its 4 KB of parameters), so
+// that the usual call needs no upload.
+constexpr int kParamRegions = 32;
+struct RegTable {
+  MRegion r[kParamRegions];
 };
 
 struct MGeom {
   int nx, nz, n_roi, chunks;
   long long pair0;  // first (image, roi) pair of this launch sequence
   double x0, z0, dx, dz;
+  float rows_per_m;
 };
 
 struct Part1 {
@@ -73,10 +104,12 @@ __device__ __forceinline__ unsigned int ordered_bits(float v) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
+__device__ __forceinline__ float unorder(unsigned int o) {
+  return __uint_as_float((o & 0x80000000u) ? (o & 0x7fffffffu) : ~o);
+}
+
 __device__ __forceinline__ float key_value(unsigned long long key) {
-  const unsigned int o = (unsigned int)(key >> 32);
-  const unsigned int u = (o & 0x80000000u) ? (o & 0x7fffffffu) : ~o;
-  return __uint_as_float(u);
+  return unorder((unsigned int)(key >> 32));
 }
 
 // Pixel-centre membership, FP64 with explicit round-to-nearest operations
@@ -103,6 +136,7 @@ __device__ int2 row_interval(int shape, double ex2, double zc, double rad, const
   // the test is weakest at the row nearest the centre (or at an end of the
   // column when the centre lies beyond it); rounding may move that by one
   double lc = (zc - g.z0) / g.dz - 0.5;
+  const float mid = (float)lc;
   lc = fmin(fmax(lc, 0.0), (double)(g.nz - 1));
   int lm = (int)rint(lc), seed = -1;
   for (int d = 0; d <= 2 && seed < 0; ++d) {
@@ -110,51 +144,154 @@ __device__ int2 row_interval(int shape, double ex2, double zc, double rad, const
     else if (lm + d < g.nz && row_in(shape, ex2, zc, rad, g, lm + d)) seed = lm + d;
   }
   if (seed < 0) return make_int2(0, 0);
-  int lo = 0, hi = seed;  // first member row in [0, seed]
+  // The ends lie about `half` rows from the centre.  The FP32 estimate decides
+  // nothing: the exact test is stepped outwards or inwards from it until it
+  // changes, in doubling steps (two tests an end as a rule, where a bisection
+  // of the column takes log2 nz).
+  const double rr = __dmul_rn(rad, rad);
+  const float half = g.rows_per_m *
+                     (shape == PA_REGION_RECT ? (float)rad : sqrtf(fmaxf((float)(rr - ex2), 0.f)));
+  auto in = [&](int l) { return row_in(shape, ex2, zc, rad, g, l); };
+  // first member row in [0, seed]
+  int lo = 0, hi = seed, e = (int)ceilf(fminf(fmaxf(mid - half, 0.f), (float)seed));
+  e = min(max(e, 0), seed);
+  if (in(e)) {
+    hi = e;
+    for (int step = 1; hi > 0; step = min(2 * step, 1 << 20)) {
+      const int t = max(hi - step, 0);
+      if (!in(t)) {
+        lo = t + 1;
+        break;
+      }
+      hi = t;
+    }
+  } else {
+    lo = e + 1;
+    for (int step = 1; lo < hi; step = min(2 * step, 1 << 20)) {
+      const int t = lo + min(step - 1, hi - lo);
+      if (in(t)) {
+        hi = t;
+        break;
+      }
+      lo = t + 1;
+    }
+  }
   while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (row_in(shape, ex2, zc, rad, g, mid)) hi = mid;
-    else lo = mid + 1;
+    const int m = (lo + hi) >> 1;
+    if (in(m)) hi = m;
+    else lo = m + 1;
   }
   const int first = lo;
+  // last member row in [seed, nz - 1]
   lo = seed;
-  hi = g.nz - 1;  // last member row in [seed, nz - 1]
+  hi = g.nz - 1;
+  e = (int)floorf(fminf(fmaxf(mid + half, (float)seed), (float)(g.nz - 1)));
+  e = min(max(e, seed), g.nz - 1);
+  if (in(e)) {
+    lo = e;
+    for (int step = 1; lo < g.nz - 1; step = min(2 * step, 1 << 20)) {
+      const int t = min(lo, g.nz - 1 - step) + step;
+      if (!in(t)) {
+        hi = t - 1;
+        break;
+      }
+      lo = t;
+    }
+  } else {
+    hi = e - 1;
+    for (int step = 1; lo < hi; step = min(2 * step, 1 << 20)) {
+      const int t = max(hi - step + 1, lo);
+      if (in(t)) {
+        lo = t;
+        break;
+      }
+      hi = t - 1;
+    }
+  }
   while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (row_in(shape, ex2, zc, rad, g, mid)) lo = mid;
-    else hi = mid - 1;
+    const int m = (lo + hi + 1) >> 1;
+    if (in(m)) lo = m;
+    else hi = m - 1;
   }
   return make_int2(first, lo + 1);
 }
 
-__global__ void k_m_ranges(MGeom g, const MRegion* regs, int n_regions, ColRange* ranges) {
-  const int r = blockIdx.y;
-  if (r >= n_regions) return;
-  const MRegion R = regs[r];
+// Member rows of column j in the region, or in an annulus's hole.
+__device__ __forceinline__ int2 column_interval(const MRegion& R, bool hole, int j, const MGeom& g) {
+  const double ex = __dsub_rn(px(g, j), R.xc);
+  if (R.shape == PA_REGION_RECT) {
+    if (hole || !(fabs(ex) <= R.a)) return make_int2(0, 0);
+    return row_interval(PA_REGION_RECT, 0.0, R.zc, R.b, g);
+  }
+  if (R.shape == PA_REGION_DISC && hole) return make_int2(0, 0);
+  // annulus: disc(b) without disc(a)
+  return row_interval(PA_REGION_DISC, __dmul_rn(ex, ex), R.zc,
+                      R.shape == PA_REGION_DISC || hole ? R.a : R.b, g);
+}
+
+// For the general path: one thread per (column, interval), threadIdx.y 0 the
+// region, 1 the hole of an annulus.
+__global__ void k_m_ranges(MGeom g, const MRegion* regs, ColRange* ranges) {
+  const MRegion R = regs[blockIdx.y];
   const int j = R.j0 + blockIdx.x * blockDim.x + threadIdx.x;
   if (j >= R.j1) return;
-  const double ex = __dsub_rn(px(g, j), R.xc);
-  const double ex2 = __dmul_rn(ex, ex);
-  ColRange c{0, 0, 0, 0};
-  if (R.shape == PA_REGION_RECT) {
-    if (fabs(ex) <= R.a) {
-      const int2 v = row_interval(PA_REGION_RECT, 0.0, R.zc, R.b, g);
-      c.lo = v.x;
-      c.hi = v.y;
-    }
-  } else if (R.shape == PA_REGION_DISC) {
-    const int2 v = row_interval(PA_REGION_DISC, ex2, R.zc, R.a, g);
-    c.lo = v.x;
-    c.hi = v.y;
-  } else {  // annulus: disc(b) without disc(a)
-    const int2 v = row_interval(PA_REGION_DISC, ex2, R.zc, R.b, g);
-    const int2 h = row_interval(PA_REGION_DISC, ex2, R.zc, R.a, g);
-    c.lo = v.x;
-    c.hi = v.y;
-    c.hlo = h.x;
-    c.hhi = h.y;
+  reinterpret_cast<int2*>(ranges + R.col0 + (j - R.j0))[threadIdx.y] =
+      column_interval(R, threadIdx.y != 0, j, g);
+}
+
+// The member pixels of region blockIdx.x, columns and rows ascending, for
+// k_m_pair: their number in counts and their indices j * nz + l in list, from
+// the region's place pix0 on.
+constexpr int kMemberCols = 1024;  // widest region of the list
+__global__ void __launch_bounds__(512) k_m_members(MGeom g, const __grid_constant__ RegTable tab,
+                                                   int tab_n, const MRegion* regs,
+                                                   long long* pix0, int* counts,
+                                                   unsigned int* list) {
+  __shared__ int2 iv[2][kMemberCols];
+  __shared__ int off[kMemberCols + 1];
+  const MRegion R = tab_n > 0 ? tab.r[blockIdx.x] : regs[blockIdx.x];
+  const int width = R.j1 - R.j0, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int sides = R.shape == PA_REGION_ANNULUS ? 2 : 1;
+  for (int i = threadIdx.x; i < sides * width; i += blockDim.x) {
+    const int hole = i >= width, c = i - (hole ? width : 0);
+    iv[hole][c] = column_interval(R, hole, R.j0 + c, g);
   }
-  ranges[R.col0 + (j - R.j0)] = c;
+  __syncthreads();
+  auto range = [&](int c) {
+    const int2 v = iv[0][c], h = sides > 1 ? iv[1][c] : make_int2(0, 0);
+    return ColRange{v.x, v.y, h.x, h.y};
+  };
+  if (w == 0) {
+    int run = 0;
+    for (int c0 = 0; c0 < width; c0 += 32) {
+      const int c = c0 + lane;
+      int n = 0;
+      if (c < width) {
+        const ColRange r = range(c);
+        n = r.before() + r.behind();
+      }
+      int inc = n;
+      for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += u;
+      }
+      if (c < width) off[c] = run + inc - n;
+      run += __shfl_sync(0xffffffffu, inc, 31);
+    }
+    if (lane == 0) {
+      counts[blockIdx.x] = run;
+      pix0[blockIdx.x] = R.pix0;
+    }
+  }
+  __syncthreads();
+  for (int c = w; c < width; c += (int)(blockDim.x >> 5)) {
+    const ColRange r = range(c);
+    const int n1 = r.before(), skip = r.behind_at() - n1;
+    const int n = min(n1 + r.behind(), (int)(R.pix1 - R.pix0) - off[c]);  // (never cut)
+    const unsigned int q = (unsigned)(R.j0 + c) * (unsigned)g.nz;
+    unsigned int* const dst = list + R.pix0 + off[c];
+    for (int t = lane; t < n; t += 32) dst[t] = q + (unsigned)(t + (t < n1 ? r.lo : skip));
+  }
 }
 
 struct SlotRef {
@@ -349,6 +486,260 @@ __global__ void k_m_final(MGeom g, long long n_pairs, const float* images, const
   out[pair] = m;
 }
 
+// A sum of floats as three floats, by exact additions (Knuth's two-sum): the
+// first two parts take no rounding error, the third rounds at 2^-72 of the
+// sum.  Not finite where a partial sum leaves FP32's range.
+__device__ __forceinline__ float two_sum(float a, float b, float* e) {
+  const float s = __fadd_rn(a, b), t = __fsub_rn(s, a);
+  *e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+  return s;
+}
+struct Sum3 {
+  float a = 0.f, b = 0.f, c = 0.f;
+  __device__ __forceinline__ void add(float v) {
+    float e, f;
+    a = two_sum(a, v, &e);
+    b = two_sum(b, e, &f);
+    c = __fadd_rn(c, f);
+  }
+  __device__ __forceinline__ void add_low(float v) {  // v far below the sum
+    float f;
+    b = two_sum(b, v, &f);
+    c = __fadd_rn(c, f);
+  }
+  __device__ __forceinline__ void merge(const Sum3& o) {
+    float e, f, h;
+    a = two_sum(a, o.a, &e);
+    b = two_sum(b, o.b, &f);
+    b = two_sum(b, e, &h);
+    c = __fadd_rn(__fadd_rn(c, o.c), __fadd_rn(f, h));
+  }
+  __device__ __forceinline__ void merge_lanes(int width) {  // over lane ^ 1, 2, .. width / 2
+    for (int o = width / 2; o >= 1; o >>= 1) {
+      Sum3 v;
+      v.a = __shfl_xor_sync(0xffffffffu, a, o);
+      v.b = __shfl_xor_sync(0xffffffffu, b, o);
+      v.c = __shfl_xor_sync(0xffffffffu, c, o);
+      merge(v);
+    }
+  }
+  __device__ __forceinline__ bool finite() const { return isfinite(a) && isfinite(b) && isfinite(c); }
+  __device__ __forceinline__ double value() const { return (double)a + ((double)b + (double)c); }
+};
+
+constexpr size_t kPairSmem = 200 * 1024;  // most dynamic shared memory of a block
+constexpr long long kListMax = 16 << 20;  // most entries of the member list (64 MiB)
+
+// One (image, ROI pair) per block; header of this file.  The dynamic shared
+// memory holds `cap` values: the target's, then the background's.  The
+// registers suffice for 2048 / T blocks of T threads (T = 1024) or half as
+// many (T = 256: 41 us instead of 44 for 960 pairs of 3600 pixels; with T =
+// 1024 it is 289 instead of 198 us for 1536 pairs of 24000).
+template <int T>
+__global__ void __launch_bounds__(T, T == 1024 ? 2 : 1024 / T)
+    k_m_pair(MGeom g, const int* counts, const unsigned int* list, const long long* pix0,
+             const float* images, int cap, pa_metrics* out) {
+  extern __shared__ float vals[];
+  __shared__ int hist[2][kBins];
+  __shared__ Sum3 sh_s[2][32];
+  __shared__ unsigned int sh_o[2][32], sh_i[2][32];
+  __shared__ long long sh_l[32];
+  __shared__ double sh_d[32], sh_mean[2], sh_rest, sh_ss;
+  __shared__ unsigned int sh_ord[2];
+  __shared__ int sh_peak[2], sh_walk[2], sh_bad;
+  const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, warps = blockDim.x >> 5;
+  const long long pair = g.pair0 + blockIdx.x;
+  const int roi = (int)(pair % g.n_roi);
+  const float* const img = images + (size_t)(pair / g.n_roi) * g.nx * g.nz;
+  // (never above the host's bounds; clamped so that nothing can leave `vals`)
+  const int n0 = min(counts[2 * roi], cap), n1 = min(counts[2 * roi + 1], cap - n0);
+  const unsigned int* const in0 = list + pix0[2 * roi];
+  const unsigned int* const in1 = list + pix0[2 * roi + 1];
+  auto fetch = [&](const unsigned int* q, int n, float* dst) {
+#pragma unroll 4
+    for (int t = tid; t < n; t += blockDim.x)
+      asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                       (unsigned)__cvta_generic_to_shared(dst + t)),
+                   "l"(img + __ldg(q + t)));
+  };
+  fetch(in0, n0, vals);
+  fetch(in1, n1, vals + n0);
+  for (int i = tid; i < 2 * kBins; i += blockDim.x) hist[0][i] = 0;
+  if (tid == 0) sh_bad = 0;
+  asm volatile("cp.async.wait_all;" ::: "memory");
+  __syncthreads();
+
+  // pass 1: sums, and the largest value with its first place
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    Sum3 s;
+    unsigned int ord = 0, idx = 0xffffffffu;
+    for (int t = tid; t < (side ? n1 : n0); t += blockDim.x) {
+      const float v = vals[side ? n0 + t : t];
+      s.add(v);
+      const unsigned int o = ordered_bits(v);
+      if (o > ord || idx == 0xffffffffu) {
+        ord = o;
+        idx = (unsigned)t;
+      }
+    }
+    const unsigned int top = __reduce_max_sync(0xffffffffu, ord);
+    const unsigned int first = __reduce_min_sync(0xffffffffu, ord == top ? idx : 0xffffffffu);
+    s.merge_lanes(32);
+    if (lane == 0) {
+      sh_s[side][w] = s;
+      sh_o[side][w] = top;
+      sh_i[side][w] = first;
+    }
+  }
+  __syncthreads();
+  if (w < 2) {
+    Sum3 s;
+    unsigned int ord = 0, idx = 0xffffffffu;
+    if (lane < warps) {
+      s = sh_s[w][lane];
+      ord = sh_o[w][lane];
+      idx = sh_i[w][lane];
+    }
+    const unsigned int top = __reduce_max_sync(0xffffffffu, ord);
+    const unsigned int first = __reduce_min_sync(0xffffffffu, ord == top ? idx : 0xffffffffu);
+    s.merge_lanes(32);
+    if (lane == 0) {
+      sh_ord[w] = top;
+      const double nn = (double)(w ? n1 : n0), mean = nn > 0 ? s.value() / nn : 0.0;
+      sh_mean[w] = mean;
+      // mean - (float)mean from the parts of the sum: n (float)mean is exact
+      if (w) sh_rest = nn > 0 ? (((double)s.a - nn * (double)(float)mean) + ((double)s.b + (double)s.c)) / nn : 0.0;
+      if (!s.finite()) sh_bad = 1;
+      if (w == 0 && n0 > 0) {
+        const unsigned int q = in0[first];
+        sh_peak[0] = (int)(q / (unsigned)g.nz);
+        sh_peak[1] = (int)(q % (unsigned)g.nz);
+      }
+    }
+  }
+  __syncthreads();
+  if (sh_bad) {  // values beyond FP32's range or not finite: in FP64
+    for (int side = 0; side < 2; ++side) {
+      const int ns = side ? n1 : n0;
+      const float* const v = vals + (side ? n0 : 0);
+      double s = 0.0;
+      for (int t = tid; t < ns; t += blockDim.x) s += (double)v[t];
+      s = block_reduce(s, sh_d, [](double x, double y) { return x + y; });
+      if (tid == 0) sh_mean[side] = ns > 0 ? s / (double)ns : 0.0;
+    }
+    __syncthreads();
+  }
+
+  // pass 2: histograms, and the background's squared deviations.  With m the
+  // mean rounded to FP32, v - m = d + e exactly, and
+  //   sum (v - mean)^2 = sum (d + e)^2 - n (mean - m)^2.
+  float vmax = -INFINITY;
+  if (n0 > 0) vmax = unorder(sh_ord[0]);
+  if (n1 > 0) vmax = fmaxf(vmax, unorder(sh_ord[1]));
+  for (int t = tid; t < n0; t += blockDim.x) atomicAdd(&hist[0][amp_bin(vals[t], vmax)], 1);
+  const double mean = sh_mean[1];
+  const float m = (float)mean;
+  Sum3 s;
+  for (int t = tid; t < n1; t += blockDim.x) {
+    const float v = vals[n0 + t];
+    atomicAdd(&hist[1][amp_bin(v, vmax)], 1);
+    float e;
+    const float d = two_sum(v, -m, &e);
+    const float p = __fmul_rn(d, d), pe = __fmaf_rn(d, d, -p);
+    const float c = __fmul_rn(2.f * d, e), ce = __fmaf_rn(2.f * d, e, -c);
+    s.add(p);
+    s.add_low(pe);
+    s.add_low(c);
+    s.c = __fadd_rn(s.c, __fmaf_rn(e, e, ce));
+  }
+  s.merge_lanes(32);
+  if (lane == 0) sh_s[0][w] = s;
+  // the walks along the row of the target's maximum, 32 columns at a time:
+  // jl, jr are the last columns before one below half the maximum
+  const float pk = unorder(sh_ord[0]);
+  const double half = 0.5 * (double)pk;
+  if (n0 > 0 && w < 2) {
+    const int jp = sh_peak[0];
+    const float* const row = img + sh_peak[1];
+    int end = w ? g.nx - 1 : 0;
+    for (int k = 1; w ? jp + k < g.nx : jp - k >= 0; k += 32) {
+      const int j = w ? jp + k + lane : jp - k - lane;
+      const bool in = j >= 0 && j < g.nx && (double)row[(size_t)j * g.nz] >= half;
+      const unsigned int stop = __ballot_sync(0xffffffffu, !in);
+      if (stop) {
+        const int f = k + __ffs(stop) - 2;
+        end = w ? jp + f : jp - f;
+        break;
+      }
+    }
+    if (lane == 0) sh_walk[w] = end;
+  }
+  __syncthreads();
+  // Eq. 12's overlap: sum_b min(c_in / n_in, c_out / n_out)
+  //                 = sum_b min(c_in n_out, c_out n_in) / (n_in n_out)
+  long long ov = 0;
+  for (int b = tid; b < kBins; b += blockDim.x) {
+    const long long u = (long long)hist[0][b] * n1, v = (long long)hist[1][b] * n0;
+    ov += u < v ? u : v;
+  }
+  ov = block_reduce(ov, sh_l, [](long long x, long long y) { return x + y; });
+  if (w == 0) {
+    s = lane < warps ? sh_s[0][lane] : Sum3();
+    s.merge_lanes(32);
+    if (lane == 0) {
+      const double ss = s.value() - (double)n1 * sh_rest * sh_rest;
+      sh_ss = ss;
+      // the products of tiny deviations lose bits to FP32's underflow
+      sh_bad = !(s.finite() && ss >= (double)n1 * 0x1p-70);
+    }
+  }
+  __syncthreads();
+  if (sh_bad) {
+    double q = 0.0;
+    for (int t = tid; t < n1; t += blockDim.x) {
+      const double e = (double)vals[n0 + t] - mean;
+      q += e * e;
+    }
+    q = block_reduce(q, sh_d, [](double x, double y) { return x + y; });
+    if (tid == 0) sh_ss = q;
+    __syncthreads();
+  }
+  if (w != 0) return;
+  // lanes 0 and 1 take the two quotients and the two ends of the FWHM
+  const double nan = __longlong_as_double(0x7ff8000000000000ll);
+  const double mu_in = n0 > 0 ? sh_mean[0] : nan, mu_out = n1 > 0 ? mean : nan;
+  const double sigma = n1 > 0 ? sqrt(sh_ss / (double)n1) : nan;
+  const double db = 20.0 * log10(mu_in / (lane ? mu_out : sigma));
+  const double cr = __shfl_sync(0xffffffffu, db, 1);
+  double fwhm = nan;
+  if (n0 > 0 && sh_walk[0] > 0 && sh_walk[1] < g.nx - 1) {
+    const float* const row = img + sh_peak[1];
+    const int step = lane ? 1 : -1, at = sh_walk[lane ? 1 : 0];
+    const double p = (double)row[(size_t)(at + step) * g.nz], q = (double)row[(size_t)at * g.nz];
+    const double f = __dmul_rn(__ddiv_rn(__dsub_rn(half, p), __dsub_rn(q, p)), g.dx);
+    const double x = __dadd_rn(g.x0, __dmul_rn((double)(at + step) + 0.5, g.dx));
+    const double end = lane ? __dsub_rn(x, f) : __dadd_rn(x, f);
+    fwhm = __dsub_rn(__shfl_sync(0xffffffffu, end, 1), end);
+  }
+  if (lane == 0) {
+    pa_metrics r;
+    r.mu_in = mu_in;
+    r.mu_out = mu_out;
+    r.sigma_out = sigma;
+    r.snr_db = db;
+    r.cr_db = cr;
+    r.gcnr = n0 > 0 && n1 > 0 ? 1.0 - (double)ov / ((double)n0 * (double)n1) : nan;
+    r.fwhm_m = fwhm;
+    r.peak = n0 > 0 ? (double)pk : nan;
+    r.n_in = n0;
+    r.n_out = n1;
+    r.peak_j = n0 > 0 ? sh_peak[0] : -1;
+    r.peak_l = n0 > 0 ? sh_peak[1] : -1;
+    out[pair] = r;
+  }
+}
+
 pa_status mfail(pa_status s, const char* msg) {
   pa::set_error_message(msg);
   return s;
@@ -365,6 +756,21 @@ void index_range(double c, double h, double o, double d, int n, int* lo, int* hi
   u = std::max(0.0, std::min((double)n, u));
   *lo = (int)l;
   *hi = std::max(*lo, (int)u);
+}
+
+// At least the members of a region: its bounding box, or for round regions
+// that lie within the image their area (in pixels) and half a boundary pixel
+// at each end of every column: with f the chord over a column, unimodal, the
+// sum of f over the columns differs from its integral by its maximum at most,
+// and the rows in a chord from its length by one.
+long long most_members(const MRegion& o, const MGeom& g) {
+  const long long box = (long long)(o.j1 - o.j0) * (o.l1 - o.l0);
+  if (o.shape == PA_REGION_RECT || o.j0 <= 0 || o.l0 <= 0 || o.j1 >= g.nx || o.l1 >= g.nz) return box;
+  const bool hole = o.shape == PA_REGION_ANNULUS;
+  const double out = hole ? o.b : o.a, in = hole ? std::min(o.a, o.b) : 0.0;
+  const double n = 3.1416 * out * out / (g.dx * g.dz) - 3.1415 * in * in / (g.dx * g.dz) +
+                   2.0 * (out + in) / g.dz + 2.0 * (o.j1 - o.j0) + 16.0;
+  return n < (double)box ? (long long)n : box;
 }
 
 }  // namespace
@@ -393,10 +799,14 @@ extern "C" pa_status pa_image_metrics(const pa_grid* grid, const float* images_d
   g.z0 = G.z0_m;
   g.dx = (G.x1_m - G.x0_m) / G.nx;
   g.dz = (G.z1_m - G.z0_m) / G.nz;
+  g.rows_per_m = (float)(1.0 / g.dz);
   std::vector<MRegion> regs(2 * (size_t)n_roi);
-  long long max_area = 0, n_cols = 0;
+  long long max_area = 0, n_cols = 0, n_pix = 0, cap = 0;
   int max_width = 0;
+  double reach = std::max(std::max(std::fabs(G.x0_m), std::fabs(G.x1_m)),
+                          std::max(std::fabs(G.z0_m), std::fabs(G.z1_m)));
   for (int r = 0; r < n_roi; ++r) {
+    long long members = 0;
     for (int side = 0; side < 2; ++side) {
       const pa_region& in = side ? rois[r].background : rois[r].target;
       MRegion& o = regs[2 * r + side];
@@ -410,16 +820,28 @@ extern "C" pa_status pa_image_metrics(const pa_grid* grid, const float* images_d
       o.zc = in.zc_m;
       o.a = in.a_m;
       o.b = in.b_m;
+      reach = std::max({reach, std::fabs(in.xc_m), std::fabs(in.zc_m), in.a_m, in.b_m});
       const double hx = in.shape == PA_REGION_ANNULUS ? in.b_m : in.a_m;
       const double hz = in.shape == PA_REGION_DISC ? in.a_m : in.b_m;
       index_range(in.xc_m, hx, g.x0, g.dx, g.nx, &o.j0, &o.j1);
       index_range(in.zc_m, hz, g.z0, g.dz, g.nz, &o.l0, &o.l1);
       o.col0 = n_cols;
       n_cols += o.j1 - o.j0;
+      const long long most = most_members(o, g);
+      o.pix0 = n_pix;
+      n_pix += most;
+      o.pix1 = n_pix;
+      members += most;
       max_width = std::max(max_width, o.j1 - o.j0);
       max_area = std::max(max_area, (long long)(o.j1 - o.j0) * (o.l1 - o.l0));
     }
+    cap = std::max(cap, members);
   }
+  // k_m_pair where the members of every pair fit.  The bounds hold as long as
+  // no coordinate is so far from the image that rounding costs a visible part
+  // of a pixel.
+  const bool in_block = (size_t)cap * 4 <= kPairSmem && max_width <= kMemberCols &&
+                        n_pix <= kListMax && reach <= 0x1p40 * std::min(g.dx, g.dz);
   // blocks per region: about 8192 bounding-box pixels each, at least one
   // column per warp
   const long long by_area = (max_area + 8191) / 8192, by_cols = (max_width + 7) / 8;
@@ -427,10 +849,12 @@ extern "C" pa_status pa_image_metrics(const pa_grid* grid, const float* images_d
 
   cudaStream_t st = (cudaStream_t)cuda_stream;
   const long long n_pairs = (long long)n_images * n_roi;
-  const long long pairs_per = std::min(n_pairs, kPairsPerLaunch);
-  const long long slots_per = 2 * pairs_per;
+  const long long pairs_per = std::min(n_pairs, in_block ? 1ll << 30 : kPairsPerLaunch);
+  const long long slots_per = in_block ? 0 : 2 * pairs_per;
   const size_t b_regs = regs.size() * sizeof(MRegion);
-  const size_t b_cols = (size_t)std::max<long long>(n_cols, 1) * sizeof(ColRange);
+  // (in_block: counts, places and members instead of the column ranges)
+  const size_t b_cols = in_block ? regs.size() * 12 + (size_t)n_pix * 4
+                                 : (size_t)std::max<long long>(n_cols, 1) * sizeof(ColRange);
   const size_t b_p1 = (size_t)slots_per * g.chunks * sizeof(Part1);
   const size_t b_st = (size_t)slots_per * sizeof(SlotStat);
   const size_t b_p2 = (size_t)slots_per * g.chunks * sizeof(double);
@@ -449,13 +873,37 @@ extern "C" pa_status pa_image_metrics(const pa_grid* grid, const float* images_d
   SlotStat* d_st = (SlotStat*)((char*)d_p1 + up(b_p1));
   double* d_p2 = (double*)((char*)d_st + up(b_st));
   int* d_h = (int*)((char*)d_p2 + up(b_p2));
-  e = cudaMemcpyAsync(d_regs, regs.data(), b_regs, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess && max_width > 0) {
-    const dim3 grid_r((unsigned)((max_width + 127) / 128), (unsigned)regs.size());
-    k_m_ranges<<<grid_r, 128, 0, st>>>(g, d_regs, (int)regs.size(), d_cols);
+  RegTable tab;
+  const int tab_n = in_block && regs.size() <= kParamRegions ? (int)regs.size() : 0;
+  if (tab_n) std::copy(regs.begin(), regs.end(), tab.r);
+  else e = cudaMemcpyAsync(d_regs, regs.data(), b_regs, cudaMemcpyHostToDevice, st);
+  if (in_block && e == cudaSuccess) {
+    long long* d_pix0 = (long long*)d_cols;
+    int* d_counts = (int*)(d_pix0 + regs.size());
+    unsigned int* d_list = (unsigned int*)(d_counts + regs.size());
+    k_m_members<<<(unsigned)regs.size(), 512, 0, st>>>(g, tab, tab_n, d_regs, d_pix0, d_counts, d_list);
+    e = cudaGetLastError();
+    // About 32 values a thread: 960 pairs of 4200 take 44, 43 and 49 us with
+    // 128, 256 and 512 threads, 1536 pairs of 24000 take 554, 327, 223 and 198
+    // with 128, 256, 512 and 1024.
+    int threads = 128;
+    while (threads < 1024 && cap > 32ll * threads) threads *= 2;
+    const size_t smem = (size_t)cap * 4;
+    const auto kernel = threads > 256 ? k_m_pair<1024> : k_m_pair<256>;
+    if (smem > 40 * 1024 && e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairSmem);
+    for (long long p0 = 0; e == cudaSuccess && p0 < n_pairs; p0 += pairs_per) {
+      g.pair0 = p0;
+      kernel<<<(unsigned)std::min(pairs_per, n_pairs - p0), threads, smem, st>>>(
+          g, d_counts, d_list, d_pix0, images_dev, (int)cap, out_dev);
+      e = cudaGetLastError();
+    }
+  } else if (e == cudaSuccess && max_width > 0) {
+    const dim3 grid_r((unsigned)((max_width + 31) / 32), (unsigned)regs.size());
+    k_m_ranges<<<grid_r, dim3(32, 2), 0, st>>>(g, d_regs, d_cols);
     e = cudaGetLastError();
   }
-  for (long long p0 = 0; e == cudaSuccess && p0 < n_pairs; p0 += pairs_per) {
+  for (long long p0 = 0; !in_block && e == cudaSuccess && p0 < n_pairs; p0 += pairs_per) {
     const long long np = std::min(pairs_per, n_pairs - p0);
     const long long ns = 2 * np;
     g.pair0 = p0;
