@@ -59,6 +59,7 @@ __global__ void __launch_bounds__(512, 2) k_bf_fine(const __grid_constant__ BfPa
     *reinterpret_cast<int*>(smem + kPipeStopOff) = 0;
     reinterpret_cast<int4*>(smem + kPipeProdOff)[1] = make_int4(0, 0, 0, 0);
   }
+  wait_previous();
   __syncthreads();
   int stage = 0, phase = 0;
   if (warp == 0)
@@ -236,6 +237,7 @@ __global__ void __launch_bounds__(512, 2) k_bf_fine(const __grid_constant__ BfPa
       phase ^= 1;
     }
     if (!last) continue;
+    if (reinterpret_cast<const volatile int4*>(smem + kPipeProdOff)[1].w == 2) launch_next();
     if constexpr (COMP) {
       if (folded) {
 #pragma unroll

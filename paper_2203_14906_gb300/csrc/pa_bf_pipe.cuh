@@ -334,6 +334,7 @@ __global__ void __launch_bounds__(256, 2) k_bf_pipe(const __grid_constant__ BfPa
   const int nwarps = blockDim.x >> 5;
   auto full_bar = [&](int s) { return sbase + kPipeFullOff + 8 * s; };
 
+  wait_previous();
   if constexpr (COMP) {
     if (warp == 0) {  // the whole warp allocates; the address lands in shared memory
       tmem_alloc(sbase + kPipeTmemOff, p.tmem_cols);
@@ -608,6 +609,7 @@ __global__ void __launch_bounds__(256, 2) k_bf_pipe(const __grid_constant__ BfPa
         phase ^= 1;
       }
       if (!last) continue;
+      if (reinterpret_cast<const volatile int4*>(smem + kPipeProdOff)[1].w == 2) launch_next();
 
       if constexpr (COMP) {
         if (tsum_live) final_tmem2<NA>(acc, tmem);

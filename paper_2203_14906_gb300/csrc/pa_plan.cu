@@ -491,6 +491,8 @@ __global__ void k_uranges(TileGeom g, FullGeom f, int slots, int u1, int kc, con
 
 // Clears the work counter and image maxima before a launch sequence.
 __global__ void k_zero_ints(int* p, int n) {
+  launch_next();
+  wait_previous();
   for (int i = threadIdx.x; i < n; i += blockDim.x) p[i] = 0;
 }
 
@@ -1450,6 +1452,7 @@ struct Step {
   LaunchSpec spec;
   void* args[2] = {nullptr, nullptr};
   int begin = -1, end = -1;  // kernel kind whose timing starts / ends here
+  bool chain = true;         // may follow the kernel before by a programmatic edge
 };
 struct ChunkLaunch {
   struct Round {
@@ -1684,6 +1687,9 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
   if (post) {
     Step t;
     post_spec(q, &t.spec);
+    // Few blocks, placed while the fused kernel's are leaving, share SMs that
+    // need not be shared (24 blocks of one 128 x 128 frame: call 20.6 -> 22 us).
+    t.chain = (long long)t.spec.grid.x * t.spec.grid.y * t.spec.grid.z >= P->num_sms;
     t.args[0] = &c->q;
     t.begin = t.end = 1;
     c->steps.push_back(t);
@@ -1737,6 +1743,21 @@ cudaKernelNodeParams node_params(Step& t) {
   return k;
 }
 
+// Adds kernel t after n_deps nodes, or, chained, after the kernel node deps[0]
+// with a programmatic edge (wait_previous).
+cudaError_t add_kernel_node(cudaGraph_t graph, Step& t, const cudaGraphNode_t* deps, int n_deps,
+                            bool chained, cudaGraphNode_t* n) {
+  const cudaKernelNodeParams kp = node_params(t);
+  if (!chained || !t.chain)
+    return cudaGraphAddKernelNode(n, graph, n_deps ? deps : nullptr, n_deps, &kp);
+  cudaError_t e = cudaGraphAddKernelNode(n, graph, nullptr, 0, &kp);
+  if (e != cudaSuccess) return e;
+  cudaGraphEdgeData edge{};
+  edge.from_port = cudaGraphKernelNodePortProgrammatic;
+  edge.type = cudaGraphDependencyTypeProgrammatic;
+  return cudaGraphAddDependencies(graph, deps, n, &edge, 1);
+}
+
 // One chunk as a CUDA graph: the chunk's launches in a row.  An executable
 // graph is kept per (frames, stages, timing); later calls only rewrite the
 // node parameters (buffer pointers, and the timing events) and launch it.
@@ -1781,6 +1802,7 @@ pa_status launch_graph(pa_plan_s* P, ChunkLaunch& c, int nf, uint32_t stages, cu
       return fail(PA_ECUDA, "graph build: %s", cudaGetErrorString(e));
     }
     cudaGraphNode_t prev = nullptr;
+    bool chained = false;  // prev is a kernel
     size_t next_ev = 0;
     for (Step& t : c.steps) {
       if (t.begin >= 0 && (prof >> t.begin & 1u)) {
@@ -1790,19 +1812,21 @@ pa_status launch_graph(pa_plan_s* P, ChunkLaunch& c, int nf, uint32_t stages, cu
         if (e != cudaSuccess) break;
         g.events.push_back(n);
         prev = n;
+        chained = false;
       }
-      const cudaKernelNodeParams kp = node_params(t);
       cudaGraphNode_t n = nullptr;
-      e = cudaGraphAddKernelNode(&n, graph, prev ? &prev : nullptr, prev ? 1 : 0, &kp);
+      e = add_kernel_node(graph, t, &prev, prev ? 1 : 0, chained, &n);
       if (e != cudaSuccess) break;
       g.kernels.push_back(n);
       prev = n;
+      chained = true;
       if (t.end >= 0 && (prof >> t.end & 1u)) {
         cudaGraphNode_t m = nullptr;
         e = cudaGraphAddEventRecordNode(&m, graph, &prev, 1, ev[next_ev++].second.second);
         if (e != cudaSuccess) break;
         g.events.push_back(m);
         prev = m;
+        chained = false;
       }
     }
     if (e == cudaSuccess) e = cudaGraphInstantiate(&g.exec, graph, 0);
@@ -2003,9 +2027,8 @@ pa_status build_host_graph(pa_plan_s* P, pa_plan_s::HostGraph& hg, const void* r
       cudaGraphNode_t deps[2] = {up, prev_last};
       int n_deps = prev_last ? 2 : 1;
       for (Step& t : cl.steps) {
-        const cudaKernelNodeParams kp = node_params(t);
         cudaGraphNode_t n = nullptr;
-        e = cudaGraphAddKernelNode(&n, graph, deps, n_deps, &kp);
+        e = add_kernel_node(graph, t, deps, n_deps, last != nullptr, &n);
         if (e != cudaSuccess) break;
         last = deps[0] = n;
         n_deps = 1;

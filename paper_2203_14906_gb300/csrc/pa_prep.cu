@@ -32,6 +32,8 @@ constexpr int kPerThread = 2;
 // samples (the same fused multiply-add then gives r[n]).
 template <int DT>
 __global__ void __launch_bounds__(256) k_prep1(const PrepParams p) {
+  launch_next();
+  wait_previous();
   if (blockIdx.x == 0)
     for (int i = threadIdx.x; i < p.n_zero; i += blockDim.x) p.zero[i] = 0;
   const int row = blockIdx.x / p.blocks_per_row;  // frame * N + channel
@@ -51,6 +53,8 @@ __global__ void __launch_bounds__(256) k_prep1(const PrepParams p) {
 
 template <int DT>
 __global__ void __launch_bounds__(256) k_prep(const PrepParams p) {
+  launch_next();
+  wait_previous();
   if (blockIdx.x == 0)
     for (int i = threadIdx.x; i < p.n_zero; i += blockDim.x) p.zero[i] = 0;
   const int row = blockIdx.x / p.blocks_per_row;  // frame pair * N + channel
