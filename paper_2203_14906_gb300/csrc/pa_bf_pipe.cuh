@@ -64,11 +64,9 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, int byt
       : "memory");
 }
 
-// Two FP32 products, in one instruction if PACK (each rounded as the scalar
-// product).  One packed product of a pair with itself or a constant issues in
-// the time of its two scalar ones and frees an issue slot; measured with the
-// lattice table (k = 3, 32 frames) 0.577 -> 0.549 ms, with the full table,
-// whose loads leave issue slots free, 0.257 -> 0.270 ms.
+// Two FP32 products, sums or multiply-adds, in one instruction if PACK (each
+// rounded as the scalar one).  A packed instruction takes the arithmetic pipe as
+// long as its two scalar ones and one issue slot instead of two.
 template <bool PACK>
 __device__ __forceinline__ void mul_pair(float& x, float& y, float a0, float a1, float b0, float b1) {
   if constexpr (!PACK) {
@@ -80,6 +78,86 @@ __device__ __forceinline__ void mul_pair(float& x, float& y, float a0, float a1,
       " mul.rn.f32x2 r, p, q;\n mov.b64 {%0, %1}, r;\n}"
       : "=f"(x), "=f"(y)
       : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+template <bool PACK>
+__device__ __forceinline__ void add_pair(float& x, float& y, float a0, float a1) {
+  if constexpr (!PACK) {
+    x += a0;
+    y += a1;
+    return;
+  }
+  asm("{\n .reg .b64 p, q, r;\n mov.b64 p, {%0, %1};\n mov.b64 q, {%2, %3};\n"
+      " add.rn.f32x2 r, p, q;\n mov.b64 {%0, %1}, r;\n}"
+      : "+f"(x), "+f"(y)
+      : "f"(a0), "f"(a1));
+}
+template <bool PACK>
+__device__ __forceinline__ void fma_pair(float& x, float& y, float a0, float a1, float b0, float b1) {
+  if constexpr (!PACK) {
+    x = fmaf(a0, b0, x);
+    y = fmaf(a1, b1, y);
+    return;
+  }
+  asm("{\n .reg .b64 p, q, r, t;\n mov.b64 p, {%2, %3};\n mov.b64 q, {%4, %5};\n"
+      " mov.b64 r, {%0, %1};\n fma.rn.f32x2 t, p, q, r;\n mov.b64 {%0, %1}, t;\n}"
+      : "+f"(x), "+f"(y)
+      : "f"(a0), "f"(a1), "f"(b0), "f"(b1));
+}
+
+// Which sums the two frames' pairs are added to by packed instructions, a bit
+// per sum: bit 0 v[0], bit 1 v[1], bit 2 v[3], bit 3 v[4], ...; with the bits,
+// kProducts packs the roots' products.  A packed sum saves an issue slot and
+// ties its operands to aligned register pairs; which of the two weighs more
+// depends on the registers a kernel has left, so every line is measured (RAW
+// images of 512 x 512, 16 frames; us of the fused kernel and its
+// preparation pass with the products alone packed -> with the sums below, and
+// the sets of table entries and blocks per SM below):
+//   k <= 2 nearest 175 -> 152, linear 232 -> 205, apodised nearest 96 -> 84,
+//     Kahan 238 -> 230; 1024 x 1024, 256 channels 428 -> 379
+//   k = 3 linear 287 -> 278, nearest 221 -> 215, apodised 140 -> 135, Kahan
+//     305 -> 294, both 147 -> 138
+//   k = 4 linear 319 (any sums: 321-328), nearest 240 -> 225, apodised 153 ->
+//     145, Kahan 348 -> 334, both 156 -> 150
+//   k = 5 linear 188 -> 178 (8 frames), nearest 303 -> 300, apodised 161 -> 157,
+//     Kahan 381 -> 371, both 171 -> 165
+//   nearest with Kahan sums: k = 3 303 -> 232, k = 4 337 -> 247, k = 5 322 -> 318;
+//     apodised nearest: k = 3 119, k = 4 137 -> 132, k = 5 154 -> 142
+//   k <= 2 with wider windows (3 samples a row): 277 -> 275
+// With the full table, whose loads leave issue slots free, nothing is packed
+// (the products alone: 0.257 -> 0.270 ms).
+constexpr int kProducts = 64;
+__host__ __device__ constexpr int packed_sums(int k, bool apod, bool comp, bool full, int mode) {
+  if (full) return 0;
+  if (k <= 2) return kProducts | (apod && comp ? 0 : 1);
+  if (k == 3) return kProducts | (mode == kNearestRoots ? 1 + 2 + 4 : 1 + 2 + 4 + 8);
+  if (k == 4) {
+    if (mode == kNearestRoots || (apod && comp)) return kProducts | (1 + 4 + 8);
+    return kProducts | (apod || comp ? 1 + 2 + 4 + 8 + 16 : 0);
+  }
+  if (apod && comp) return kProducts | (1 + 8);
+  if (comp) return kProducts | (1 + 4 + 8 + 32);
+  if (apod || mode == kNearestRoots) return kProducts | (1 + 4 + 8);
+  return kProducts | 63;
+}
+
+// Blocks per SM.  Orders <= 2 have 24 sums a thread and run 24 warps a SM on 80
+// registers (16 warps: nearest k = 2 174 us instead of 153; 32 warps on 64
+// registers: 168), but for Kahan sums over the full aperture: their folds leave
+// room for one set of table entries only there, which takes 222 us instead of 230
+// in a full launch, but 33.0 instead of 31.9 in one of 200 blocks (six BF16 frames
+// of 256 x 256) and 289 instead of 285 with wide windows.
+__host__ __device__ constexpr int pipe_blocks(int k, bool apod, bool comp) {
+  return k <= 2 && (apod || !comp) ? 3 : 2;
+}
+// Sets of table entries: with one the next block's entries replace those just
+// used, with two they are loaded a block ahead.  Two where registers last for
+// them (k = 4 linear 319, with one 350; k <= 2 205, with one 222; apodised plain
+// k = 3 135, with one 137); one for k = 5 and apodised plans (k = 5 188, with two
+// 225; apodised k = 5 161, with two 179), and with Kahan sums or all the sums of
+// k = 3 packed (Kahan k = 4 334, with two 340).
+__host__ __device__ constexpr bool one_entry_set(int k, bool apod, bool comp, int mode) {
+  if (apod) return !(k == 3 && !comp);
+  return k == 5 || (k >= 3 && mode != kNearestRoots && (k == 3 || comp));
 }
 
 // The root a sample's power sums start from: sgn sqrt|s| (orders <= 2),
@@ -95,54 +173,40 @@ __device__ __forceinline__ float base_root(float s) {
 
 // The power sums of one pixel for the samples s, t of two frames with their
 // base roots y, z: pair_update's operations in its order, so a frame's sums
-// have the bits of the one-frame kernel.
-template <int K, bool PACK>
+// have the bits of the one-frame kernel.  PK: packed_sums.
+template <int K, int PK>
 __device__ __forceinline__ void sums2(float* v, float* w, float s, float t, float y, float z) {
-  v[0] += s;
-  w[0] += t;
+  constexpr bool kMul = (PK & kProducts) != 0;
+  add_pair<(PK & 1) != 0>(v[0], w[0], s, t);
   v[2] += fabsf(s);
   w[2] += fabsf(t);
   if constexpr (K <= 2) {
-    v[1] += y;
-    w[1] += z;
-  } else if constexpr (K == 3 || K == 5) {
-    float y2, z2;
-    mul_pair<PACK>(y2, z2, y, z, y, z);
-    const float x = copysignf(y2, s), u = copysignf(z2, t);
-    if constexpr (K == 3) {
-      v[1] = fmaf(x, y, v[1]);
-      w[1] = fmaf(u, z, w[1]);
-      v[3] += x;
-      w[3] += u;
-      v[4] = fmaf(y2, y2, v[4]);
-      w[4] = fmaf(z2, z2, w[4]);
-    } else {
-      float x2, u2, y3, z3;
-      mul_pair<PACK>(x2, u2, y2, z2, y2, z2);
-      mul_pair<PACK>(y3, z3, y2, z2, y, z);
-      v[1] = fmaf(x, y3, v[1]);
-      w[1] = fmaf(u, z3, w[1]);
-      v[3] += x;
-      w[3] += u;
-      v[4] += x2;
-      w[4] += u2;
-      v[5] = fmaf(x, x2, v[5]);
-      w[5] = fmaf(u, u2, w[5]);
-      v[6] = fmaf(x2, x2, v[6]);
-      w[6] = fmaf(u2, u2, w[6]);
-    }
+    add_pair<(PK & 2) != 0>(v[1], w[1], y, z);
   } else {
     float y2, z2;
-    mul_pair<PACK>(y2, z2, y, z, y, z);
-    const float x = copysignf(y, s), u = copysignf(z, t);
-    v[1] = fmaf(x, y, v[1]);
-    w[1] = fmaf(u, z, w[1]);
-    v[3] += x;
-    w[3] += u;
-    v[4] += y2;
-    w[4] += z2;
-    v[5] = fmaf(x, y2, v[5]);
-    w[5] = fmaf(u, z2, w[5]);
+    mul_pair<kMul>(y2, z2, y, z, y, z);
+    if constexpr (K == 3) {
+      const float x = copysignf(y2, s), u = copysignf(z2, t);
+      fma_pair<(PK & 2) != 0>(v[1], w[1], x, u, y, z);
+      add_pair<(PK & 4) != 0>(v[3], w[3], x, u);
+      fma_pair<(PK & 8) != 0>(v[4], w[4], y2, z2, y2, z2);
+    } else if constexpr (K == 4) {
+      const float x = copysignf(y, s), u = copysignf(z, t);
+      fma_pair<(PK & 2) != 0>(v[1], w[1], x, u, y, z);
+      add_pair<(PK & 4) != 0>(v[3], w[3], x, u);
+      add_pair<(PK & 8) != 0>(v[4], w[4], y2, z2);
+      fma_pair<(PK & 16) != 0>(v[5], w[5], x, u, y2, z2);
+    } else {
+      const float x = copysignf(y2, s), u = copysignf(z2, t);
+      float x2, u2, y3, z3;
+      mul_pair<kMul>(x2, u2, y2, z2, y2, z2);
+      mul_pair<kMul>(y3, z3, y2, z2, y, z);
+      fma_pair<(PK & 2) != 0>(v[1], w[1], x, u, y3, z3);
+      add_pair<(PK & 4) != 0>(v[3], w[3], x, u);
+      add_pair<(PK & 8) != 0>(v[4], w[4], x2, u2);
+      fma_pair<(PK & 16) != 0>(v[5], w[5], x, u, x2, u2);
+      fma_pair<(PK & 32) != 0>(v[6], w[6], x2, u2, x2, u2);
+    }
   }
 }
 
@@ -157,7 +221,7 @@ __device__ __forceinline__ int4 load_entries16(const int2* p) {
 }
 
 // One slot of a step: load, form the samples of both frames, add.
-template <int K, int MODE, bool APOD, bool PACK>
+template <int K, int MODE, bool APOD, int PK>
 __device__ __forceinline__ void slot_pair(float* v, float* w, int addr, float a, float weight) {
   float s, t, y = 0.f, z = 0.f;
   if constexpr (MODE == kNearest) {
@@ -179,7 +243,7 @@ __device__ __forceinline__ void slot_pair(float* v, float* w, int addr, float a,
     if constexpr (K == 3 || K == 5) {
       constexpr float c = K == 3 ? 1.0f / 6.0f : 0.1f;
       float ls, lt;
-      mul_pair<PACK>(ls, lt, lg2_approx(fabsf(s)), lg2_approx(fabsf(t)), c, c);
+      mul_pair<(PK & kProducts) != 0>(ls, lt, lg2_approx(fabsf(s)), lg2_approx(fabsf(t)), c, c);
       y = ex2_approx(ls);
       z = ex2_approx(lt);
     } else {
@@ -187,7 +251,7 @@ __device__ __forceinline__ void slot_pair(float* v, float* w, int addr, float a,
       z = base_root<K>(t);
     }
   }
-  sums2<K, PACK>(v, w, s, t, y, z);
+  sums2<K, PK>(v, w, s, t, y, z);
 }
 
 // Kahan totals in TMEM as in the one-frame kernel; frame h of the item owns
@@ -326,8 +390,9 @@ __device__ __forceinline__ void produce(const BfParams& p, unsigned char* smem, 
 }
 
 template <int K, bool APOD, bool COMP, bool FULL, int MODE>
-__global__ void __launch_bounds__(256, 2) k_bf_pipe(const __grid_constant__ BfParams p) {
+__global__ void __launch_bounds__(256, pipe_blocks(K, APOD, COMP)) k_bf_pipe(const __grid_constant__ BfParams p) {
   constexpr int NA = NAcc<K>::value, SB = slot_bytes(MODE);
+  constexpr int PK = packed_sums(K, APOD, COMP, FULL, MODE);
   extern __shared__ __align__(128) unsigned char smem[];
   const uint32_t sbase = (uint32_t)__cvta_generic_to_shared(smem);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -368,11 +433,7 @@ __global__ void __launch_bounds__(256, 2) k_bf_pipe(const __grid_constant__ BfPa
              ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)((warp >> 2) * NA * 16);
     }
     constexpr bool LAZY = APOD;
-    // One register set of table entries where registers are short.  Measured
-    // (fused kernel with its preparation pass, two sets -> one): apodised
-    // k = 4 batch 2.229 -> 2.052 ms, k = 5 0.1945 -> 0.1907 ms, but plain
-    // k = 3 0.555 -> 0.581 ms.
-    constexpr bool kRing = APOD || K == 5;
+    constexpr bool kRing = one_entry_set(K, APOD, COMP, MODE);
     // Lanes -> (warp slot, depth row), as in the one-frame kernel; a 128-bit
     // shared load is served 8 lanes at a time, so with 8-row groups those are
     // 4 rows of 2 neighbouring slots, whose delays span fewer slots.
@@ -506,7 +567,7 @@ __global__ void __launch_bounds__(256, 2) k_bf_pipe(const __grid_constant__ BfPa
             load_step(e2, w2, u + tt + 2);
 #pragma unroll
             for (int c = 0; c < kC; ++c)
-              slot_pair<K, MODE, APOD, !FULL>(acc[0][c], acc[1][c], checked(cb[tt + c] + ea[c].x * (SB / 8)),
+              slot_pair<K, MODE, APOD, PK>(acc[0][c], acc[1][c], checked(cb[tt + c] + ea[c].x * (SB / 8)),
                                        __int_as_float(ea[c].y), APOD ? wa[c] : 0.f);
 #pragma unroll
             for (int c = 0; c < kC; ++c) {
@@ -550,7 +611,7 @@ __global__ void __launch_bounds__(256, 2) k_bf_pipe(const __grid_constant__ BfPa
             const int off = ee[tt].x * (SB / 8);
 #pragma unroll
             for (int c = 0; c < kC; ++c)
-              slot_pair<K, MODE, APOD, !FULL>(acc[0][c], acc[1][c], checked(cb[tt + c] + off),
+              slot_pair<K, MODE, APOD, PK>(acc[0][c], acc[1][c], checked(cb[tt + c] + off),
                                        __int_as_float(ee[tt].y), APOD ? ww[tt] : 0.f);
           }
           kahan();
@@ -574,7 +635,7 @@ __global__ void __launch_bounds__(256, 2) k_bf_pipe(const __grid_constant__ BfPa
               if ((tt & 1) && more) load_half(ea, wa, tt >> 1);
 #pragma unroll
               for (int c = 0; c < kC; ++c)
-                slot_pair<K, MODE, APOD, !FULL>(acc[0][c], acc[1][c], checked(cb[tt + c] + off), a, weight);
+                slot_pair<K, MODE, APOD, PK>(acc[0][c], acc[1][c], checked(cb[tt + c] + off), a, weight);
             }
             tblock -= tstep;
             kahan();
