@@ -4,8 +4,8 @@
 //
 // All frames of a launch share the delays.  A thread works on the same 4
 // pixels of two frames: one table entry, one slot address and one 128-bit
-// shared load serve a pair of each frame, and multiplies of the two run as one
-// packed instruction.  Per pair that leaves 13 of the one-frame form's 18
+// shared load serve a pair of each frame, and products and sums of the two run as
+// packed instructions.  Per pair that leaves 11.3 of the one-frame form's 18
 // instruction slots (k = 3, counted by ncu).
 //
 // Staging is gone from the arithmetic warps: the slots of a channel window are
@@ -19,10 +19,11 @@
 //
 // Bounds, in slots of 1/128 SM clock per pair at k = 3 (measured rates per SM
 // and clock: 128 issue, ex2 32, lg2 / rsqrt / sqrt 16 threads): MUFU 12, issue
-// 13, shared loads 8 (16 B a pair-of-frames, conflict-free) + table 2.  A loop
-// of these roots with as many other instructions takes about the issue count
-// plus 3 by itself; 16 warps a SM (128 registers: 40 sums) reach 18.
-// Measured against the one-frame form on GB300 (whole calls, with the
+// 11.3, shared loads 8 (16 B a pair-of-frames, conflict-free) + table 2.  A loop
+// of these roots with 13 instructions a pair takes about 16 by itself; 16 warps a
+// SM (128 registers: 40 sums) reach 19 (59 % issue active).
+// Measured against the one-frame form on GB300, before the sums were packed
+// (packed_sums; whole calls, with the slot
 // preparation pass; see pick_form for where the line lies): 32 frames of
 // 512 x 512, k = 3 730 -> 679 us; nearest k = 2 203 -> 176; 4 frames of 1024 x
 // 1024 BF16 + Kahan 677 -> 644; full table 399 -> 290; 5 frames of 1501 samples
