@@ -224,14 +224,7 @@ __global__ void __launch_bounds__(512, 2) k_bf_fine(const __grid_constant__ BfPa
         }
       }
     }
-    __syncwarp();
-    int before = 0;
-    if (lane == 0) before = count_arrival(sbase + kPipeCountOff + 4 * stage);
-    if (__shfl_sync(0xffffffffu, before, 0) == nwarps - 1) {
-      if (lane == 0) reinterpret_cast<int*>(smem + kPipeCountOff)[stage] = 0;
-      produce<FULL, 8, 1>(p, smem, sbase, stage, lane);
-      __syncwarp();
-    }
+    leave_chunk<FULL, 8, 1>(p, smem, sbase, stage, lane, nwarps);
     if (++stage == p.stages) {
       stage = 0;
       phase ^= 1;

@@ -390,6 +390,23 @@ __device__ __forceinline__ void produce(const BfParams& p, unsigned char* smem, 
   }
 }
 
+// Counts the warp out of the stage's chunk; the last warp out loads the chunk
+// after next into it.  The arrival count's acquire is lane 0's: a shuffle orders
+// no memory, so the warp synchronises before every lane of it reads the running
+// item, which another warp wrote.
+template <bool FULL, int SB, int NF>
+__device__ __forceinline__ void leave_chunk(const BfParams& p, unsigned char* smem, uint32_t sbase,
+                                            int stage, int lane, int nwarps) {
+  __syncwarp();
+  int before = 0;
+  if (lane == 0) before = count_arrival(sbase + kPipeCountOff + 4 * stage);
+  if (__shfl_sync(0xffffffffu, before, 0) != nwarps - 1) return;
+  if (lane == 0) reinterpret_cast<int*>(smem + kPipeCountOff)[stage] = 0;
+  __syncwarp();
+  produce<FULL, SB, NF>(p, smem, sbase, stage, lane);
+  __syncwarp();
+}
+
 template <int K, bool APOD, bool COMP, bool FULL, int MODE>
 __global__ void __launch_bounds__(256, pipe_blocks(K, APOD, COMP)) k_bf_pipe(const __grid_constant__ BfParams p) {
   constexpr int NA = NAcc<K>::value, SB = slot_bytes(MODE);
@@ -658,14 +675,7 @@ __global__ void __launch_bounds__(256, pipe_blocks(K, APOD, COMP)) k_bf_pipe(con
         }
         }
       }
-      __syncwarp();
-      int before = 0;
-      if (lane == 0) before = count_arrival(sbase + kPipeCountOff + 4 * stage);
-      if (__shfl_sync(0xffffffffu, before, 0) == nwarps - 1) {
-        if (lane == 0) reinterpret_cast<int*>(smem + kPipeCountOff)[stage] = 0;
-        produce<FULL, SB, 2>(p, smem, sbase, stage, lane);
-        __syncwarp();
-      }
+      leave_chunk<FULL, SB, 2>(p, smem, sbase, stage, lane, nwarps);
       if (++stage == p.stages) {
         stage = 0;
         phase ^= 1;
