@@ -42,7 +42,8 @@ def _sources():
 
 
 def _deps():
-    return _sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(INCLUDE, "*.h"))
+    headers = [os.path.join(d, p) for d, p in ((CSRC, "*.cuh"), (CSRC, "*.h"), (INCLUDE, "*.h"))]
+    return _sources() + [h for p in headers for h in glob.glob(p)]
 
 
 def _stale(target: str) -> bool:

@@ -43,6 +43,7 @@
 #include <vector>
 
 #include "pa_internal.cuh"
+#include "pa_regions.h"
 
 namespace {
 
@@ -73,12 +74,14 @@ struct ColRange {
   __device__ __forceinline__ int behind() const { return hhi > hlo ? max(0, hi - behind_at()) : 0; }
 };
 
-// Regions passed with the launch (32 x 64 B of its 4 KB of parameters), so
+// Regions passed with the launch (32 x 80 B of its 4 KB of parameters), so
 // that the usual call needs no upload.
 constexpr int kParamRegions = 32;
 struct RegTable {
   MRegion r[kParamRegions];
 };
+static_assert(sizeof(RegTable) == kParamRegions * 80 && sizeof(RegTable) < 3500,
+              "launch parameters");
 
 struct MGeom {
   int nx, nz, n_roi, chunks;
@@ -252,6 +255,7 @@ __global__ void __launch_bounds__(512) k_m_members(MGeom g, const __grid_constan
   const MRegion R = tab_n > 0 ? tab.r[blockIdx.x] : regs[blockIdx.x];
   const int width = R.j1 - R.j0, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int sides = R.shape == PA_REGION_ANNULUS ? 2 : 1;
+  const int room = (int)(R.pix1 - R.pix0);
   for (int i = threadIdx.x; i < sides * width; i += blockDim.x) {
     const int hole = i >= width, c = i - (hole ? width : 0);
     iv[hole][c] = column_interval(R, hole, R.j0 + c, g);
@@ -279,7 +283,7 @@ __global__ void __launch_bounds__(512) k_m_members(MGeom g, const __grid_constan
       run += __shfl_sync(0xffffffffu, inc, 31);
     }
     if (lane == 0) {
-      counts[blockIdx.x] = run;
+      counts[blockIdx.x] = min(run, room);  // entries that the list holds, never more
       pix0[blockIdx.x] = R.pix0;
     }
   }
@@ -287,7 +291,7 @@ __global__ void __launch_bounds__(512) k_m_members(MGeom g, const __grid_constan
   for (int c = w; c < width; c += (int)(blockDim.x >> 5)) {
     const ColRange r = range(c);
     const int n1 = r.before(), skip = r.behind_at() - n1;
-    const int n = min(n1 + r.behind(), (int)(R.pix1 - R.pix0) - off[c]);  // (never cut)
+    const int n = min(n1 + r.behind(), room - off[c]);  // (most_members: never cut)
     const unsigned int q = (unsigned)(R.j0 + c) * (unsigned)g.nz;
     unsigned int* const dst = list + R.pix0 + off[c];
     for (int t = lane; t < n; t += 32) dst[t] = q + (unsigned)(t + (t < n1 ? r.lo : skip));
@@ -758,21 +762,6 @@ void index_range(double c, double h, double o, double d, int n, int* lo, int* hi
   *hi = std::max(*lo, (int)u);
 }
 
-// At least the members of a region: its bounding box, or for round regions
-// that lie within the image their area (in pixels) and half a boundary pixel
-// at each end of every column: with f the chord over a column, unimodal, the
-// sum of f over the columns differs from its integral by its maximum at most,
-// and the rows in a chord from its length by one.
-long long most_members(const MRegion& o, const MGeom& g) {
-  const long long box = (long long)(o.j1 - o.j0) * (o.l1 - o.l0);
-  if (o.shape == PA_REGION_RECT || o.j0 <= 0 || o.l0 <= 0 || o.j1 >= g.nx || o.l1 >= g.nz) return box;
-  const bool hole = o.shape == PA_REGION_ANNULUS;
-  const double out = hole ? o.b : o.a, in = hole ? std::min(o.a, o.b) : 0.0;
-  const double n = 3.1416 * out * out / (g.dx * g.dz) - 3.1415 * in * in / (g.dx * g.dz) +
-                   2.0 * (out + in) / g.dz + 2.0 * (o.j1 - o.j0) + 16.0;
-  return n < (double)box ? (long long)n : box;
-}
-
 }  // namespace
 
 extern "C" pa_status pa_image_metrics(const pa_grid* grid, const float* images_dev,
@@ -827,7 +816,9 @@ extern "C" pa_status pa_image_metrics(const pa_grid* grid, const float* images_d
       index_range(in.zc_m, hz, g.z0, g.dz, g.nz, &o.l0, &o.l1);
       o.col0 = n_cols;
       n_cols += o.j1 - o.j0;
-      const long long most = most_members(o, g);
+      const bool inside = o.j0 > 0 && o.l0 > 0 && o.j1 < g.nx && o.l1 < g.nz;
+      const long long most =
+          pa::most_members(o.shape, o.a, o.b, o.j1 - o.j0, o.l1 - o.l0, inside, g.dx, g.dz);
       o.pix0 = n_pix;
       n_pix += most;
       o.pix1 = n_pix;
