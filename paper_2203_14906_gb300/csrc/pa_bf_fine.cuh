@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(512, 2) k_bf_fine(const __grid_constant__ BfPa
       const int j = jt + p.m * (cp * PX + c);
       if (j < p.nx && z < p.nz) {
         float das, dmas, ho;
-        combine<K>(acc[c], das, dmas, ho);
+        combine<K>(acc[c], p.ek_top, das, dmas, ho);
         const size_t px = fbase + (size_t)j * p.nz + z;
         if (p.plane_das >= 0) p.out[px + (size_t)p.plane_das * plane] = das;
         if (p.plane_dmas >= 0) p.out[px + (size_t)p.plane_dmas * plane] = dmas;

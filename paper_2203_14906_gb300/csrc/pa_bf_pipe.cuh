@@ -697,7 +697,7 @@ __global__ void __launch_bounds__(256, pipe_blocks(K, APOD, COMP)) k_bf_pipe(con
           const int j = jt + p.m * c;
           if (j < p.nx && z < p.nz) {
             float das, dmas, ho;
-            combine<K>(acc[h][c], das, dmas, ho);
+            combine<K>(acc[h][c], p.ek_top, das, dmas, ho);
             const size_t px = fbase + (size_t)j * p.nz + z;
             if (p.plane_das >= 0) p.out[px + (size_t)p.plane_das * plane] = das;
             if (p.plane_dmas >= 0) p.out[px + (size_t)p.plane_dmas * plane] = dmas;

@@ -171,6 +171,7 @@ struct BfParams {  // aligned as CUtensorMap requires
   int planes;             // planes per frame (n_stages * n_outputs)
   int plane_das, plane_dmas, plane_ho;  // raw plane of each output or -1
   int nx, nz;
+  float ek_top;           // amplitude sums from here on take the FP64 e_k (df_in_range)
   int n_frames;           // frames in this launch
   int n_items;            // n_tiles * ngroups * n_frames (two-frame kernel: * n_fgroups)
   // two-frame kernel

@@ -72,7 +72,7 @@ __global__ void __launch_bounds__(256) k_lanes(const __grid_constant__ BfParams 
       for (int q = 0; q < NA; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], off);
     if (g == 0 && j < p.nx && z < p.nz) {
       float das, dmas, ho;
-      combine<3>(acc, das, dmas, ho);
+      combine<3>(acc, p.ek_top, das, dmas, ho);
       const size_t px = fbase + (size_t)j * p.nz + z;
       if (p.plane_das >= 0) p.out[px + (size_t)p.plane_das * plane] = das;
       if (p.plane_dmas >= 0) p.out[px + (size_t)p.plane_dmas * plane] = dmas;

@@ -1515,6 +1515,11 @@ const FusedForm& pick_form(const pa_plan_s* P, int nf) {
   return pays ? two : one;
 }
 
+// Amplitude sums below this take the two-float e_k (df_in_range says why).
+float ek_top(int k, int n_elem) {
+  return (float)std::min(std::ldexp(1.0, 40), std::ldexp(1.0, 120) / std::pow((double)n_elem, k - 1));
+}
+
 // Launch parameters of one round of the fused kernel in form f: nf frames
 // from frame f0 of the chunk on.
 pa_status fused_params(pa_plan_s* P, const FusedForm& f, const void* rf, int nf, float* out,
@@ -1578,6 +1583,7 @@ pa_status fused_params(pa_plan_s* P, const FusedForm& f, const void* rf, int nf,
   b.plane_ho = P->out_id[2] >= 0 ? s_raw * P->n_out + P->out_id[2] : -1;
   b.nx = d.nx;
   b.nz = d.nz;
+  b.ek_top = ek_top(P->K, d.n_elem);
   b.n_frames = nf;
   b.n_fgroups = (nf + f.nf - 1) / f.nf;
   b.splits = f.splits;
