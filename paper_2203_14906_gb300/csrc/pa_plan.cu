@@ -312,8 +312,8 @@ __device__ double pixel_z(const TableGeom& g, int z) { return g.z0 + ((double)z 
 // Lattice table: every lattice offset d = j - m i and depth row, entry
 // {n0 * 8 (the byte stride of an interpolation slot), FP32 bits of a}.
 __global__ void k_table(TableGeom g, int2* table, float* wtab) {
-  const int z = blockIdx.x * blockDim.x + threadIdx.x;
-  const int row = blockIdx.y;
+  const int z = blockIdx.y * blockDim.x + threadIdx.x;
+  const int row = blockIdx.x;  // (x: a wide aperture has more than 65535 rows)
   if (z >= g.nzp || row >= g.ndrows) return;
   const double dxv = g.x_const + ((double)(g.dmin + row) + 0.5) * g.dx;
   const double zp = pixel_z(g, z);
@@ -1284,7 +1284,7 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
     k_table_full<<<gt, 256, 0, st>>>(tg, fg, P->lo, P->ftab, P->wtab);
     PA_CUDA(cudaGetLastError());
   } else {
-    dim3 gt((P->nz_pad + 127) / 128, P->ndrows);
+    dim3 gt(P->ndrows, (P->nz_pad + 127) / 128);
     k_table<<<gt, 128, 0, st>>>(tg, P->table, P->wtab);
     PA_CUDA(cudaGetLastError());
     dim3 gw((P->nv + 127) / 128, P->n_tiles);
