@@ -831,6 +831,7 @@ size_t slots_size(const pa_plan_s* P, int form, int* frames) {
   const size_t sb = form == 1 ? pipe_slot_bytes(P->slot_mode) : sizeof(float2);
   const size_t row = (size_t)P->slot_pitch * sb;
   const size_t per_item = (size_t)P->d.n_elem * row;
+  if (per_item > kSlotBytesMax) return 0;  // (one item alone would pass the bound)
   size_t items = ((size_t)P->d.max_batch + item - 1) / item;
   if (form > 1)
     items = std::min<size_t>(items, std::max<int64_t>(1, std::max(lim.px1, lim.px2) / frame_warps(P)));
@@ -1101,7 +1102,9 @@ pa_status build_form1(pa_plan_s* P) {
 
 // The two-frame form; a plan it does not fit keeps the one-frame form alone.
 pa_status build_form2(pa_plan_s* P) {
-  if (!wants_pairs(P)) return PA_OK;
+  int frames = 0;
+  slots_size(P, 1, &frames);
+  if (!wants_pairs(P) || frames == 0) return PA_OK;
   FusedForm f;
   f.nf = 2;
   f.slot_bytes = pipe_slot_bytes(P->slot_mode);
@@ -1162,6 +1165,9 @@ pa_status build_form3(pa_plan_s* P, int px) {
   const FineLimits lim = fine_limits(P);
   if (frame_warps(P) > (px == 1 ? lim.px1 : lim.px2) || P->window > P->slot_margin) return PA_OK;
   if (fine_steps(P) < (px == 1 ? kFineSteps1 : kFineSteps2)) return PA_OK;
+  int frames = 0;
+  slots_size(P, 2, &frames);
+  if (frames == 0) return PA_OK;
   FusedForm f;
   f.nf = 1;
   f.slot_bytes = sizeof(float2);
