@@ -191,7 +191,8 @@ typedef struct {
  * caps the channel steps per staged chunk, PA_LANE_ROWS=32|16|8 sets the
  * depth rows per lane group of the fused kernel, PA_ITEM_FRAMES the form of
  * the fused kernel (1: one frame per work item, 2: two where the launch and the
- * order allow it, 3: one pixel per thread where the launch allows it).  In the
+ * order allow it, 3 and 4: one and two pixels per thread where the launch
+ * allows it; pa_plan_form says which form a launch runs).  In the
  * checked build only
  * (device bounds checks, PA_CHECK_BOUNDS), PA_INJECT_TMA_SHORTFALL makes
  * every TMA chunk expect 16 bytes more than it receives, so each block's
@@ -208,6 +209,11 @@ pa_status pa_plan_footprint(const pa_plan_desc* desc, int32_t n_frames,
                             size_t* bytes);
 
 pa_status pa_plan_get_info(pa_plan_t plan, pa_plan_info* info);
+
+/* The form of the fused kernel that a launch of n_frames frames (1..max_batch)
+ * runs, for tests and measurements: 1 one frame per work item, 2 two, 3 and 4
+ * one and two pixels per thread.  PA_EINVAL (null argument, n_frames). */
+pa_status pa_plan_form(pa_plan_t plan, int32_t n_frames, int32_t* form);
 
 /*
  * pa_beamform -- the hot path (Sections 2-3 and 5) on n_frames frames that

@@ -32,6 +32,7 @@ EXPORTS = (
     "pa_plan",
     "pa_plan_footprint",
     "pa_plan_get_info",
+    "pa_plan_form",
     "pa_beamform",
     "pa_beamform_host",
     "pa_plan_use_graph",
@@ -215,6 +216,8 @@ def load(checked: bool = False, build: bool = True):
         L.pa_plan_footprint.restype = ctypes.c_int
         L.pa_plan_get_info.argtypes = [vp, ctypes.POINTER(PlanInfo)]
         L.pa_plan_get_info.restype = ctypes.c_int
+        L.pa_plan_form.argtypes = [vp, i32, ctypes.POINTER(i32)]
+        L.pa_plan_form.restype = ctypes.c_int
         L.pa_beamform.argtypes = [vp, vp, i32, vp, u32, vp]
         L.pa_beamform.restype = ctypes.c_int
         L.pa_beamform_host.argtypes = [vp, vp, i32, vp, u32, vp]
@@ -318,6 +321,13 @@ class Plan:
         inf = PlanInfo()
         check(self._L, self._L.pa_plan_get_info(self._h, ctypes.byref(inf)))
         return inf.as_dict()
+
+    def form(self, n_frames: int) -> int:
+        """Form of the fused kernel that a launch of ``n_frames`` frames runs
+        (1 one frame per work item, 2 two, 3 / 4 one / two pixels per thread)."""
+        f = ctypes.c_int32()
+        check(self._L, self._L.pa_plan_form(self._h, int(n_frames), ctypes.byref(f)))
+        return f.value
 
     def out_shape(self, n_frames, stages):
         n_st = bin(int(stages) & 7).count("1")

@@ -106,7 +106,7 @@ struct pa_plan_s {
   long long timeouts_seen = 0;  // timed-out waits already reported by pa_beamform_host
   int* host_flag = nullptr;  // pinned word a timed-out wait sets (host path)
   int wr = 0;         // raw samples per channel delivered by one TMA box
-  int item_frames = 0;  // PA_ITEM_FRAMES: 1 or 2 picks the form (measurements, tests)
+  int item_frames = 0;  // PA_ITEM_FRAMES: 1-4 picks the form (measurements, tests)
   double steps_per_pixel = 0;  // channel steps evaluated per pixel, mean
   bool pairs_pay = false;  // resident warps and slot reuse of the two-frame form suffice
   // post
@@ -794,7 +794,7 @@ cudaError_t fused_blocks_per_sm(const pa_plan_s* P, const FusedForm& f, size_t s
 
 // Whether a plan of this descriptor gets the two-frame form (if it fits).
 bool wants_pairs(const pa_plan_s* P) {
-  return P->d.max_batch > 1 && P->K <= 5 && P->item_frames != 1 && P->item_frames != 3;
+  return P->d.max_batch > 1 && P->K <= 5 && (P->item_frames == 0 || P->item_frames == 2);
 }
 
 // The one-frame form stages this plan's RF windows sample by sample (rows off
@@ -809,13 +809,14 @@ struct FineLimits {
   int px1, px2;
 };
 FineLimits fine_limits(const pa_plan_s* P) {
-  if (P->item_frames == 3) return {1 << 20, 1 << 20};  // tests
+  if (P->item_frames == 3) return {1 << 20, 0};  // tests
+  if (P->item_frames == 4) return {0, 1 << 20};
   if (P->item_frames != 0) return {0, 0};
   return P->comp || P->full || staged_by_samples(P) ? FineLimits{1100, 2400} : FineLimits{600, 0};
 }
 // Least mean channel steps per pixel of those forms.
 constexpr double kFineSteps1 = 28, kFineSteps2 = 50;
-double fine_steps(const pa_plan_s* P) { return P->item_frames == 3 ? 1e9 : P->steps_per_pixel; }
+double fine_steps(const pa_plan_s* P) { return P->item_frames >= 3 ? 1e9 : P->steps_per_pixel; }
 // Warps of 4-pixel threads of one frame.
 int64_t frame_warps(const pa_plan_s* P) { return (int64_t)P->n_tiles * P->slots; }
 
@@ -2263,6 +2264,14 @@ pa_status pa_plan_get_info(pa_plan_t P, pa_plan_info* info) {
       info->device_error_flags |= (uint32_t)flag;
     }
   }
+  return PA_OK;
+}
+
+pa_status pa_plan_form(pa_plan_t P, int32_t n_frames, int32_t* form) {
+  if (!P || !form) return fail(PA_EINVAL, "null argument");
+  if (n_frames < 1 || n_frames > P->d.max_batch)
+    return fail(PA_EINVAL, "a launch of %d frames is outside 1..max_batch (%d)", n_frames, P->d.max_batch);
+  *form = 1 + (int32_t)(&pick_form(P, n_frames) - P->form);
   return PA_OK;
 }
 
