@@ -801,10 +801,9 @@ bool wants_pairs(const pa_plan_s* P) {
 // 16-byte boundaries).
 bool staged_by_samples(const pa_plan_s* P) { return !P->use_tma && P->d.n_samples % 4 != 0; }
 
-// Largest launch, in warps of 4-pixel threads, of the fine-grained forms
-// (pick_form says where the lines lie): one pixel a thread, and two.  They
-// reach further where the one-frame form is slow for its size: compensated
-// sums, the full table, records staged sample by sample.
+// Largest launch, in warps of 4-pixel threads, for which the fine-grained forms
+// (one pixel a thread, and two) are built; pick_form says which of these
+// launches run them.
 struct FineLimits {
   int px1, px2;
 };
@@ -812,11 +811,19 @@ FineLimits fine_limits(const pa_plan_s* P) {
   if (P->item_frames == 3) return {1 << 20, 0};  // tests
   if (P->item_frames == 4) return {0, 1 << 20};
   if (P->item_frames != 0) return {0, 0};
+  const bool loads = !P->full && !P->use_tma && !staged_by_samples(P);
+  if (!P->full && P->use_tma && !P->comp) return {0, 0};
+  if (loads && !P->comp && (P->K < 3 || P->K > 5)) return {0, 0};
   return P->comp || P->full || staged_by_samples(P) ? FineLimits{1100, 2400} : FineLimits{600, 0};
 }
-// Least mean channel steps per pixel of those forms.
-constexpr double kFineSteps1 = 28, kFineSteps2 = 50;
+// Least mean channel steps per pixel of those forms: fewer do not repay the
+// preparation pass (0.84-1.0), nor fewer than 48 at orders up to 3 where the
+// one-frame form reads whole rows by vector loads (0.91-1.0).
 double fine_steps(const pa_plan_s* P) { return P->item_frames >= 3 ? 1e9 : P->steps_per_pixel; }
+double least_fine_steps(const pa_plan_s* P, int px) {
+  if (px == 2) return !P->full && P->use_tma ? 110 : 50;
+  return !P->full && !P->use_tma && !staged_by_samples(P) && P->K <= 3 ? 48 : 28;
+}
 // Warps of 4-pixel threads of one frame.
 int64_t frame_warps(const pa_plan_s* P) { return (int64_t)P->n_tiles * P->slots; }
 
@@ -1165,7 +1172,7 @@ pa_status build_form2(pa_plan_s* P) {
 pa_status build_form3(pa_plan_s* P, int px) {
   const FineLimits lim = fine_limits(P);
   if (frame_warps(P) > (px == 1 ? lim.px1 : lim.px2) || P->window > P->slot_margin) return PA_OK;
-  if (fine_steps(P) < (px == 1 ? kFineSteps1 : kFineSteps2)) return PA_OK;
+  if (fine_steps(P) < least_fine_steps(P, px)) return PA_OK;
   int frames = 0;
   slots_size(P, 2, &frames);
   if (frames == 0) return PA_OK;
@@ -1489,37 +1496,72 @@ bool encode_rf_map(pa_plan_s* P, const void* rf, int nf, CUtensorMap* map) {
                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The form a launch of nf frames runs.  Measured over 120 plans of 24-256
-// elements, 48-1024 depth rows and 2-57 frames (whole calls, one-frame form
-// time / two-frame form time):
-//   * two frames an item halve the items, so the launch has to fill the GPU
-//     all the same: below 0.65 resident blocks' worth of one-frame items
-//     0.72-0.95, above it 0.98-1.4;
-//   * an odd launch's last item does a frame's work twice: 3 and 5 frames
-//     0.85-0.99, 7 and more 1.04-1.3;
-//   * records whose rows are not 16-byte aligned (4 samples) are staged
-//     sample by sample in the one-frame form but prepared all the same in the
-//     other: 1.3-1.8 down to half as many items, odd launches included.
-// Small launches (110 plans, 1-6 frames) leave most of the GPU idle with
-// 4-pixel threads: at one pixel a thread 1.0-2.0 up to 600 warps of 4-pixel
-// threads (1100 for the plans fine_limits names), where the launch fills the
-// GPU on its own; two pixels a thread 1.04-1.55 from there to 2400 for the
-// same plans (plain FP32 0.84-1.0).  Pixels of fewer than 28 channel steps
-// (50 from 1100 warps on) do not repay the preparation pass (0.84-1.0).
-const FusedForm& pick_form(const pa_plan_s* P, int nf) {
-  const FusedForm &one = P->form[0], &two = P->form[1];
+// The form a launch of nf frames runs.  The lines follow 4500 random plans (24-256
+// elements, 48-1024 depth rows, 1-48 frames, every option), each form timed
+// warm and with the record and tables out of L2; the figures are means of
+// one-frame form time / this form's time.  What decides is how many work items
+// of the one-frame form an SM gets (`per_sm`; a block is an item, so few items
+// leave SMs idle or one SM with twice another's work), and how the one-frame
+// form stages its record: by TMA (16-bit rows on 16-byte boundaries), by vector
+// loads, or, rows off 16-byte boundaries, sample by sample.
+//
+// One pixel a thread (up to 1100 warps of 4-pixel threads; 600 for plain sums
+// off vector loads, 0.8 beyond):
+//   full table 1.25-1.5 up to two items an SM, with Kahan sums at any number;
+//   lattice, TMA: plain sums 0.75-0.95, never; Kahan sums 1.1-1.3 between one
+//     item an SM and two, 0.87-0.97 on either side;
+//   lattice, by samples: Kahan sums 1.0-1.5; plain sums 1.1-1.25 up to one item
+//     an SM, with 50 steps and more 1.05 up to 1.5, 0.8-0.9 beyond;
+//   lattice, vector loads: Kahan sums 1.0-1.45; plain sums of orders 3-5
+//     1.03-1.13 up to half an item an SM, with 50 steps and more 1.03 up to one,
+//     0.75-0.98 beyond; other orders 0.87-1.02.
+// Two pixels a thread (Kahan sums, full table, records by samples; up to 2400
+// warps), from two items an SM on (0.6-0.95 below):
+//   full table 1.1-1.45, with Kahan sums up to four items an SM (0.85-1.05
+//     beyond); lattice with Kahan sums 1.1-1.3 up to four (TMA: from 110 steps
+//     on), 0.8-0.95 beyond; plain sums by samples 1.06-1.4 above four, or above
+//     three with 110 steps.
+// Two frames an item (orders up to 5):
+//   Kahan sums: from 0.65 of the resident blocks on 1.05-1.5 (0.3 where the
+//     record is staged by samples: 1.2-1.6); plain sums need pairs of items
+//     enough as well, two an SM, 2.5 at orders up to 2: 1.06-1.4, and 0.7-0.97
+//     below that (0.6 of the resident blocks by samples);
+//   an odd launch's last item does a frame's work twice: 3 and 5 frames 0.85-1.0
+//     but where the record is staged by samples; from 7 on 1.04-1.3;
+//   and the samples of a row have to serve pairs enough (pairs_pay).
+bool fine_pays(const pa_plan_s* P, int px, int nf) {
   const FineLimits lim = fine_limits(P);
-  const int64_t warps = frame_warps(P) * nf;
+  if (frame_warps(P) * nf > (px == 1 ? lim.px1 : lim.px2)) return false;
+  if (P->item_frames != 0) return true;
+  const double per_sm = (double)P->n_tiles * P->ngroups * nf / P->num_sms, steps = fine_steps(P);
+  if (px == 1) {
+    if (P->full) return P->comp || per_sm <= 2;
+    if (P->use_tma) return P->comp && per_sm > 1 && per_sm <= 2;
+    if (P->comp) return true;
+    if (staged_by_samples(P)) return per_sm <= 1 || (per_sm <= 1.5 && steps >= 50);
+    return per_sm <= 0.5 || (per_sm <= 1 && steps >= 50);
+  }
+  if (per_sm <= 2) return false;
+  if (P->comp) return per_sm <= 4;
+  return P->full || per_sm > 4 || (per_sm > 3 && steps >= 110);
+}
+
+bool pairs_pay(const pa_plan_s* P, int nf) {
+  const double items = (double)P->n_tiles * P->ngroups;
+  const double fill = items * nf / ((double)P->form[0].blocks_per_sm * P->num_sms);
+  const bool enough = P->comp || items * ((nf + 1) / 2) >= (P->K <= 2 ? 2.5 : 2.0) * P->num_sms;
+  if (staged_by_samples(P)) return enough && fill >= (P->comp ? 0.3 : 0.6);
+  return enough && fill >= 0.65 && (nf % 2 == 0 || nf >= 7) && P->pairs_pay;
+}
+
+const FusedForm& pick_form(const pa_plan_s* P, int nf) {
   for (int px = 1; px <= 2; ++px) {
     const FusedForm& f = P->form[px + 1];
-    if (f.nf && nf <= f.max_frames && warps <= (px == 1 ? lim.px1 : lim.px2)) return f;
+    if (f.nf && nf <= f.max_frames && fine_pays(P, px, nf)) return f;
   }
-  if (two.nf == 0 || nf < 2) return one;
-  if (P->item_frames == 2) return two;
-  const double fill = (double)P->n_tiles * P->ngroups * nf / ((double)one.blocks_per_sm * P->num_sms);
-  const bool pays = staged_by_samples(P) ? fill >= 0.3
-                           : fill >= 0.65 && (nf % 2 == 0 || nf >= 7) && P->pairs_pay;
-  return pays ? two : one;
+  const FusedForm& two = P->form[1];
+  if (two.nf && nf >= 2 && (P->item_frames == 2 || pairs_pay(P, nf))) return two;
+  return P->form[0];
 }
 
 // Amplitude sums below this take the two-float e_k (df_in_range says why).
