@@ -146,9 +146,13 @@ __host__ __device__ constexpr int packed_sums(int k, bool apod, bool comp, bool 
 // registers: 168), but for Kahan sums over the full aperture: their folds leave
 // room for one set of table entries only there, which takes 222 us instead of 230
 // in a full launch, but 33.0 instead of 31.9 in one of 200 blocks (six BF16 frames
-// of 256 x 256) and 289 instead of 285 with wide windows.
-__host__ __device__ constexpr int pipe_blocks(int k, bool apod, bool comp) {
-  return k <= 2 && (apod || !comp) ? 3 : 2;
+// of 256 x 256) and 289 instead of 285 with wide windows.  With the full table 80
+// registers spill (entries and weights of three steps at once: up to 134 bytes) and
+// fewer loads are in flight; over 500 plans of 2-48 frames 24 warps take 1.17-1.20
+// of the time of 16 (apodised 1.26-1.37, with Kahan sums 1.16-1.26; nearest samples
+// 1.0-1.24).
+constexpr int pipe_blocks(int k, bool apod, bool comp, bool full) {
+  return k <= 2 && (apod || !comp) && !full ? 3 : 2;
 }
 // Sets of table entries: with one the next block's entries replace those just
 // used, with two they are loaded a block ahead.  Two where registers last for
@@ -408,7 +412,7 @@ __device__ __forceinline__ void leave_chunk(const BfParams& p, unsigned char* sm
 }
 
 template <int K, bool APOD, bool COMP, bool FULL, int MODE>
-__global__ void __launch_bounds__(256, pipe_blocks(K, APOD, COMP)) k_bf_pipe(const __grid_constant__ BfParams p) {
+__global__ void __launch_bounds__(256, pipe_blocks(K, APOD, COMP, FULL)) k_bf_pipe(const __grid_constant__ BfParams p) {
   constexpr int NA = NAcc<K>::value, SB = slot_bytes(MODE);
   constexpr int PK = packed_sums(K, APOD, COMP, FULL, MODE);
   extern __shared__ __align__(128) unsigned char smem[];
