@@ -12,8 +12,12 @@
 // four.  Chunks come as in the two-frame form, by bulk copies from slots
 // prepared for the launch ({r, d} per sample; the pass takes the place of the
 // clearing kernel) into two buffers; a tile's channel windows are copied once
-// per block of up to 16 warps.  Kahan totals stay in registers (a pixel's 2 x 5
-// at k = 3).
+// per block of up to 16 warps.  Kahan totals are kept beside the sums (a pixel's
+// 2 x 5 at k = 3), in registers as far as the 64 of two blocks a SM go: one pixel
+// a thread spills 6-36 bytes at k = 3 and 250 at k = 8, two pixels 112 to 500,
+// outside the channel loop's inner steps (the totals are touched every 64).  Over
+// 900 plans these variants still take 0.78-0.92 of the one-frame form's time where
+// pick_form sends them.
 // Measured on GB300 (RAW images, one-frame form -> this): one frame of 128 x 128,
 // 64 channels, k = 3 18.9 -> 14.8 us; one and two frames of 256 x 256, 64
 // channels, k = 2 BF16 + Kahan 16.7 -> 14.8 and 27.4 -> 18.9; one frame of 400 x

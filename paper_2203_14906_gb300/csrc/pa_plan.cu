@@ -1507,7 +1507,8 @@ bool encode_rf_map(pa_plan_s* P, const void* rf, int nf, CUtensorMap* map) {
 //
 // One pixel a thread (up to 1100 warps of 4-pixel threads; 600 for plain sums
 // off vector loads, 0.8 beyond):
-//   full table 1.25-1.5 up to two items an SM, with Kahan sums at any number;
+//   full table 1.25-1.5 up to two items an SM, with Kahan sums at any number
+//     (1.28 at order 6, 1.09 at 7, 0.98 at 8, whose sums spill most);
 //   lattice, TMA: plain sums 0.75-0.95, never; Kahan sums 1.1-1.3 between one
 //     item an SM and two, 0.87-0.97 on either side;
 //   lattice, by samples: Kahan sums 1.0-1.5; plain sums 1.1-1.25 up to one item
@@ -1535,7 +1536,7 @@ bool fine_pays(const pa_plan_s* P, int px, int nf) {
   if (P->item_frames != 0) return true;
   const double per_sm = (double)P->n_tiles * P->ngroups * nf / P->num_sms, steps = fine_steps(P);
   if (px == 1) {
-    if (P->full) return P->comp || per_sm <= 2;
+    if (P->full) return P->comp ? P->K <= 7 : per_sm <= 2;
     if (P->use_tma) return P->comp && per_sm > 1 && per_sm <= 2;
     if (P->comp) return true;
     if (staged_by_samples(P)) return per_sm <= 1 || (per_sm <= 1.5 && steps >= 50);

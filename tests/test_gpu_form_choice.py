@@ -45,6 +45,8 @@ def _form(k, frames, n_elem, m, nz, dtype="f32", comp=0, ns=1024, f_number=0.0, 
     (ONE, 1.5, 2, dict(k=3, frames=2, n_elem=64, m=4, nz=256, ns=1022)),
     (FINE1, 1.5, 2, dict(k=3, frames=2, n_elem=64, m=4, nz=256, ns=1022, comp=1)),
     (FINE1, 1, 2, dict(k=3, frames=2, n_elem=64, m=4, nz=256, table="full")),
+    (FINE1, 1, 2, dict(k=7, frames=2, n_elem=64, m=4, nz=256, table="full", comp=1)),
+    (ONE, 1, 2, dict(k=8, frames=2, n_elem=64, m=4, nz=256, table="full", comp=1)),
     (FINE2, 2, 4, dict(k=3, frames=4, n_elem=64, m=4, nz=256, table="full")),
     (FINE2, 2, 4, dict(k=3, frames=4, n_elem=64, m=4, nz=256, comp=1)),
     (ONE, 2.5, 4, dict(k=2, frames=4, n_elem=64, m=4, nz=256)),  # two pairs of items an SM, not 2.5
