@@ -9,6 +9,7 @@
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -58,6 +59,67 @@ struct DeviceGuard {
 // Buffer sets (and streams) of the host-buffer path.
 constexpr int kHostSets = 3;
 
+// Pinned words that a timed-out wait sets, one per plan that takes the host
+// path.  The first small cudaHostAlloc of a process costs about 140 us and the
+// next 1.5 us, but the last cudaFreeHost gives the memory back, so a plan with a
+// word of its own paid 125 us in its first call and as much when it was destroyed.
+// The words come from pages of 1024 that stay with the library (4 KiB per 1024
+// plans alive at once); a page belongs to the context it was made in, as a reset
+// device takes it along.
+class HostWords {
+ public:
+  int* take() {
+    std::lock_guard<std::mutex> lk(mu_);
+    const unsigned long long ctx = context_id();
+    for (Page& pg : pages_)
+      if (pg.ctx == ctx && !pg.free.empty()) {
+        int* w = pg.free.back();
+        pg.free.pop_back();
+        return w;
+      }
+    int* base = nullptr;
+    if (cudaHostAlloc((void**)&base, kWords * sizeof(int),
+                      cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess)
+      return nullptr;
+    pages_.push_back({ctx, base, {}});
+    for (int i = kWords - 1; i > 0; --i) pages_.back().free.push_back(base + i);
+    return base;
+  }
+  void give(int* w) {
+    std::lock_guard<std::mutex> lk(mu_);
+    for (Page& pg : pages_)
+      if (w >= pg.base && w < pg.base + kWords) {
+        pg.free.push_back(w);
+        return;
+      }
+  }
+
+ private:
+  static constexpr int kWords = 1024;
+  struct Page {
+    unsigned long long ctx;
+    int* base;
+    std::vector<int*> free;
+  };
+  static unsigned long long context_id() {
+    static PFN_cuCtxGetId_v12000 fn = [] {
+      void* f = nullptr;
+      cudaDriverEntryPointQueryResult q;
+      if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &f, 12000, cudaEnableDefault, &q) !=
+              cudaSuccess ||
+          q != cudaDriverEntryPointSuccess)
+        f = nullptr;
+      return reinterpret_cast<PFN_cuCtxGetId_v12000>(f);
+    }();
+    unsigned long long id = 0;
+    if (fn) fn(nullptr, &id);
+    return id;
+  }
+  std::mutex mu_;
+  std::vector<Page> pages_;
+};
+HostWords g_host_words;
+
 // One form of the fused kernel and the shared-memory geometry that goes with
 // it: form 0 runs one frame per work item (pa_bf_kernel.cuh), form 1 two
 // frames from prepared slots (pa_bf_pipe.cuh), forms 2 and 3 one and two of a
@@ -104,7 +166,7 @@ struct pa_plan_s {
   int lo_align = 4;   // window starts are multiples of this many samples
   int expect_extra = 0;   // > 0 only under PA_INJECT_TMA_SHORTFALL (tests the bounded wait)
   long long timeouts_seen = 0;  // timed-out waits already reported by pa_beamform_host
-  int* host_flag = nullptr;  // pinned word a timed-out wait sets (host path)
+  int* host_flag = nullptr;  // pinned word a timed-out wait sets (host path; HostWords)
   int wr = 0;         // raw samples per channel delivered by one TMA box
   int item_frames = 0;  // PA_ITEM_FRAMES: 1-4 picks the form (measurements, tests)
   double steps_per_pixel = 0;  // channel steps evaluated per pixel, mean
@@ -801,6 +863,12 @@ bool wants_pairs(const pa_plan_s* P) {
 // 16-byte boundaries).
 bool staged_by_samples(const pa_plan_s* P) { return !P->use_tma && P->d.n_samples % 4 != 0; }
 
+// Whether some kernel of the plan waits for copies (and may give up): the
+// one-frame form by TMA, the others always.
+bool may_wait(const pa_plan_s* P) {
+  return P->use_tma || P->form[1].nf || P->form[2].nf || P->form[3].nf;
+}
+
 // Largest launch, in warps of 4-pixel threads, for which the fine-grained forms
 // (one pixel a thread, and two) are built; pick_form says which of these
 // launches run them.
@@ -927,7 +995,7 @@ void free_plan(pa_plan_s* P) {
   cudaFree(P->h_out);
   for (int s = 0; s < kHostSets; ++s)
     if (P->hs[s]) cudaStreamDestroy(P->hs[s]);
-  if (P->host_flag) cudaFreeHost(P->host_flag);
+  if (P->host_flag) g_host_words.give(P->host_flag);
   if (P->h_ev) cudaEventDestroy(P->h_ev);
   for (int s = 0; s < kHostSets; ++s)
     if (P->h_done[s]) cudaEventDestroy(P->h_done[s]);
@@ -2130,7 +2198,7 @@ pa_status host_call_done(pa_plan_s* P, pa_plan_s::HostTune* tune, bool tuning, i
   // (the counts are read only after some wait has run out: a blocking copy a
   // buffer set costs about 10 us; an earlier launch of the plan may have run
   // out before the word existed, so it starts out set)
-  if (*reinterpret_cast<volatile int*>(P->host_flag)) {
+  if (P->host_flag && *reinterpret_cast<volatile int*>(P->host_flag)) {
     *reinterpret_cast<volatile int*>(P->host_flag) = 0;
     long long total = 0;
     for (int b = 0; b < kHostSets; ++b) {
@@ -2392,8 +2460,9 @@ pa_status pa_beamform_host(pa_plan_t P, const void* rf_host, int32_t n_frames, f
     P->h_out_bytes = need_out;
     P->device_bytes += need_out;
   }
-  if (!P->host_flag) {
-    PA_CUDA(cudaHostAlloc((void**)&P->host_flag, sizeof(int), cudaHostAllocMapped));
+  if (!P->host_flag && may_wait(P)) {
+    P->host_flag = g_host_words.take();
+    if (!P->host_flag) return fail(PA_ECUDA, "pinned memory: %s", cudaGetErrorString(cudaGetLastError()));
     *P->host_flag = 1;
   }
   if (!P->h_ev) PA_CUDA(cudaEventCreateWithFlags(&P->h_ev, cudaEventDisableTiming));
