@@ -11,6 +11,7 @@
 #include <cstring>
 #include <mutex>
 #include <string>
+#include <type_traits>
 #include <vector>
 
 #include <cudaTypedefs.h>
@@ -136,7 +137,8 @@ struct FusedForm {
   int blocks_per_sm = 0;
   int tmem_cols = 0;      // TMEM columns per block (compensated sums)
   int splits = 1;         // work items per tile (forms 2, 3)
-  int2* vchunks = nullptr;  // chunk range of a work item (forms 2, 3: of a tile)
+  int2* vchunks = nullptr;  // chunk range of a work item (forms 2, 3: of a tile),
+  size_t chunk_at = 0;      // from this entry of the plan's chunk ranges on
   // prepared slots: a row of zeros, then one row of slot_pitch slots per
   // (frames of an item, channel), for max_frames frames a round (forms 2 and
   // 3: at most that many frames a launch)
@@ -158,7 +160,13 @@ struct pa_plan_s {
   int u0 = 0, u1 = 0, nv = 0, dmin = 0, ndrows = 0, tgroups = 0, window = 0;
   size_t full_entries = 0;  // entries of the full table (n_tiles * (steps + 3) * 32 * slots * kC)
   FusedForm form[4];
-  unsigned char* form_mem = nullptr;  // slots of forms 1-3 and all forms' chunk ranges
+  unsigned char* arena = nullptr;     // the plan's device memory but for the slots (plan_arena)
+  unsigned char* slot_mem = nullptr;  // prepared slots of forms 1-3 (optional)
+  size_t slot_mem_bytes = 0;
+  bool slots_joined = false;          // slot_mem is the end of the arena's allocation
+  unsigned char* spare = nullptr;     // what that allocation's last page leaves
+  size_t spare_bytes = 0;
+  size_t slot_limit = (size_t)-1;     // most bytes of slots the plan may take
   long long slot_pitch = 0;
   int used_lo = 0, used_hi = 0;  // samples [used_lo, used_hi) lie in some window
   int slot_margin = 0, slot_mode = 0;
@@ -184,6 +192,8 @@ struct pa_plan_s {
   float* wtab = nullptr;
   int* lo = nullptr;
   int2* urange = nullptr;
+  int2* chunks = nullptr;  // chunk ranges of all forms
+  unsigned long long* active = nullptr;  // count of active pairs (plan build)
   int4* items = nullptr;   // work-item table (tile, group, tx, tz)
   int2* slot_rg = nullptr; // warp slot -> (column residue, column group)
   float2* tw = nullptr;
@@ -193,7 +203,7 @@ struct pa_plan_s {
   int* scratch[kHostSets] = {nullptr, nullptr, nullptr};
   size_t scratch_ints = 0;
   // host-buffer path
-  void* h_rf = nullptr;
+  void* h_rf = nullptr;       // staging buffers, one allocation or the arena's spare
   float* h_out = nullptr;
   size_t h_rf_bytes = 0, h_out_bytes = 0;
   cudaStream_t hs[kHostSets] = {nullptr, nullptr, nullptr};
@@ -824,7 +834,9 @@ void configure(pa_plan_s* P) {
 int blocks_by_attributes(const FusedForm& f, const cudaFuncAttributes& a, size_t smem) {
   struct Limits {
     int regs = 0, smem = 0, threads = 0, blocks = 0, reserved = 0;
-    explicit Limits(int dev) {
+    Limits() {
+      int dev = 0;
+      if (cudaGetDevice(&dev) != cudaSuccess) return;
       cudaDeviceGetAttribute(&regs, cudaDevAttrMaxRegistersPerMultiprocessor, dev);
       cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev);
       cudaDeviceGetAttribute(&threads, cudaDevAttrMaxThreadsPerMultiProcessor, dev);
@@ -832,9 +844,7 @@ int blocks_by_attributes(const FusedForm& f, const cudaFuncAttributes& a, size_t
       cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev);
     }
   };
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-  const Limits lim(dev);
+  static const Limits lim;  // (one architecture: the same on every device)
   const int warps = (f.threads + 31) / 32;
   const int regs_warp = ((a.numRegs * 32 + 255) / 256) * 256;  // 256-register units per warp
   int b = std::min(lim.regs / std::max(1, regs_warp * warps), lim.threads / (32 * warps));
@@ -852,11 +862,6 @@ cudaError_t fused_blocks_per_sm(const pa_plan_s* P, const FusedForm& f, size_t s
   if (e != cudaSuccess) return e;
   *n = blocks_by_attributes(f, a, smem);
   return cudaSuccess;
-}
-
-// Whether a plan of this descriptor gets the two-frame form (if it fits).
-bool wants_pairs(const pa_plan_s* P) {
-  return P->d.max_batch > 1 && P->K <= 5 && (P->item_frames == 0 || P->item_frames == 2);
 }
 
 // The one-frame form stages this plan's RF windows sample by sample (rows off
@@ -895,25 +900,46 @@ double least_fine_steps(const pa_plan_s* P, int px) {
 // Warps of 4-pixel threads of one frame.
 int64_t frame_warps(const pa_plan_s* P) { return (int64_t)P->n_tiles * P->slots; }
 
-// Frames per round of form 1 (of a launch of forms 2 and 3) and the bytes of
-// their slots; 0 frames: no such form.  The slots
-// of a round are written by the preparation pass and read back by every tile.
+bool fine_pays(const pa_plan_s* P, int px, int nf);  // (with pick_form)
+bool pairs_pay(const pa_plan_s* P, int nf);
+
+// Bytes of a row of form i's prepared slots, and of the rows of a work item.
+size_t slot_row_bytes(const pa_plan_s* P, int i) {
+  return (size_t)P->slot_pitch * (i == 1 ? pipe_slot_bytes(P->slot_mode) : sizeof(float2));
+}
+size_t slot_item_bytes(const pa_plan_s* P, int i) { return (size_t)P->d.n_elem * slot_row_bytes(P, i); }
+// Bound of a round's slots; a plan whose work items are larger has no such form.
 constexpr size_t kSlotBytesMax = (size_t)512 << 20;
-size_t slots_size(const pa_plan_s* P, int form, int* frames) {
-  const int item = form == 1 ? 2 : 1;
+
+// Whether some launch of the plan picks the two-frame form (an even one or an
+// odd one of the largest; build_form2 may still find that it does not fit).
+bool pairs_wanted(const pa_plan_s* P) {
+  if (P->d.max_batch <= 1 || P->K > 5 || slot_item_bytes(P, 1) > kSlotBytesMax) return false;
+  if (P->item_frames != 0) return P->item_frames == 2;
+  return pairs_pay(P, P->d.max_batch) || pairs_pay(P, P->d.max_batch - 1);
+}
+
+// Most frames of a launch that picks a fine-grained form of px pixels a thread
+// (0: none does).
+int fine_wanted(const pa_plan_s* P, int px) {
   const FineLimits lim = fine_limits(P);
-  *frames = 0;
-  if (form > 1 && frame_warps(P) > std::max(lim.px1, lim.px2)) return 0;
-  const size_t sb = form == 1 ? pipe_slot_bytes(P->slot_mode) : sizeof(float2);
-  const size_t row = (size_t)P->slot_pitch * sb;
-  const size_t per_item = (size_t)P->d.n_elem * row;
-  if (per_item > kSlotBytesMax) return 0;  // (one item alone would pass the bound)
-  size_t items = ((size_t)P->d.max_batch + item - 1) / item;
-  if (form > 1)
-    items = std::min<size_t>(items, std::max<int64_t>(1, std::max(lim.px1, lim.px2) / frame_warps(P)));
-  items = std::max<size_t>(1, std::min(items, kSlotBytesMax / per_item));
+  if (slot_item_bytes(P, 2) > kSlotBytesMax || fine_steps(P) < least_fine_steps(P, px)) return 0;
+  for (int64_t nf = std::min<int64_t>(P->d.max_batch, (px == 1 ? lim.px1 : lim.px2) / frame_warps(P));
+       nf > 0; --nf)
+    if (fine_pays(P, px, (int)nf)) return (int)nf;
+  return 0;
+}
+
+// Frames per round of form 1 (of a launch of forms 2 and 3) and the bytes of
+// their slots.  The slots of a round are written by the preparation pass and
+// read back by every tile.
+size_t slots_size(const pa_plan_s* P, int i, int* frames) {
+  const int item = i == 1 ? 2 : 1;
+  const size_t want = i == 1 ? ((size_t)P->d.max_batch + 1) / 2
+                             : (size_t)std::max(fine_wanted(P, 1), fine_wanted(P, 2));
+  const size_t items = std::min(want, kSlotBytesMax / slot_item_bytes(P, i));
   *frames = (int)(item * items);
-  return row + items * per_item;
+  return slot_row_bytes(P, i) + items * slot_item_bytes(P, i);
 }
 
 // Bytes of the delay table and its apodisation weights.
@@ -931,20 +957,32 @@ pa_status check_table_size(const pa_plan_s* P) {
   return PA_OK;
 }
 
-size_t table_bytes(const pa_plan_s* P) {
-  size_t b = delay_table_bytes(P);
-  b += (size_t)P->n_tiles * P->ngroups * sizeof(int4) + (size_t)P->slots * sizeof(int2);
-  b += (size_t)P->n_tiles * P->nv * sizeof(int);
-  b += (size_t)P->n_tiles * P->slots * sizeof(int2);
-  b += (size_t)P->n_tiles * P->ngroups * sizeof(int2);
-  // chunk ranges and slots of the other forms
-  int frames;
-  if (wants_pairs(P))
-    b += (size_t)P->n_tiles * P->ngroups * sizeof(int2) + slots_size(P, 1, &frames);
-  const size_t fine = slots_size(P, 2, &frames);
-  if (frames) b += fine + 2 * (size_t)P->n_tiles * sizeof(int2);
-  b += (size_t)3 * P->M * sizeof(float2) + (size_t)3 * P->M * sizeof(float);
-  return b;
+// The plan's device memory but for the optional prepared slots, one allocation:
+// lays the arrays out from `base` on (null: sizes only) and returns the bytes.
+// (One cudaMalloc of some megabytes costs 30 us and its cudaFree as much; eleven
+// allocations of their own 50-80 us more.)
+size_t plan_arena(pa_plan_s* P, unsigned char* base) {
+  size_t at = 0;
+  auto take = [&](auto** p, size_t n) {
+    if (base) *p = reinterpret_cast<std::remove_reference_t<decltype(**p)>*>(base + at);
+    at += (n * sizeof(**p) + 255) & ~(size_t)255;
+  };
+  const size_t tab_n = P->full ? P->full_entries : (size_t)P->ndrows * P->nz_pad;
+  take(P->full ? &P->ftab : &P->table, tab_n);
+  if (P->apod) take(&P->wtab, tab_n);
+  take(&P->items, (size_t)P->n_tiles * P->ngroups);
+  take(&P->slot_rg, (size_t)P->slots);
+  take(&P->lo, (size_t)P->n_tiles * P->nv);
+  take(&P->urange, (size_t)P->n_tiles * P->slots);
+  take(&P->chunks, (size_t)P->n_tiles * (2 * P->ngroups + 2));  // of forms 0, 1 and 2, 3
+  take(&P->tw, (size_t)3 * P->M);  // n_tw <= 2 M, tw_reg
+  take(&P->mask, (size_t)3 * P->M);
+  take(&P->active, (size_t)1);
+  // [0] error flags, [1] work counter, [2, 2 + 3 max_batch) image maxima,
+  // [last] running count of timed-out waits
+  P->scratch_ints = 3 + (size_t)P->d.max_batch * 3;
+  take(&P->scratch[0], P->scratch_ints);
+  return at;
 }
 
 // cuTensorMapEncodeTiled from the driver, looked up once through the runtime.
@@ -961,6 +999,8 @@ PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   return fn;
 }
 
+size_t round256(size_t b) { return (b + 255) & ~(size_t)255; }
+
 template <typename T>
 pa_status dalloc(pa_plan_s* P, T** ptr, size_t n) {
   if (n == 0) n = 1;
@@ -975,24 +1015,45 @@ pa_status dalloc(pa_plan_s* P, T** ptr, size_t n) {
   return PA_OK;
 }
 
+void drop_host_graphs(pa_plan_s* P) {
+  for (auto& g : P->host_graphs) {
+    cudaGraphExecDestroy(g.exec);
+    cudaGraphDestroy(g.graph);
+  }
+  P->host_graphs.clear();
+}
+
+// Staging buffers of the host path: one allocation, or what the arena's last
+// page leaves if they fit there.
+void free_staging(pa_plan_s* P) {
+  drop_host_graphs(P);
+  if (P->h_rf != P->spare) cudaFree(P->h_rf);
+  P->device_bytes -= P->h_rf_bytes + P->h_out_bytes;
+  P->h_rf = nullptr;
+  P->h_out = nullptr;
+  P->h_rf_bytes = P->h_out_bytes = 0;
+}
+pa_status alloc_staging(pa_plan_s* P, size_t rf, size_t out) {
+  free_staging(P);
+  const size_t at = round256(rf);
+  if (at + out <= P->spare_bytes) P->h_rf = P->spare;
+  else PA_CUDA(cudaMalloc(&P->h_rf, at + out));
+  P->h_out = reinterpret_cast<float*>((unsigned char*)P->h_rf + at);
+  P->h_rf_bytes = rf;
+  P->h_out_bytes = out;
+  P->device_bytes += rf + out;
+  return PA_OK;
+}
+
 void free_plan(pa_plan_s* P) {
   if (!P) return;
   DeviceGuard g(P->device);
   for (int s = 0; s < kHostSets; ++s)
     if (P->hs[s]) cudaStreamSynchronize(P->hs[s]);
-  cudaFree(P->table);
-  cudaFree(P->ftab);
-  cudaFree(P->wtab);
-  cudaFree(P->lo);
-  cudaFree(P->urange);
-  cudaFree(P->form_mem);
-  cudaFree(P->items);
-  cudaFree(P->slot_rg);
-  cudaFree(P->tw);
-  cudaFree(P->mask);
-  for (int s = 0; s < kHostSets; ++s) cudaFree(P->scratch[s]);
-  cudaFree(P->h_rf);
-  cudaFree(P->h_out);
+  free_staging(P);
+  if (!P->slots_joined) cudaFree(P->slot_mem);
+  cudaFree(P->arena);
+  for (int s = 1; s < kHostSets; ++s) cudaFree(P->scratch[s]);
   for (int s = 0; s < kHostSets; ++s)
     if (P->hs[s]) cudaStreamDestroy(P->hs[s]);
   if (P->host_flag) g_host_words.give(P->host_flag);
@@ -1000,10 +1061,6 @@ void free_plan(pa_plan_s* P) {
   for (int s = 0; s < kHostSets; ++s)
     if (P->h_done[s]) cudaEventDestroy(P->h_done[s]);
   for (auto& g : P->graphs) {
-    cudaGraphExecDestroy(g.exec);
-    cudaGraphDestroy(g.graph);
-  }
-  for (auto& g : P->host_graphs) {
     cudaGraphExecDestroy(g.exec);
     cudaGraphDestroy(g.graph);
   }
@@ -1073,41 +1130,119 @@ std::vector<int2> form_chunks(const pa_plan_s* P, const FusedForm& f, const std:
   return vk;
 }
 
-// Device memory of the plan's forms, in one allocation: the slots of form 1,
-// those forms 2 and 3 share, and every form's chunk ranges.  Without room for
-// the slots the plan keeps the one-frame form alone.
-pa_status alloc_forms(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st) {
-  for (;;) {
-    auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
-    int frames1 = 0, frames2 = 0;
-    const size_t s1 = P->form[1].nf ? up(slots_size(P, 1, &frames1)) : 0;
-    const size_t s2 = P->form[2].nf || P->form[3].nf ? up(slots_size(P, 2, &frames2)) : 0;
-    std::vector<int2> all;
-    size_t at[4] = {0, 0, 0, 0};
-    for (int i = 0; i < 4; ++i) {
-      if (!P->form[i].nf) continue;
-      at[i] = all.size();
-      const std::vector<int2> vk = form_chunks(P, P->form[i], ur);
-      all.insert(all.end(), vk.begin(), vk.end());
-    }
-    const pa_status s = dalloc(P, &P->form_mem, s1 + s2 + all.size() * sizeof(int2));
-    if (s != PA_OK) {
-      if (s1 + s2 == 0) return s;
-      for (int i = 1; i < 4; ++i) P->form[i] = FusedForm();
-      continue;
-    }
-    if (s1 + s2) PA_CUDA(cudaMemsetAsync(P->form_mem, 0, s1 + s2, st));
-    int2* vk = reinterpret_cast<int2*>(P->form_mem + s1 + s2);
-    // (pageable: the call returns once `all` has been read)
-    PA_CUDA(cudaMemcpyAsync(vk, all.data(), all.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
-    for (int i = 0; i < 4; ++i) {
-      if (!P->form[i].nf) continue;
-      P->form[i].vchunks = vk + at[i];
-      if (i) P->form[i].slots = P->form_mem + (i == 1 ? 0 : s1);
-      P->form[i].max_frames = i == 1 ? frames1 : frames2;
-    }
-    return PA_OK;
+// Prepared slots are extra: a plan runs the one-frame form without them.  They
+// are taken within the plan's limit and while an eighth of the device's memory
+// stays free beside them.
+bool room_for_slots(const pa_plan_s* P, size_t bytes) {
+  size_t free_b = 0, total = 0;
+  return bytes <= P->slot_limit && cudaMemGetInfo(&free_b, &total) == cudaSuccess &&
+         bytes + total / 8 <= free_b;
+}
+
+// The arena, and with it the slots that the plan is expected to want: one
+// allocation takes half the time of two.  The device maps pages of 2 MiB, so
+// such an allocation asks for whole ones; what its last page leaves serves the
+// staging buffers of the host path if they fit.
+pa_status alloc_arena(pa_plan_s* P, size_t slots) {
+  constexpr size_t kPage = (size_t)2 << 20;
+  const size_t n = plan_arena(P, nullptr);
+  const size_t pages = (n + slots + kPage - 1) / kPage * kPage;
+  if (slots && n + slots > kPage && room_for_slots(P, slots) && dalloc(P, &P->arena, pages) == PA_OK) {
+    P->slot_mem = P->arena + n;
+    P->slot_mem_bytes = slots;
+    P->slots_joined = true;
+    P->spare = P->slot_mem + slots;
+    P->spare_bytes = pages - n - slots;
+    P->device_bytes -= P->spare_bytes;
+  } else if (const pa_status s = dalloc(P, &P->arena, n)) {
+    return s;
   }
+  plan_arena(P, P->arena);
+  return PA_OK;
+}
+
+// Gives the slots' memory back (the device idle, no graph of the plan alive):
+// joined with the arena, the arena moves to an allocation of its own.
+pa_status drop_slot_memory(pa_plan_s* P) {
+  if (P->slots_joined) {
+    const size_t n = plan_arena(P, nullptr);
+    unsigned char* a = nullptr;
+    if (P->h_rf && P->h_rf == P->spare) free_staging(P);
+    PA_CUDA(cudaMalloc(&a, n));
+    const cudaError_t e = cudaMemcpy(a, P->arena, n, cudaMemcpyDeviceToDevice);
+    if (e != cudaSuccess) {
+      cudaFree(a);
+      return fail(PA_ECUDA, "plan arena: %s", cudaGetErrorString(e));
+    }
+    cudaFree(P->arena);
+    P->spare = nullptr;
+    P->spare_bytes = 0;
+    P->arena = a;
+    plan_arena(P, a);
+    for (FusedForm& f : P->form) f.vchunks = P->chunks + f.chunk_at;
+  } else {
+    cudaFree(P->slot_mem);
+  }
+  P->slot_mem = nullptr;
+  P->device_bytes -= P->slot_mem_bytes;
+  P->slot_mem_bytes = 0;
+  P->slots_joined = false;
+  return PA_OK;
+}
+
+// Bytes of slots a plan over the full aperture will want, from its descriptor
+// alone, for the arena's allocation.  Stands on estimates that the build then
+// replaces; apodised plans, whose channel steps come from the tables, are left
+// for later (0).
+size_t expected_slots(pa_plan_s* P) {
+  if (P->apod) return 0;
+  const double steps = P->u1 - P->u0;
+  P->steps_per_pixel = steps;
+  P->form[0].blocks_per_sm = std::max(1, 24 / P->warps);
+  // samples between the nearest delay and the farthest
+  const pa_plan_desc& d = P->d;
+  const double half = 0.5 * (d.n_elem - 1) * d.pitch_m;
+  const double far = std::hypot(d.z1_m, std::max(d.x1_m, -d.x0_m) + half);
+  const double used = std::min((double)d.n_samples, d.fs_hz / d.c_m_s * (far - d.z0_m));
+  P->pairs_pay = steps * P->nx_pad * P->nz_pad >= 48.0 * d.n_elem * used;
+  int frames = 0;
+  size_t b = 0;
+  if (pairs_wanted(P)) b += round256(slots_size(P, 1, &frames));
+  if (fine_wanted(P, 1) || fine_wanted(P, 2)) b += round256(slots_size(P, 2, &frames));
+  return b;
+}
+
+// Slots of form 1 and those forms 2 and 3 share, in one allocation, and the
+// chunk ranges of every form.
+pa_status alloc_forms(pa_plan_s* P, const std::vector<int2>& ur, cudaStream_t st) {
+  int frames1 = 0, frames2 = 0;
+  const size_t s1 = P->form[1].nf ? round256(slots_size(P, 1, &frames1)) : 0;
+  const size_t s2 = P->form[2].nf || P->form[3].nf ? round256(slots_size(P, 2, &frames2)) : 0;
+  if (P->slot_mem && (P->slot_mem_bytes < s1 + s2 || s1 + s2 == 0)) {  // expected otherwise
+    PA_CUDA(cudaStreamSynchronize(st));
+    if (const pa_status s = drop_slot_memory(P)) return s;
+  }
+  if (s1 + s2 && !P->slot_mem) {
+    if (room_for_slots(P, s1 + s2) && dalloc(P, &P->slot_mem, s1 + s2) == PA_OK)
+      P->slot_mem_bytes = s1 + s2;
+    else
+      for (int i = 1; i < 4; ++i) P->form[i] = FusedForm();
+  }
+  if (P->slot_mem) PA_CUDA(cudaMemsetAsync(P->slot_mem, 0, s1 + s2, st));
+  std::vector<int2> all;
+  for (int i = 0; i < 4; ++i) {
+    FusedForm& f = P->form[i];
+    if (!f.nf) continue;
+    f.chunk_at = all.size();
+    f.vchunks = P->chunks + f.chunk_at;
+    if (i) f.slots = P->slot_mem + (i == 1 ? 0 : s1);
+    f.max_frames = i == 1 ? frames1 : frames2;
+    const std::vector<int2> vk = form_chunks(P, f, ur);
+    all.insert(all.end(), vk.begin(), vk.end());
+  }
+  // (pageable: the call returns once `all` has been read)
+  PA_CUDA(cudaMemcpyAsync(P->chunks, all.data(), all.size() * sizeof(int2), cudaMemcpyHostToDevice, st));
+  return PA_OK;
 }
 
 // The one-frame form.
@@ -1178,9 +1313,7 @@ pa_status build_form1(pa_plan_s* P) {
 
 // The two-frame form; a plan it does not fit keeps the one-frame form alone.
 pa_status build_form2(pa_plan_s* P) {
-  int frames = 0;
-  slots_size(P, 1, &frames);
-  if (!wants_pairs(P) || frames == 0) return PA_OK;
+  if (P->d.max_batch <= 1 || P->K > 5) return PA_OK;
   FusedForm f;
   f.nf = 2;
   f.slot_bytes = pipe_slot_bytes(P->slot_mode);
@@ -1227,8 +1360,7 @@ pa_status build_form2(pa_plan_s* P) {
   const double reuse = (double)P->executed_pairs /
                        ((double)P->d.n_elem * std::max(1, P->used_hi - P->used_lo));
   P->pairs_pay = reuse >= 48 && f.blocks_per_sm * P->warps >= (P->K <= 2 ? 12 : 14);
-  // (no launch would pick the form)
-  if (!P->pairs_pay && !staged_by_samples(P) && P->item_frames != 2) return PA_OK;
+  if (!pairs_wanted(P)) return PA_OK;
   if (P->window > P->slot_margin) return PA_OK;  // (the margin bounds it)
   f.slots_form = 1;
   P->form[1] = f;
@@ -1238,12 +1370,7 @@ pa_status build_form2(pa_plan_s* P) {
 // The fine-grained forms: a tile's pixels at px of a thread's four per thread,
 // in blocks of at most 16 warps.
 pa_status build_form3(pa_plan_s* P, int px) {
-  const FineLimits lim = fine_limits(P);
-  if (frame_warps(P) > (px == 1 ? lim.px1 : lim.px2) || P->window > P->slot_margin) return PA_OK;
-  if (fine_steps(P) < least_fine_steps(P, px)) return PA_OK;
-  int frames = 0;
-  slots_size(P, 2, &frames);
-  if (frames == 0) return PA_OK;
+  if (!fine_wanted(P, px) || P->window > P->slot_margin) return PA_OK;
   FusedForm f;
   f.nf = 1;
   f.slot_bytes = sizeof(float2);
@@ -1290,24 +1417,8 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
   PA_CUDA(cudaDeviceGetAttribute(&P->num_sms, cudaDevAttrMultiProcessorCount, P->device));
 
   pa_status s;
-  const size_t tab_n = (size_t)P->ndrows * P->nz_pad;
   if ((s = check_table_size(P)) != PA_OK) return s;
-  if (P->full) {
-    if ((s = dalloc(P, &P->ftab, P->full_entries)) != PA_OK) return s;
-  } else if ((s = dalloc(P, &P->table, tab_n)) != PA_OK) {
-    return s;
-  }
-  if (P->apod && (s = dalloc(P, &P->wtab, P->full ? P->full_entries : tab_n)) != PA_OK) return s;
-  if ((s = dalloc(P, &P->items, (size_t)P->n_tiles * P->ngroups)) != PA_OK) return s;
-  if ((s = dalloc(P, &P->slot_rg, (size_t)P->slots)) != PA_OK) return s;
-  if ((s = dalloc(P, &P->lo, (size_t)P->n_tiles * P->nv)) != PA_OK) return s;
-  if ((s = dalloc(P, &P->urange, (size_t)P->n_tiles * P->slots)) != PA_OK) return s;
-  if ((s = dalloc(P, &P->tw, (size_t)3 * P->M)) != PA_OK) return s;  // n_tw <= 2 M, tw_reg
-  if ((s = dalloc(P, &P->mask, (size_t)3 * P->M)) != PA_OK) return s;
-  // [0] error flags, [1] work counter, [2, 2 + 3 max_batch) image maxima,
-  // [last] running count of timed-out waits
-  P->scratch_ints = 3 + (size_t)P->d.max_batch * 3;
-  if ((s = dalloc(P, &P->scratch[0], P->scratch_ints)) != PA_OK) return s;
+  if ((s = alloc_arena(P, expected_slots(P))) != PA_OK) return s;
   PA_CUDA(cudaMemsetAsync(P->scratch[0], 0, P->scratch_ints * sizeof(int), st));
 
   if ((size_t)36 * P->M > (size_t)200 * 1024)
@@ -1378,9 +1489,8 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
     k_uranges<<<grid, 32, 0, st>>>(g, fg, P->slots, P->u1, kC, P->wtab, P->urange);
     PA_CUDA(cudaGetLastError());
   }
-  unsigned long long* cnt = nullptr;
   if (P->apod) {
-    PA_CUDA(cudaMalloc(&cnt, sizeof(unsigned long long)));
+    unsigned long long* const cnt = P->active;
     PA_CUDA(cudaMemsetAsync(cnt, 0, sizeof(unsigned long long), st));
     if (P->full) {
       const size_t per_tile = P->full_entries / P->n_tiles;
@@ -1390,46 +1500,10 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
       dim3 grid((d.nz + 127) / 128, d.nx);
       k_count_active<<<grid, 128, 0, st>>>(g, d.nx, d.nz, d.n_elem, P->wtab, cnt);
     }
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) {
-      cudaFree(cnt);
-      return fail(PA_ECUDA, "k_count_active: %s", cudaGetErrorString(e));
-    }
+    PA_CUDA(cudaGetLastError());
   }
 
-  int head[5] = {0, 0, 0, 0, 0};
-  std::vector<int2> ur((size_t)P->n_tiles * P->slots);
-  PA_CUDA(cudaMemcpyAsync(head, P->scratch[0], sizeof head, cudaMemcpyDeviceToHost, st));
-  PA_CUDA(cudaMemcpyAsync(ur.data(), P->urange, ur.size() * sizeof(int2), cudaMemcpyDeviceToHost,
-                          st));
-  unsigned long long active = 0;
-  if (cnt) PA_CUDA(cudaMemcpyAsync(&active, cnt, sizeof active, cudaMemcpyDeviceToHost, st));
-  cudaError_t se = cudaStreamSynchronize(st);
-  if (cnt) cudaFree(cnt);
-  if (se != cudaSuccess) return fail(PA_ECUDA, "plan build: %s", cudaGetErrorString(se));
-  if (head[0] != 0) return fail(PA_ECUDA, "plan build: table row outside range (flag %d)", head[0]);
-  const int width = head[2];
-  P->window = ((std::max(width, 1) + 3) / 4) * 4;
-  // samples any window holds
-  P->used_lo = std::max(0, kLoBias - head[4]);
-  P->used_hi = std::min(d.n_samples, head[3] - kLoBias + P->window);
-
-  PA_CUDA(cudaMemsetAsync(P->scratch[0], 0, P->scratch_ints * sizeof(int), st));
-
-  // TMA box geometry of one staged channel
-  P->wr = ((P->window + 1 + P->lo_align - 1) / P->lo_align) * P->lo_align;
-  if (P->wr > 256) P->use_tma = false;  // TMA boxes span at most 256 elements
-  if (P->use_tma && !tensor_map_encoder()) P->use_tma = false;
-  P->executed_pairs = 0;
-  for (int t = 0; t < P->n_tiles * P->slots; ++t)
-    if (ur[t].y > ur[t].x) P->executed_pairs += (int64_t)(ur[t].y - ur[t].x) * 32 * kC;
-  P->steps_per_pixel = (double)P->executed_pairs / ((double)P->nx_pad * P->nz_pad);
-  P->active_pairs = P->apod ? (int64_t)active : (int64_t)d.nx * d.nz * d.n_elem;
-  if ((s = build_form1(P)) != PA_OK) return s;
-  if ((s = build_form2(P)) != PA_OK) return s;
-  if ((s = build_form3(P, 1)) != PA_OK) return s;
-  if ((s = build_form3(P, 2)) != PA_OK) return s;
-  if ((s = alloc_forms(P, ur, st)) != PA_OK) return s;
+  // what does not wait for the kernels, while they run
   // work items (tile, residue group) deepest tiles first; the frame is the
   // fastest index of a work item, so frames of one tile run back to back
   std::vector<int4> it((size_t)P->n_tiles * P->ngroups);
@@ -1503,6 +1577,39 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
                           st));
   // post kernels: at most 200 KiB of shared memory a block
   PA_CUDA(post_configure((size_t)200 * 1024));
+
+  int head[5] = {0, 0, 0, 0, 0};
+  std::vector<int2> ur((size_t)P->n_tiles * P->slots);
+  PA_CUDA(cudaMemcpyAsync(head, P->scratch[0], sizeof head, cudaMemcpyDeviceToHost, st));
+  PA_CUDA(cudaMemcpyAsync(ur.data(), P->urange, ur.size() * sizeof(int2), cudaMemcpyDeviceToHost,
+                          st));
+  unsigned long long active = 0;
+  if (P->apod) PA_CUDA(cudaMemcpyAsync(&active, P->active, sizeof active, cudaMemcpyDeviceToHost, st));
+  cudaError_t se = cudaStreamSynchronize(st);
+  if (se != cudaSuccess) return fail(PA_ECUDA, "plan build: %s", cudaGetErrorString(se));
+  if (head[0] != 0) return fail(PA_ECUDA, "plan build: table row outside range (flag %d)", head[0]);
+  const int width = head[2];
+  P->window = ((std::max(width, 1) + 3) / 4) * 4;
+  // samples any window holds
+  P->used_lo = std::max(0, kLoBias - head[4]);
+  P->used_hi = std::min(d.n_samples, head[3] - kLoBias + P->window);
+
+  PA_CUDA(cudaMemsetAsync(P->scratch[0], 0, P->scratch_ints * sizeof(int), st));
+
+  // TMA box geometry of one staged channel
+  P->wr = ((P->window + 1 + P->lo_align - 1) / P->lo_align) * P->lo_align;
+  if (P->wr > 256) P->use_tma = false;  // TMA boxes span at most 256 elements
+  if (P->use_tma && !tensor_map_encoder()) P->use_tma = false;
+  P->executed_pairs = 0;
+  for (int t = 0; t < P->n_tiles * P->slots; ++t)
+    if (ur[t].y > ur[t].x) P->executed_pairs += (int64_t)(ur[t].y - ur[t].x) * 32 * kC;
+  P->steps_per_pixel = (double)P->executed_pairs / ((double)P->nx_pad * P->nz_pad);
+  P->active_pairs = P->apod ? (int64_t)active : (int64_t)d.nx * d.nz * d.n_elem;
+  if ((s = build_form1(P)) != PA_OK) return s;
+  if ((s = build_form2(P)) != PA_OK) return s;
+  if ((s = build_form3(P, 1)) != PA_OK) return s;
+  if ((s = build_form3(P, 2)) != PA_OK) return s;
+  if ((s = alloc_forms(P, ur, st)) != PA_OK) return s;
   PA_CUDA(cudaStreamSynchronize(st));
   return PA_OK;
 }
@@ -2091,14 +2198,6 @@ void host_tune_record(pa_plan_s::HostTune* t, int cur, double ms, bool cold) {
   t->chosen = (int)(std::min_element(t->best_ms.begin(), t->best_ms.end()) - t->best_ms.begin());
 }
 
-void drop_host_graphs(pa_plan_s* P) {
-  for (auto& g : P->host_graphs) {
-    cudaGraphExecDestroy(g.exec);
-    cudaGraphDestroy(g.graph);
-  }
-  P->host_graphs.clear();
-}
-
 bool is_pinned(const void* p) {
   cudaPointerAttributes a{};
   if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
@@ -2327,8 +2426,7 @@ pa_status pa_plan_footprint(const pa_plan_desc* desc, int32_t n_frames, size_t* 
   P.d = *desc;
   configure(&P);
   if ((s = check_table_size(&P)) != PA_OK) return s;
-  size_t b = table_bytes(&P);
-  b += (3 + (size_t)P.d.max_batch * 3) * sizeof(int);  // scratch, as pa_plan allocates it
+  size_t b = plan_arena(&P, nullptr);
   const size_t elt = desc->rf_dtype == PA_RF_F32 ? 4 : 2;
   b += (size_t)n_frames * desc->n_elem * desc->n_samples * elt;
   b += (size_t)n_frames * 3 * P.n_out * desc->nx * desc->nz * sizeof(float);
@@ -2440,25 +2538,11 @@ pa_status pa_beamform_host(pa_plan_t P, const void* rf_host, int32_t n_frames, f
   const size_t out_frame = (size_t)popcount3(stages) * P->n_out * d.nx * d.nz;
   const size_t need_rf = (size_t)sets_needed * chunk * rf_frame;
   const size_t need_out = (size_t)sets_needed * chunk * out_frame * sizeof(float);
-  if (need_rf > P->h_rf_bytes) {
+  if (need_rf > P->h_rf_bytes || need_out > P->h_out_bytes) {
     grew = true;
-    drop_host_graphs(P);
-    cudaFree(P->h_rf);
-    P->device_bytes -= P->h_rf_bytes;
-    P->h_rf_bytes = 0;
-    PA_CUDA(cudaMalloc(&P->h_rf, need_rf));
-    P->h_rf_bytes = need_rf;
-    P->device_bytes += need_rf;
-  }
-  if (need_out > P->h_out_bytes) {
-    grew = true;
-    drop_host_graphs(P);
-    cudaFree(P->h_out);
-    P->device_bytes -= P->h_out_bytes;
-    P->h_out_bytes = 0;
-    PA_CUDA(cudaMalloc(&P->h_out, need_out));
-    P->h_out_bytes = need_out;
-    P->device_bytes += need_out;
+    const pa_status s = alloc_staging(P, std::max(need_rf, P->h_rf_bytes),
+                                      std::max(need_out, P->h_out_bytes));
+    if (s != PA_OK) return s;
   }
   if (!P->host_flag && may_wait(P)) {
     P->host_flag = g_host_words.take();
