@@ -66,7 +66,8 @@ static_assert(kPipeSlotOff >= kPipeCbOff + kPipeStages * kCbInts * 4 && kPipeSlo
 // from it.  The fused kernels come to it before their last epilogue: from their
 // start on, the successor's blocks crowd onto the SMs that are free first
 // (one quick-look frame 20.6 -> 22.4 us, five ragged frames 74.0 -> 75.5;
-// prepare_chunk says when the post filter keeps a plain edge).
+// prepare_chunk says when the post filter keeps a plain edge, and why the one-frame
+// form has one after the clearing kernel).
 // Loads of the chain's buffers are plain or bulk loads, never the read-only
 // path; the proxy fence orders bulk copies of slots that the preparation pass
 // stored.  Measured on GB300 (whole calls back to back, plain -> programmatic
