@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(512, 2) k_bf_fine(const __grid_constant__ BfPa
       reinterpret_cast<int*>(smem + kPipeCountOff)[s] = 0;
     }
     *reinterpret_cast<int*>(smem + kPipeStopOff) = 0;
-    reinterpret_cast<int4*>(smem + kPipeProdOff)[1] = make_int4(0, 0, 0, 0);
+    reinterpret_cast<int4*>(smem + kPipeProdOff)[1] = make_int4(0, 0, 0, 3);
   }
   wait_previous();
   __syncthreads();

@@ -317,10 +317,12 @@ __device__ __forceinline__ void produce(const BfParams& p, unsigned char* smem, 
   __syncwarp();
   if (run.w == 2) return;  // no work left
   bool first = false;
-  if (run.w == 0) {
-    int item = 0;
-    if (lane == 0) item = atomicAdd(p.counter, 1);
-    item = __shfl_sync(0xffffffffu, item, 0);
+  if (run.w == 0 || run.w == 3) {  // 3: the block's first item (see k_bf_fused)
+    int item = (int)blockIdx.x;
+    if (run.w == 0) {
+      if (lane == 0) item = (int)gridDim.x + atomicAdd(p.counter, 1);
+      item = __shfl_sync(0xffffffffu, item, 0);
+    }
     if (item >= p.n_items) {
       if (lane == 0) {
         prod[1] = make_int4(0, 0, 0, 2);
@@ -434,7 +436,7 @@ __global__ void __launch_bounds__(256, pipe_blocks(K, APOD, COMP, FULL)) k_bf_pi
       reinterpret_cast<int*>(smem + kPipeCountOff)[s] = 0;
     }
     *reinterpret_cast<int*>(smem + kPipeStopOff) = 0;
-    reinterpret_cast<int4*>(smem + kPipeProdOff)[1] = make_int4(0, 0, 0, 0);
+    reinterpret_cast<int4*>(smem + kPipeProdOff)[1] = make_int4(0, 0, 0, 3);
   }
   __syncthreads();
   int stage = 0, phase = 0;
