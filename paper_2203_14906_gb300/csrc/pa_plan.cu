@@ -1889,12 +1889,17 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
     sb.spec.block = dim3(f.threads);
     sb.spec.smem = f.smem;
     sb.args[0] = &rd.b;
-    // The clearing kernel's one block lets its successor come up at once, before
-    // it is spread evenly: where the graph's parameters were rewritten (a call
-    // on other buffers than the last) its blocks crowded onto some SMs (one frame
-    // of 512 x 512 41.3 -> 47.8 us, of 880 x 435 70 -> 98; with a plain edge 41.3
-    // and 70 on the same buffers and on others).
-    sb.chain = f.slots != nullptr;
+    // The kernel before lets its successor come up from its start on, and blocks
+    // that are placed while it still runs are not spread evenly.  So a fused
+    // kernel has a plain edge unless it has more items than resident blocks, or
+    // Kahan sums in the two-frame form (whose blocks allocate tensor memory
+    // first).  Measured: after the clearing kernel on buffers other than the last
+    // call's, one frame of 512 x 512 41.3 -> 47.8 us, of 880 x 435 70 -> 98 (plain
+    // edge 41.3 and 70 on any buffers); fine-grained, one frame of 492 x 62 29.1,
+    // plain 21.0, one of 572 x 125 with Kahan sums 39.4, plain 29.3; two frames of
+    // 292 x 765 at order 4 74.5, plain 64.3; but six BF16 frames of 256 x 256 with
+    // Kahan sums 39.3, plain 41.3.
+    sb.chain = f.nf == 2 && (P->comp || rd.b.n_items > (int)sb.spec.grid.x);
     sb.begin = f.slots ? -1 : 0;
     sb.end = 0;
     c->steps.push_back(sb);
