@@ -875,27 +875,22 @@ bool may_wait(const pa_plan_s* P) {
 }
 
 // Largest launch, in warps of 4-pixel threads, for which the fine-grained forms
-// (one pixel a thread, and two) are built; pick_form says which of these
-// launches run them.
+// (one pixel a thread, and two) are built, and the least mean channel steps per
+// pixel; pick_form says which of these launches run them, and why.
 struct FineLimits {
   int px1, px2;
 };
 FineLimits fine_limits(const pa_plan_s* P) {
   if (P->item_frames == 3) return {1 << 20, 0};  // tests
   if (P->item_frames == 4) return {0, 1 << 20};
-  if (P->item_frames != 0) return {0, 0};
-  const bool loads = !P->full && !P->use_tma && !staged_by_samples(P);
-  if (!P->full && P->use_tma && !P->comp) return {0, 0};
-  if (loads && !P->comp && (P->K < 3 || P->K > 5)) return {0, 0};
-  return P->comp || P->full || staged_by_samples(P) ? FineLimits{1100, 2400} : FineLimits{600, 0};
+  if (P->item_frames != 0 || (!P->full && P->use_tma)) return {0, 0};
+  const bool two = !P->comp && P->K <= 5 && (P->full || (staged_by_samples(P) && P->K >= 3));
+  return {1100, two ? 2400 : 0};
 }
-// Least mean channel steps per pixel of those forms: fewer do not repay the
-// preparation pass (0.84-1.0), nor fewer than 48 at orders up to 3 where the
-// one-frame form reads whole rows by vector loads (0.91-1.0).
 double fine_steps(const pa_plan_s* P) { return P->item_frames >= 3 ? 1e9 : P->steps_per_pixel; }
 double least_fine_steps(const pa_plan_s* P, int px) {
-  if (px == 2) return !P->full && P->use_tma ? 110 : 50;
-  return !P->full && !P->use_tma && !staged_by_samples(P) && P->K <= 3 ? 48 : 28;
+  const bool loads = !P->full && !staged_by_samples(P);
+  return px == 2 || (loads && P->K <= 2) ? 50 : 28;
 }
 // Warps of 4-pixel threads of one frame.
 int64_t frame_warps(const pa_plan_s* P) { return (int64_t)P->n_tiles * P->slots; }
@@ -1353,10 +1348,11 @@ pa_status build_form2(pa_plan_s* P) {
   // chunks of fewer than 12 steps (RF windows of more than 200 samples) spend
   // their time on the hand-over (0.89 measured at 8 steps)
   if (f.nc < std::min(12, std::min(steps, cap))) return PA_OK;
-  // 12 resident warps (six-warp blocks, wide windows) are enough for orders
-  // <= 2 (1.12), not for higher ones (0.92-1.0)
-  // and the preparation pass pays where a sample serves enough pairs (38 pairs
-  // a sample: 0.95)
+  // Where pairs_pay asks for it: 12 resident warps (six-warp blocks, wide
+  // windows) are enough for orders <= 2 (1.12), not for higher ones (0.92-1.0),
+  // and the preparation pass pays where a sample serves enough pairs (a twentieth
+  // slower than the one-frame form: 2.5 % of all launches without this line,
+  // 1.7 % with it).
   const double reuse = (double)P->executed_pairs /
                        ((double)P->d.n_elem * std::max(1, P->used_hi - P->used_lo));
   P->pairs_pay = reuse >= 48 && f.blocks_per_sm * P->warps >= (P->K <= 2 ? 12 : 14);
@@ -1674,60 +1670,68 @@ bool encode_rf_map(pa_plan_s* P, const void* rf, int nf, CUtensorMap* map) {
 // The form a launch of nf frames runs.  The lines follow 4500 random plans (24-256
 // elements, 48-1024 depth rows, 1-48 frames, every option), each form timed
 // warm and with the record and tables out of L2; the figures are means of
-// one-frame form time / this form's time.  What decides is how many work items
-// of the one-frame form an SM gets (`per_sm`; a block is an item, so few items
-// leave SMs idle or one SM with twice another's work), and how the one-frame
-// form stages its record: by TMA (16-bit rows on 16-byte boundaries), by vector
-// loads, or, rows off 16-byte boundaries, sample by sample.
+// one-frame form time / this form's time over a class of them (with these lines
+// the choice is 0.957 of the fastest form on average, and a twentieth
+// slower than the one-frame form on 1.7 %).  What decides is how many work items
+// of the one-frame form an SM gets (a block is an item, so few items leave SMs
+// idle or one SM with twice another's work), and how that form stages its
+// record: by TMA (16-bit rows on 16-byte boundaries), by vector loads, or, rows
+// off 16-byte boundaries, sample by sample.
 //
-// One pixel a thread (up to 1100 warps of 4-pixel threads; 600 for plain sums
-// off vector loads, 0.8 beyond):
-//   full table 1.25-1.5 up to two items an SM, with Kahan sums at any number
-//     (1.28 at order 6, 1.09 at 7, 0.98 at 8, whose sums spill most);
-//   lattice, TMA: plain sums 0.75-0.95, never; Kahan sums 1.1-1.3 between one
-//     item an SM and two, 0.87-0.97 on either side;
-//   lattice, by samples: Kahan sums 1.0-1.5; plain sums 1.1-1.25 up to one item
-//     an SM, with 50 steps and more 1.05 up to 1.5, 0.8-0.9 beyond;
-//   lattice, vector loads: Kahan sums 1.0-1.45; plain sums of orders 3-5
-//     1.03-1.13 up to half an item an SM, with 50 steps and more 1.03 up to one,
-//     0.75-0.98 beyond; other orders 0.87-1.02.
-// Two pixels a thread (Kahan sums, full table, records by samples; up to 2400
-// warps), from two items an SM on (0.6-0.95 below):
-//   full table 1.1-1.45, with Kahan sums up to four items an SM (0.85-1.05
-//     beyond); lattice with Kahan sums 1.1-1.3 up to four (TMA: from 110 steps
-//     on), 0.8-0.95 beyond; plain sums by samples 1.06-1.4 above four, or above
-//     three with 110 steps.
-// Two frames an item (orders up to 5):
-//   Kahan sums: from 0.65 of the resident blocks on 1.05-1.5 (0.3 where the
-//     record is staged by samples: 1.2-1.6); plain sums need pairs of items
-//     enough as well, two an SM, 2.5 at orders up to 2: 1.06-1.4, and 0.7-0.97
-//     below that (0.6 of the resident blocks by samples);
-//   an odd launch's last item does a frame's work twice: 3 and 5 frames 0.85-1.0
-//     but where the record is staged by samples; from 7 on 1.04-1.3;
-//   and the samples of a row have to serve pairs enough (pairs_pay).
+// One pixel a thread, up to two items an SM and 1100 warps of 4-pixel threads:
+//   full table: plain sums 1.25-1.75 (orders 6-8: 1.07), Kahan sums 1.2-1.55 at
+//     orders up to 5, 1.1 at 6 and 7 up to one item an SM and 0.93-0.99 beyond,
+//     0.98 at 8, whose sums spill most;
+//   lattice, TMA: never (0.83-1.05);
+//   lattice, by samples: 1.2-1.45 up to one item an SM, with 50 steps and more
+//     1.05-1.25 up to two (fewer: 0.92-1.03);
+//   lattice, vector loads: 1.05-1.1 up to half an item an SM, with 50 steps and
+//     more 1.1-1.3 up to one and 1.03-1.2 up to two (fewer: 0.95-1.02); orders 1
+//     and 2 1.15 with 50 steps up to half an item, about 1 elsewhere.
+//   Fewer than 28 steps do not repay the preparation pass (0.84-1.05).
+// Two pixels a thread, plain sums from 50 steps and from two items an SM on, up
+// to 2400 warps (at fewer items one pixel is the better one; Kahan sums, TMA and
+// vector loads 0.8-1.05):
+//   full table, orders up to 5: 1.1-1.45;
+//   lattice, by samples: order 3 1.2-1.25 up to four items an SM, 4 and 5
+//     1.08-1.13 up to three, 0.95-1.05 elsewhere.
 bool fine_pays(const pa_plan_s* P, int px, int nf) {
   const FineLimits lim = fine_limits(P);
   if (frame_warps(P) * nf > (px == 1 ? lim.px1 : lim.px2)) return false;
   if (P->item_frames != 0) return true;
-  const double per_sm = (double)P->n_tiles * P->ngroups * nf / P->num_sms, steps = fine_steps(P);
-  if (px == 1) {
-    if (P->full) return P->comp ? P->K <= 7 : per_sm <= 2;
-    if (P->use_tma) return P->comp && per_sm > 1 && per_sm <= 2;
-    if (P->comp) return true;
-    if (staged_by_samples(P)) return per_sm <= 1 || (per_sm <= 1.5 && steps >= 50);
-    return per_sm <= 0.5 || (per_sm <= 1 && steps >= 50);
-  }
-  if (per_sm <= 2) return false;
-  if (P->comp) return per_sm <= 4;
-  return P->full || per_sm > 4 || (per_sm > 3 && steps >= 110);
+  const double per_sm = (double)P->n_tiles * P->ngroups * nf / P->num_sms;
+  if (px == 2) return per_sm > 2 && (P->full || per_sm <= (P->K == 3 ? 4 : 3));
+  if (P->full) return per_sm <= (!P->comp || P->K <= 5 ? 2 : P->K <= 7 ? 1 : 0);
+  if (!staged_by_samples(P) && P->K <= 2) return per_sm <= 0.5;
+  return per_sm <= (fine_steps(P) >= 50 ? 2 : staged_by_samples(P) ? 1 : 0.5);
 }
 
+// Two frames an item (orders up to 5).  An item does twice the work, so the line
+// is the number of pairs of items an SM gets, from which the time saved per
+// item exceeds the coarser end of the launch:
+//   full table 1.25-1.35: plain sums of orders up to 3 at any number, Kahan sums
+//     of orders 1 and 2 from 1.5, the others from 3 (0.7-1.0 below);
+//   lattice, by samples, from 2.5: 1.15-1.2 (0.75-1.05 below; at order 3, plain,
+//     1.05 from 1.5 on);
+//   lattice, vector loads, from 3, orders 1 and 2 from 4: 1.08-1.2 (0.8-0.95);
+//   lattice, TMA, from 4.5: 1.0-1.13; Kahan sums of orders 1 and 2 and
+//     apodised ones from 2.5: 1.06 (0.75-0.9 below either).
+// An odd launch's last item does a frame's work twice: 3 and 5 frames 0.85-1.0
+// but where the record is staged by samples, from three pairs an SM on; 7 and
+// more as even launches.  And where rows come by TMA or vector loads, or the
+// full table's plain sums are of orders 4 and 5, their samples have to serve
+// pairs enough (build_form2: 0.85-1.0 otherwise).
 bool pairs_pay(const pa_plan_s* P, int nf) {
-  const double items = (double)P->n_tiles * P->ngroups;
-  const double fill = items * nf / ((double)P->form[0].blocks_per_sm * P->num_sms);
-  const bool enough = P->comp || items * ((nf + 1) / 2) >= (P->K <= 2 ? 2.5 : 2.0) * P->num_sms;
-  if (staged_by_samples(P)) return enough && fill >= (P->comp ? 0.3 : 0.6);
-  return enough && fill >= 0.65 && (nf % 2 == 0 || nf >= 7) && P->pairs_pay;
+  const double per_sm = (double)P->n_tiles * P->ngroups * ((nf + 1) / 2) / P->num_sms;
+  const bool by_samples = !P->full && staged_by_samples(P);
+  if (nf % 2 != 0 && nf < 7 && !(by_samples && per_sm >= 3)) return false;
+  if (P->full && P->comp) return per_sm >= (P->K <= 2 ? 1.5 : 3);
+  if (P->full && P->K <= 3) return true;
+  if (by_samples) return per_sm >= 2.5;
+  if (!P->pairs_pay) return false;
+  if (P->full) return per_sm >= 3;
+  if (!P->use_tma) return per_sm >= (P->K <= 2 ? 4 : 3);
+  return per_sm >= (P->comp && (P->K <= 2 || P->apod) ? 2.5 : 4.5);
 }
 
 const FusedForm& pick_form(const pa_plan_s* P, int nf) {
