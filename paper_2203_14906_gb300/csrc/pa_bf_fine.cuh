@@ -12,12 +12,11 @@
 // four.  Chunks come as in the two-frame form, by bulk copies from slots
 // prepared for the launch ({r, d} per sample; the pass takes the place of the
 // clearing kernel) into two buffers; a tile's channel windows are copied once
-// per block of up to 16 warps.  Kahan totals are kept beside the sums (a pixel's
-// 2 x 5 at k = 3), in registers as far as the 64 of two blocks a SM go: one pixel
-// a thread spills 6-36 bytes at k = 3 and 250 at k = 8, two pixels 112 to 500,
-// outside the channel loop's inner steps (the totals are touched every 64).  Over
-// 900 plans these variants still take 0.78-0.92 of the one-frame form's time where
-// pick_form sends them.
+// per block of up to 16 warps.  Kahan totals (one pixel a thread) are kept beside
+// the sums (2 x 5 at k = 3), in registers as far as the 64 of two blocks a SM go:
+// they spill 6-36 bytes at k = 3 and 250 at k = 8, outside the channel loop's
+// inner steps (the totals are touched every 64).  These variants still take
+// 0.65-0.9 of the one-frame form's time where pick_form sends them.
 // Measured on GB300 (RAW images, one-frame form -> this): one frame of 128 x 128,
 // 64 channels, k = 3 18.9 -> 14.8 us; one and two frames of 256 x 256, 64
 // channels, k = 2 BF16 + Kahan 16.7 -> 14.8 and 27.4 -> 18.9; one frame of 400 x
@@ -266,18 +265,23 @@ __global__ void __launch_bounds__(512, 2) k_bf_fine(const __grid_constant__ BfPa
 
 }  // namespace pa
 
+// (Null where no launch takes the form: fine_limits.)
 #define PA_DEFINE_FINE(K)                                                          \
   namespace pa {                                                                   \
-  template <bool FULL, int PX>                                                     \
-  static const void* pick_fine_k##K(bool apod, bool comp) {                        \
-    void (*f)(BfParams) = apod ? (comp ? k_bf_fine<K, true, true, FULL, PX>        \
-                                       : k_bf_fine<K, true, false, FULL, PX>)      \
-                               : (comp ? k_bf_fine<K, false, true, FULL, PX>       \
-                                       : k_bf_fine<K, false, false, FULL, PX>);    \
+  template <bool FULL>                                                             \
+  static const void* pick_fine_k##K(bool apod, bool comp, int px) {                \
+    void (*f)(BfParams) = nullptr;                                                 \
+    if (px == 1 && !comp)                                                          \
+      f = apod ? k_bf_fine<K, true, false, FULL, 1> : k_bf_fine<K, false, false, FULL, 1>; \
+    if constexpr (!FULL || K < 8)                                                  \
+      if (px == 1 && comp)                                                         \
+        f = apod ? k_bf_fine<K, true, true, FULL, 1> : k_bf_fine<K, false, true, FULL, 1>; \
+    if constexpr (K <= 5 && (FULL || K >= 3))                                      \
+      if (px == 2 && !comp)                                                        \
+        f = apod ? k_bf_fine<K, true, false, FULL, 2> : k_bf_fine<K, false, false, FULL, 2>; \
     return reinterpret_cast<const void*>(f);                                       \
   }                                                                                \
   const void* bf_fine_func_k##K(bool apod, bool comp, bool full, int px) {         \
-    if (px == 1) return full ? pick_fine_k##K<true, 1>(apod, comp) : pick_fine_k##K<false, 1>(apod, comp); \
-    return full ? pick_fine_k##K<true, 2>(apod, comp) : pick_fine_k##K<false, 2>(apod, comp); \
+    return full ? pick_fine_k##K<true>(apod, comp, px) : pick_fine_k##K<false>(apod, comp, px); \
   }                                                                                \
   }

@@ -881,11 +881,13 @@ struct FineLimits {
   int px1, px2;
 };
 FineLimits fine_limits(const pa_plan_s* P) {
-  if (P->item_frames == 3) return {1 << 20, 0};  // tests
-  if (P->item_frames == 4) return {0, 1 << 20};
+  // (the variants that have kernels)
+  const bool one = !P->full || !P->comp || P->K < 8;
+  const bool two = !P->comp && P->K <= 5 && (P->full || P->K >= 3);
+  if (P->item_frames == 3) return {one ? 1 << 20 : 0, 0};  // tests
+  if (P->item_frames == 4) return {0, two ? 1 << 20 : 0};
   if (P->item_frames != 0 || (!P->full && P->use_tma)) return {0, 0};
-  const bool two = !P->comp && P->K <= 5 && (P->full || (staged_by_samples(P) && P->K >= 3));
-  return {1100, two ? 2400 : 0};
+  return {one ? 1100 : 0, two && (P->full || staged_by_samples(P)) ? 2400 : 0};
 }
 double fine_steps(const pa_plan_s* P) { return P->item_frames >= 3 ? 1e9 : P->steps_per_pixel; }
 double least_fine_steps(const pa_plan_s* P, int px) {
@@ -1701,7 +1703,7 @@ bool fine_pays(const pa_plan_s* P, int px, int nf) {
   if (P->item_frames != 0) return true;
   const double per_sm = (double)P->n_tiles * P->ngroups * nf / P->num_sms;
   if (px == 2) return per_sm > 2 && (P->full || per_sm <= (P->K == 3 ? 4 : 3));
-  if (P->full) return per_sm <= (!P->comp || P->K <= 5 ? 2 : P->K <= 7 ? 1 : 0);
+  if (P->full) return per_sm <= (!P->comp || P->K <= 5 ? 2 : 1);
   if (!staged_by_samples(P) && P->K <= 2) return per_sm <= 0.5;
   return per_sm <= (fine_steps(P) >= 50 ? 2 : staged_by_samples(P) ? 1 : 0.5);
 }

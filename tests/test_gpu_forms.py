@@ -32,6 +32,15 @@ def _wl(m, **kw):
     return wl
 
 
+def _has(form, k, comp, table):
+    """Whether the form has a kernel for these sums."""
+    if form == TWO:
+        return k <= 5
+    if form == FINE1:
+        return not (comp and table == "full" and k == 8)
+    return form == ONE or (not comp and k <= 5 and (table == "full" or k >= 3))
+
+
 def _run(wl, k, form, rf, frames, monkeypatch, dtype="f32", checked=False):
     import torch
 
@@ -70,7 +79,9 @@ def test_every_variant_runs_and_has_the_one_frame_bits(m, k, monkeypatch):
         rf = _frames(wl, 3)
         ref = _run(wl, k, ONE, rf, 3, monkeypatch)
         assert float(ref.abs().max()) > 0
-        for form in (TWO, FINE1, FINE2) if k <= 5 else (FINE1, FINE2):
+        for form in (TWO, FINE1, FINE2):
+            if not _has(form, k, comp, table):
+                continue
             out = _run(wl, k, form, rf, 3, monkeypatch)
             assert torch.equal(out, ref), (form, f_number, comp, interp, table)
 
@@ -78,9 +89,12 @@ def test_every_variant_runs_and_has_the_one_frame_bits(m, k, monkeypatch):
 @pytest.mark.parametrize("form", [ONE, TWO, FINE1, FINE2])
 @pytest.mark.parametrize("k,m,comp,f_number,interp,table,dtype", [
     (3, 4, 0, 0.0, "linear", "lattice", "f32"), (3, 4, 1, 0.0, "linear", "lattice", "bf16"),
+    (4, 4, 0, 1.4, "nearest", "lattice", "bf16"),
     (5, 8, 1, 0.0, "nearest", "lattice", "f32"), (2, 4, 1, 1.4, "linear", "lattice", "f16"),
     (2, 4, 0, 1.4, "nearest", "full", "f32"), (4, 4, 1, 1.4, "linear", "full", "bf16")])
 def test_checked_build_of_every_form(form, k, m, comp, f_number, interp, table, dtype, monkeypatch):
+    if not _has(form, k, comp, table):
+        pytest.skip("no such kernel")
     wl = _wl(m, f_number=f_number, interp=interp, delay_table=table, compensated=comp)
     _run(wl, k, form, _frames(wl, 3, dtype), 3, monkeypatch, dtype=dtype, checked=True)
 
@@ -94,7 +108,7 @@ def test_a_wait_that_runs_out_is_reported(form, monkeypatch):
 
     wl = synth.workload("cfg1", nx=128, nz=64, z1_m=10e-3)  # 2 columns a pitch: 4 warps
     store, _ = synth.quantize(np.stack([synth.make_frame(wl, s) for s in (1, 2)]), "bf16")
-    desc = pa.make_desc(wl, order_k=3, rf_dtype="bf16", compensated=1, max_batch=2)
+    desc = pa.make_desc(wl, order_k=3, rf_dtype="bf16", compensated=int(form != FINE2), max_batch=2)
     monkeypatch.setenv("PA_ITEM_FRAMES", str(form))
     for shortfall in (True, False):
         if shortfall:
