@@ -203,8 +203,13 @@ typedef struct {
  */
 pa_status pa_plan(const pa_plan_desc* desc, void* cuda_stream, pa_plan_t* out);
 
-/* Bytes of device memory a plan for desc holds, plus the RF and output
- * buffers of n_frames frames with all stages (for admission control). */
+/* Bytes of device memory a plan for desc cannot do without, plus the RF and
+ * output buffers of n_frames frames with all stages (for admission control).
+ * A plan some of whose launches run another form than the one-frame one holds
+ * prepared samples for them besides, at most 512 MiB for either kind (16 bytes
+ * a sample and frame pair; 8 a sample and frame of small launches), as long as
+ * an eighth of the device's memory stays free beside them: pa_plan_info's
+ * device_bytes counts them. */
 pa_status pa_plan_footprint(const pa_plan_desc* desc, int32_t n_frames,
                             size_t* bytes);
 

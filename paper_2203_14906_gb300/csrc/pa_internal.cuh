@@ -303,6 +303,16 @@ void set_error_message(const char* msg);
 int* plan_timeout_counter(pa_plan_s* P);
 // Device memory the plan owns (without synchronising, unlike pa_plan_get_info).
 size_t plan_device_bytes(const pa_plan_s* P);
+// Of these, the prepared slots, without which the plan runs its one-frame form.
+size_t plan_slot_bytes(const pa_plan_s* P);
+// pa_plan with at most slot_limit bytes of slots, which plan_drop_slots can give
+// back; and that: nothing of the plan in flight, no graph of it kept
+// (pa_plan_use_graph 0).
+constexpr size_t kNoSlotLimit = (size_t)-1;
+pa_status plan_create(const pa_plan_desc* desc, cudaStream_t st, size_t slot_limit, pa_plan_s** out);
+pa_status plan_drop_slots(pa_plan_s* P);
+// Device memory a plan for desc cannot do without, and a bound of its slots.
+pa_status plan_memory(const pa_plan_desc* desc, size_t* bytes, size_t* slots);
 // The fused kernel's parameters for one launch of nf frames (what pa_beamform
 // would launch), the plan's order, and whether the plan is the plain FP32
 // lattice form with linear interpolation.

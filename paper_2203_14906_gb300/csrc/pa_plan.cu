@@ -166,7 +166,7 @@ struct pa_plan_s {
   bool slots_joined = false;          // slot_mem is the end of the arena's allocation
   unsigned char* spare = nullptr;     // what that allocation's last page leaves
   size_t spare_bytes = 0;
-  size_t slot_limit = (size_t)-1;     // most bytes of slots the plan may take
+  size_t slot_limit = kNoSlotLimit;   // most bytes of slots the plan may take
   long long slot_pitch = 0;
   int used_lo = 0, used_hi = 0;  // samples [used_lo, used_hi) lie in some window
   int slot_margin = 0, slot_mode = 0;
@@ -1416,7 +1416,9 @@ pa_status build_plan(pa_plan_s* P, cudaStream_t st) {
 
   pa_status s;
   if ((s = check_table_size(P)) != PA_OK) return s;
-  if ((s = alloc_arena(P, expected_slots(P))) != PA_OK) return s;
+  // (slots that a caller limits may be given back later: an allocation of their own)
+  const bool join = P->slot_limit == kNoSlotLimit;
+  if ((s = alloc_arena(P, join ? expected_slots(P) : 0)) != PA_OK) return s;
   PA_CUDA(cudaMemsetAsync(P->scratch[0], 0, P->scratch_ints * sizeof(int), st));
 
   if ((size_t)36 * P->M > (size_t)200 * 1024)
@@ -2345,6 +2347,55 @@ int* plan_timeout_counter(pa_plan_s* P) {
 
 size_t plan_device_bytes(const pa_plan_s* P) { return P ? P->device_bytes : 0; }
 
+size_t plan_slot_bytes(const pa_plan_s* P) { return P ? P->slot_mem_bytes : 0; }
+
+pa_status plan_create(const pa_plan_desc* desc, cudaStream_t st, size_t slot_limit, pa_plan_s** out) {
+  *out = nullptr;
+  pa_status s = validate(desc);
+  if (s != PA_OK) return s;
+  pa_plan_s* P = new (std::nothrow) pa_plan_s();
+  if (!P) return fail(PA_ENOMEM, "host allocation failed");
+  P->d = *desc;
+  P->slot_limit = slot_limit;
+  configure(P);
+  s = build_plan(P, st);
+  if (s != PA_OK) {
+    const std::string keep = g_err;
+    free_plan(P);
+    g_err = keep;
+    return s;
+  }
+  *out = P;
+  return PA_OK;
+}
+
+pa_status plan_drop_slots(pa_plan_s* P) {
+  if (!P->slot_mem) return PA_OK;
+  for (int i = 1; i < 4; ++i) P->form[i] = FusedForm();
+  return drop_slot_memory(P);
+}
+
+pa_status plan_memory(const pa_plan_desc* desc, size_t* bytes, size_t* slots) {
+  pa_status s = validate(desc);
+  if (s != PA_OK) return s;
+  pa_plan_s P;
+  P.d = *desc;
+  configure(&P);
+  if ((s = check_table_size(&P)) != PA_OK) return s;
+  *bytes = plan_arena(&P, nullptr);
+  // bounds, before the tables say which forms pay: the two-frame form at the
+  // largest launch, the fine-grained ones at the most frames they are built for
+  *slots = 0;
+  int frames = 0;
+  if (desc->max_batch > 1 && P.K <= 5 && slot_item_bytes(&P, 1) <= kSlotBytesMax)
+    *slots += round256(slots_size(&P, 1, &frames));
+  const FineLimits lim = fine_limits(&P);
+  const int64_t nf = std::min<int64_t>(desc->max_batch, std::max(lim.px1, lim.px2) / frame_warps(&P));
+  if (slot_item_bytes(&P, 2) <= kSlotBytesMax)
+    *slots += round256(std::min(kSlotBytesMax, (size_t)nf * slot_item_bytes(&P, 2)) + slot_row_bytes(&P, 2));
+  return PA_OK;
+}
+
 pa_status plan_bf_params(pa_plan_s* P, const void* rf, int nf, float* out, uint32_t stages,
                          BfParams* b, int* k, bool* lattice_fp32_plain) {
   const pa_status s = fused_params(P, P->form[0], rf, nf, out, stages, P->scratch[0], b);
@@ -2416,37 +2467,17 @@ extern "C" {
 
 pa_status pa_plan(const pa_plan_desc* desc, void* cuda_stream, pa_plan_t* out) {
   if (!out) return fail(PA_EINVAL, "null output handle");
-  *out = nullptr;
-  pa_status s = validate(desc);
-  if (s != PA_OK) return s;
-  pa_plan_s* P = new (std::nothrow) pa_plan_s();
-  if (!P) return fail(PA_ENOMEM, "host allocation failed");
-  P->d = *desc;
-  configure(P);
-  s = build_plan(P, (cudaStream_t)cuda_stream);
-  if (s != PA_OK) {
-    const std::string keep = g_err;
-    free_plan(P);
-    g_err = keep;
-    return s;
-  }
-  *out = P;
-  return PA_OK;
+  return plan_create(desc, (cudaStream_t)cuda_stream, kNoSlotLimit, out);
 }
 
 pa_status pa_plan_footprint(const pa_plan_desc* desc, int32_t n_frames, size_t* bytes) {
   if (!bytes) return fail(PA_EINVAL, "null bytes pointer");
-  pa_status s = validate(desc);
-  if (s != PA_OK) return s;
   if (n_frames < 0) return fail(PA_EINVAL, "n_frames < 0");
-  pa_plan_s P;
-  P.d = *desc;
-  configure(&P);
-  if ((s = check_table_size(&P)) != PA_OK) return s;
-  size_t b = plan_arena(&P, nullptr);
+  size_t b = 0, slots = 0;
+  if (const pa_status s = plan_memory(desc, &b, &slots)) return s;
   const size_t elt = desc->rf_dtype == PA_RF_F32 ? 4 : 2;
   b += (size_t)n_frames * desc->n_elem * desc->n_samples * elt;
-  b += (size_t)n_frames * 3 * P.n_out * desc->nx * desc->nz * sizeof(float);
+  b += (size_t)n_frames * 3 * popcount3(desc->outputs) * desc->nx * desc->nz * sizeof(float);
   *bytes = b;
   return PA_OK;
 }

@@ -15,6 +15,9 @@
 // in another slot is taken, with up to max_batch - 1 later visible requests
 // of the same descriptor; the batch is admitted if its buffers (and a new
 // plan's tables) fit in the device budget next to the batches in flight.
+// A new plan gets its prepared slots, without which it runs its one-frame form,
+// only from what the budget has left; when memory is short, idle plans give
+// theirs back before any plan is evicted.
 // Completion is detected by polling each slot's event; the request's latency
 // is the server-clock time of that detection minus its arrival time.
 //
@@ -64,6 +67,7 @@ constexpr double kSpinWindow = 1e-3;
 struct PlanEntry {
   pa_plan_t plan = nullptr;
   size_t bytes = 0;
+  size_t slot_bytes = 0;  // of these, prepared slots
   bool busy = false;
   bool building = false;  // queued for, or in, the builder thread
   int tmem_cols = 0;      // > 0: compensated plan (Kahan totals in TMEM)
@@ -72,13 +76,20 @@ struct PlanEntry {
   int timeouts_seen = 0;  // timed-out waits of this plan already charged to a batch
 };
 
+// A plan for the builder thread, and the slots it may take.
+struct BuildJob {
+  std::string key;
+  pa_plan_desc desc{};
+  size_t slot_limit = 0;
+};
+
 // A plan the builder thread finished (or failed to build).
 struct Built {
   std::string key;
   pa_plan_t plan = nullptr;
   pa_status status = PA_OK;
   std::string error;
-  size_t bytes = 0;
+  size_t bytes = 0, slot_bytes = 0;
   int tmem_cols = 0;
   bool tmem_dense = false;
 };
@@ -133,7 +144,7 @@ struct pa_server_s {
   int comp_in_flight = 0, dense_in_flight = 0;  // compensated / TMEM-dense batches in flight
   int plans_count = 0;  // plans.size(), kept under mu for pa_server_get_stats
   // builder thread (queue and results guarded by mu)
-  std::deque<std::pair<std::string, pa_plan_desc>> build_q;
+  std::deque<BuildJob> build_q;
   std::vector<Built> built;
   std::condition_variable cv_build;
   bool stop_build = false;
@@ -141,7 +152,10 @@ struct pa_server_s {
   // statistics (guarded by mu)
   uint64_t submitted = 0, completed = 0, failed = 0, batches = 0;
   size_t in_use = 0, peak = 0;
+  size_t slots_reserved = 0;  // of in_use: for slots of plans being built, which may take fewer
   std::thread th;
+
+  size_t held() const { return in_use - slots_reserved; }  // (caller holds mu)
 
   double now() const {
     return std::chrono::duration<double>(clock_type::now() - t0).count();
@@ -197,9 +211,9 @@ struct pa_server_s {
     return any;
   }
 
-  // Destroy least recently used idle plans until `need` more bytes fit and,
-  // when a plan is about to be added, the resident plans stay within
-  // max_plans.
+  // Make room for `need` more bytes and, when a plan is about to be added, for
+  // it within max_plans: idle plans give their prepared slots back, least
+  // recently used first, then idle plans are destroyed in that order.
   void evict_for(size_t need, bool adding_plan) {
     for (;;) {
       size_t cur;
@@ -210,20 +224,28 @@ struct pa_server_s {
       const bool over_count =
           (int)plans.size() + (adding_plan ? 1 : 0) > std::max(1, cfg.max_plans);
       if (cur + need <= cfg.device_budget_bytes && !over_count) return;
-      auto victim = plans.end();
+      auto victim = plans.end(), holder = plans.end();
       for (auto it = plans.begin(); it != plans.end(); ++it) {
-        if (it->second.busy || it->second.building) continue;
-        if (victim == plans.end() || it->second.last_used < victim->second.last_used) victim = it;
+        const PlanEntry& pe = it->second;
+        if (pe.busy || pe.building) continue;
+        if (victim == plans.end() || pe.last_used < victim->second.last_used) victim = it;
+        if (pe.slot_bytes && (holder == plans.end() || pe.last_used < holder->second.last_used))
+          holder = it;
       }
       if (victim == plans.end()) return;
-      pa_destroy(victim->second.plan);
-      const size_t freed = victim->second.bytes;
-      plans.erase(victim);
-      {
-        std::lock_guard<std::mutex> lk(mu);
-        in_use -= freed;
-        plans_count = (int)plans.size();
+      size_t freed;
+      if (!over_count && holder != plans.end() && pa::plan_drop_slots(holder->second.plan) == PA_OK) {
+        freed = holder->second.slot_bytes;
+        holder->second.bytes -= freed;
+        holder->second.slot_bytes = 0;
+      } else {
+        pa_destroy(victim->second.plan);
+        freed = victim->second.bytes;
+        plans.erase(victim);
       }
+      std::lock_guard<std::mutex> lk(mu);
+      in_use -= freed;
+      plans_count = (int)plans.size();
     }
   }
 
@@ -255,18 +277,26 @@ struct pa_server_s {
         // requests of resident plans go on meanwhile
         pa_plan_desc d = head->desc;
         d.max_batch = cfg.max_batch;
-        size_t plan_bytes = 0;
-        if (pa_plan_footprint(&d, 0, &plan_bytes) != PA_OK) plan_bytes = 0;
+        size_t plan_bytes = 0, slots_most = 0;
+        if (pa::plan_memory(&d, &plan_bytes, &slots_most) != PA_OK) plan_bytes = slots_most = 0;
         evict_for(plan_bytes, true);
+        PlanEntry pe;
+        pe.building = true;
+        // slots from what is left beside the buffers of one full batch
+        const size_t batch = align_up(head->rf_bytes * cfg.max_batch) +
+                             align_up(head->out_bytes * cfg.max_batch);
         {
           std::lock_guard<std::mutex> lk(mu);
           if (in_use + plan_bytes > cfg.device_budget_bytes) continue;  // wait for memory
+          const size_t left = cfg.device_budget_bytes - in_use - plan_bytes;
+          const size_t slots = std::min(slots_most, left > batch ? left - batch : 0);
+          plan_bytes += slots;
+          pe.slot_bytes = slots;
           in_use += plan_bytes;
-          peak = std::max(peak, in_use);
-          build_q.emplace_back(head->key, d);
+          slots_reserved += slots;
+          peak = std::max(peak, held());
+          build_q.push_back({head->key, d, slots});
         }
-        PlanEntry pe;
-        pe.building = true;
         pe.bytes = plan_bytes;
         plans.emplace(head->key, pe);
         {
@@ -346,7 +376,7 @@ struct pa_server_s {
       }
       s.bytes = buf_rf + buf_out;
       in_use += s.bytes;
-      peak = std::max(peak, in_use);
+      peak = std::max(peak, held());
       pe.busy = true;
       pe.last_used = ++use_clock;
       ++batches;
@@ -380,6 +410,7 @@ struct pa_server_s {
       PlanEntry& pe = pit->second;
       std::lock_guard<std::mutex> lk(mu);
       in_use -= pe.bytes;  // the reservation, replaced by what the plan holds
+      slots_reserved -= pe.slot_bytes;
       if (b.status != PA_OK) {
         const double t = now();
         for (auto it = visible.begin(); it != visible.end();) {
@@ -397,11 +428,12 @@ struct pa_server_s {
       }
       pe.plan = b.plan;
       pe.bytes = b.bytes;
+      pe.slot_bytes = b.slot_bytes;
       pe.building = false;
       pe.tmem_cols = b.tmem_cols;
       pe.tmem_dense = b.tmem_dense;
       in_use += pe.bytes;
-      peak = std::max(peak, in_use);
+      peak = std::max(peak, held());
     }
     return true;
   }
@@ -409,7 +441,7 @@ struct pa_server_s {
   void build_loop() {
     cudaSetDevice(device);
     for (;;) {
-      std::pair<std::string, pa_plan_desc> job;
+      BuildJob job;
       {
         std::unique_lock<std::mutex> lk(mu);
         cv_build.wait(lk, [&] { return stop_build || !build_q.empty(); });
@@ -418,8 +450,8 @@ struct pa_server_s {
         build_q.pop_front();
       }
       Built b;
-      b.key = job.first;
-      b.status = pa_plan(&job.second, plan_stream, &b.plan);
+      b.key = job.key;
+      b.status = pa::plan_create(&job.desc, plan_stream, job.slot_limit, &b.plan);
       // Batches are launched kernel by kernel: with batch sizes 1..max_batch
       // per plan, graph launch would instantiate a new graph on the
       // scheduler thread for every new (plan, batch size), each a stall of
@@ -427,6 +459,7 @@ struct pa_server_s {
       if (b.status == PA_OK) b.status = pa_plan_use_graph(b.plan, 0);
       if (b.status == PA_OK) {
         b.bytes = pa::plan_device_bytes(b.plan);
+        b.slot_bytes = pa::plan_slot_bytes(b.plan);
         pa::plan_tmem(b.plan, &b.tmem_cols, &b.tmem_dense);
       }
       {
@@ -648,7 +681,7 @@ pa_status pa_server_get_stats(pa_server_t S, pa_server_stats* st) {
   st->completed = S->completed;
   st->failed = S->failed;
   st->batches = S->batches;
-  st->bytes_in_use = S->in_use;
+  st->bytes_in_use = S->held();
   st->bytes_peak = S->peak;
   st->plans_resident = S->plans_count;
   return PA_OK;
