@@ -213,8 +213,9 @@ struct pa_server_s {
 
   // Make room for `need` more bytes and, when a plan is about to be added, for
   // it within max_plans: idle plans give their prepared slots back, least
-  // recently used first, then idle plans are destroyed in that order.
-  void evict_for(size_t need, bool adding_plan) {
+  // recently used first, then idle plans are destroyed in that order, but for
+  // `keep`, the plan about to run.
+  void evict_for(size_t need, bool adding_plan, const PlanEntry* keep) {
     for (;;) {
       size_t cur;
       {
@@ -228,16 +229,18 @@ struct pa_server_s {
       for (auto it = plans.begin(); it != plans.end(); ++it) {
         const PlanEntry& pe = it->second;
         if (pe.busy || pe.building) continue;
-        if (victim == plans.end() || pe.last_used < victim->second.last_used) victim = it;
+        if (&pe != keep &&
+            (victim == plans.end() || pe.last_used < victim->second.last_used)) victim = it;
         if (pe.slot_bytes && (holder == plans.end() || pe.last_used < holder->second.last_used))
           holder = it;
       }
-      if (victim == plans.end()) return;
       size_t freed;
       if (!over_count && holder != plans.end() && pa::plan_drop_slots(holder->second.plan) == PA_OK) {
         freed = holder->second.slot_bytes;
         holder->second.bytes -= freed;
         holder->second.slot_bytes = 0;
+      } else if (victim == plans.end()) {
+        return;
       } else {
         pa_destroy(victim->second.plan);
         freed = victim->second.bytes;
@@ -279,7 +282,7 @@ struct pa_server_s {
         d.max_batch = cfg.max_batch;
         size_t plan_bytes = 0, slots_most = 0;
         if (pa::plan_memory(&d, &plan_bytes, &slots_most) != PA_OK) plan_bytes = slots_most = 0;
-        evict_for(plan_bytes, true);
+        evict_for(plan_bytes, true, nullptr);
         PlanEntry pe;
         pe.building = true;
         // slots from what is left beside the buffers of one full batch
@@ -316,13 +319,20 @@ struct pa_server_s {
         }
       }
       blocked.pop_back();
+      // a batch no larger than the budget holds beside the plan without its
+      // slots (pa_server_submit has seen to one frame)
+      const PlanEntry& own = pit->second;
+      int most = cfg.max_batch;
+      while (most > 1 && own.bytes - own.slot_bytes + align_up(head->rf_bytes * most) +
+                                 align_up(head->out_bytes * most) > cfg.device_budget_bytes)
+        --most;
       std::vector<std::list<Request*>::iterator> pick{it};
-      for (auto jt = std::next(it); jt != visible.end() && (int)pick.size() < cfg.max_batch; ++jt)
+      for (auto jt = std::next(it); jt != visible.end() && (int)pick.size() < most; ++jt)
         if ((*jt)->key_hash == head->key_hash && (*jt)->key == head->key) pick.push_back(jt);
       const int nf = (int)pick.size();
       const size_t buf_rf = align_up(head->rf_bytes * nf), buf_out = align_up(head->out_bytes * nf);
       const size_t need = buf_rf + buf_out;
-      evict_for(need, false);
+      evict_for(need, false, &own);
       {
         std::lock_guard<std::mutex> lk(mu);
         if (in_use + need > cfg.device_budget_bytes) return false;  // wait for memory

@@ -59,3 +59,35 @@ def test_slots_are_taken_where_the_budget_has_them():
     frames = _frames(wl, 8)
     st = _serve(wl, (3,), frames, 64 * MB, slots=1, max_batch=8)
     assert st["bytes_in_use"] > 20 * MB
+
+
+@pytest.mark.parametrize("budget_mb,slots", [(12, 1), (12, 2), (20, 2), (40, 3)])
+def test_a_batch_larger_than_the_budget_is_cut(budget_mb, slots):
+    """A plan and eight frames' buffers (4.5 + 16 MB) do not fit in the two smaller
+    budgets: the batch is cut, and the plan about to run is not evicted for its own
+    buffers.  The larger ones evict one plan for another."""
+    wl = synth.workload("cfg2")
+    _serve(wl, (3, 2, 4), _frames(wl, 8), budget_mb * MB, slots=slots, max_batch=8)
+
+
+def test_mixed_orders_under_a_tight_budget():
+    """Requests of several plans at once, two batches in flight, room for two plans."""
+    import torch
+
+    import paper_2203_14906_gb300 as pa
+    from paper_2203_14906_gb300.serving import Server
+
+    wl = synth.workload("cfg2")
+    frames = _frames(wl, 4)
+    with Server(budget_bytes=24 * MB, stages=RAW, slots=2, max_batch=4) as srv:
+        jobs = []
+        for i in range(24):
+            k, f = 2 + i % 3, frames[i % 4]
+            o = torch.zeros((1, 1, wl["nx"], wl["nz"])).pin_memory()
+            jobs.append((k, f, o, srv.submit(pa.make_desc(wl, order_k=k, outputs=1), f.data_ptr(), o.data_ptr())))
+        assert all(srv.wait(j[3], timeout_ms=60000)["status"] == 0 for j in jobs)
+        assert srv.stats()["bytes_peak"] <= 24 * MB
+    for k in (2, 3, 4):
+        with pa.Plan(pa.make_desc(wl, order_k=k, outputs=1)) as plan:
+            want = [pa.beamform(plan, f.cuda()[None], RAW).cpu()[0] for f in frames]
+        assert all(torch.equal(o, want[i % 4]) for i, (kk, f, o, t) in enumerate(jobs) if kk == k)
