@@ -192,12 +192,11 @@ typedef struct {
  * depth rows per lane group of the fused kernel, PA_ITEM_FRAMES the form of
  * the fused kernel (1: one frame per work item, 2: two where the launch and the
  * order allow it, 3 and 4: one and two pixels per thread where the launch
- * allows it; pa_plan_form says which form a launch runs).  In the
- * checked build only
- * (device bounds checks, PA_CHECK_BOUNDS), PA_INJECT_TMA_SHORTFALL makes
- * every TMA chunk expect 16 bytes more than it receives, so each block's
- * bounded wait runs out (failure-detection tests); the release build ignores
- * it.  After a PA_ETIMEOUT that was not injected (a copy that never
+ * allows it; pa_plan_form says which form a launch runs).  In the checked
+ * build only (device bounds checks, PA_CHECK_BOUNDS), PA_INJECT_TMA_SHORTFALL
+ * makes every chunk of copies expect 16 bytes more than it receives, so each
+ * block's bounded wait runs out (failure-detection tests); the release build
+ * ignores it.  After a PA_ETIMEOUT that was not injected (a copy that never
  * arrived), copies may still be in flight into the stopped blocks' shared
  * memory: destroy the plan and treat the CUDA context as suspect.
  */

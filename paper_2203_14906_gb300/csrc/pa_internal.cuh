@@ -188,7 +188,7 @@ struct BfParams {  // aligned as CUtensorMap requires
   int* err;               // error flags: 1, 2 index checks (checked builds), 8 a wait ran out
   int* timeouts;          // running count of blocks whose bounded TMA wait ran out
   int* host_flag;         // pinned host word set when one did (null before the
-                          // plan's first host-path call)
+                          // plan's first host-path call, and where no kernel waits)
   int expect_extra;       // bytes added to every chunk's expected transaction
                           // count: 0, or > 0 only to test the bounded wait
 };
@@ -323,7 +323,5 @@ pa_status plan_bf_params(pa_plan_s* P, const void* rf, int nf, float* out, uint3
 void plan_tmem(const pa_plan_s* P, int* cols, bool* dense);
 
 cudaError_t post_configure(size_t smem);
-cudaError_t post_launch(const PostParams& p, cudaStream_t s);
-cudaError_t log_launch(const LogParams& p, int num_sms, cudaStream_t s);
 
 }  // namespace pa

@@ -5,12 +5,13 @@
 // r'[n+1] - r'[n]} for linear interpolation, {r[n], r'[n], y, y'} with the base
 // root y of the sample or {r[n], r'[n]} for nearest samples.  Samples past the
 // record read as zero; the margins around the record and the row of zeros were
-// cleared when the plan was built; samples no window holds are left out.  The partner of an odd launch's last frame
-// is the frame itself (its results are not stored).  The pass also clears the
-// launch's work counter and maxima.
+// cleared when the plan was built; samples no window holds are left out.  The
+// partner of an odd launch's last frame is the frame itself (its results are not
+// stored).  The pass also clears the launch's work counter and maxima.
 //
 // Bound by the slot writes: 16 bytes per sample and frame pair against 8 read
-// (FP32), one slot per thread so that a warp's stores are contiguous.
+// (FP32); a thread takes slots a block's width apart, so that a warp's stores are
+// contiguous.
 #include <algorithm>
 
 #include "pa_bf_pipe.cuh"
