@@ -60,16 +60,19 @@ __global__ void __launch_bounds__(512, 2) k_bf_fine(const __grid_constant__ BfPa
       reinterpret_cast<int*>(smem + kPipeCountOff)[s] = 0;
     }
     *reinterpret_cast<int*>(smem + kPipeStopOff) = 0;
-    reinterpret_cast<int4*>(smem + kPipeProdOff)[1] = make_int4(0, 0, 0, 3);
+    reinterpret_cast<int4*>(smem + kPipeProdOff)[1] = make_int4(0, 0, 0, 0);
   }
   wait_previous();
   __syncthreads();
   int stage = 0, phase = 0;
-  if (warp == 0)
-    for (int s = 0; s < p.stages; ++s) {
-      produce<FULL, 8, 1>(p, smem, sbase, s, lane);
+  if (warp == 0) {
+    produce<FULL, 8, 1, true>(p, smem, sbase, 0, lane);
+    __syncwarp();
+    for (int s = 1; s < p.stages; ++s) {
+      produce<FULL, 8, 1, false>(p, smem, sbase, s, lane);
       __syncwarp();
     }
+  }
 #ifdef PA_CHECK_BOUNDS
   const int slots_lo = (int)sbase + kFineSlotOff;
   const int slots_hi = slots_lo + (p.stages * p.ncs * p.window - 1) * 8;

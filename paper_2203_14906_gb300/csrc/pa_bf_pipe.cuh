@@ -303,11 +303,16 @@ __device__ __forceinline__ void final_tmem2(float (&acc)[2][kC][NA], uint32_t tm
 // The running item and chunk live in shared memory; calls follow one another
 // (each is made by the last warp to finish the stage's previous chunk, and
 // that warp finishes no later chunk before it returns).
+// START: the block's first chunk, of the item that is its own (k_bf_fused says
+// why); the others come from the counter, which the preparation pass sets to the
+// number of blocks.  (Told apart or added here, in the loop, they cost the
+// variants at 128 registers spills: four frames of 1024 x 1024 with Kahan sums
+// 593 -> 620 us.)
 // NF frames per item.  With one (pa_bf_fine.cuh) an item is a share of a tile's
 // warps, its chunks cover the whole tile, and the channel bases are written
 // kC times, shifted by 0 .. kC - 1 channels, so that a warp whose first pixel
 // pairs with channel u + c reads aligned fours.
-template <bool FULL, int SB, int NF>
+template <bool FULL, int SB, int NF, bool START>
 __device__ __forceinline__ void produce(const BfParams& p, unsigned char* smem, uint32_t sbase,
                                      int stage, int lane) {
   int4* prod = reinterpret_cast<int4*>(smem + kPipeProdOff);
@@ -317,10 +322,10 @@ __device__ __forceinline__ void produce(const BfParams& p, unsigned char* smem, 
   __syncwarp();
   if (run.w == 2) return;  // no work left
   bool first = false;
-  if (run.w == 0 || run.w == 3) {  // 3: the block's first item (see k_bf_fused)
-    int item = (int)blockIdx.x;
-    if (run.w == 0) {
-      if (lane == 0) item = (int)gridDim.x + atomicAdd(p.counter, 1);
+  if (START || run.w == 0) {
+    int item = START ? (int)blockIdx.x : 0;
+    if constexpr (!START) {
+      if (lane == 0) item = atomicAdd(p.counter, 1);
       item = __shfl_sync(0xffffffffu, item, 0);
     }
     if (item >= p.n_items) {
@@ -409,7 +414,7 @@ __device__ __forceinline__ void leave_chunk(const BfParams& p, unsigned char* sm
   if (__shfl_sync(0xffffffffu, before, 0) != nwarps - 1) return;
   if (lane == 0) reinterpret_cast<int*>(smem + kPipeCountOff)[stage] = 0;
   __syncwarp();
-  produce<FULL, SB, NF>(p, smem, sbase, stage, lane);
+  produce<FULL, SB, NF, false>(p, smem, sbase, stage, lane);
   __syncwarp();
 }
 
@@ -436,15 +441,18 @@ __global__ void __launch_bounds__(256, pipe_blocks(K, APOD, COMP, FULL)) k_bf_pi
       reinterpret_cast<int*>(smem + kPipeCountOff)[s] = 0;
     }
     *reinterpret_cast<int*>(smem + kPipeStopOff) = 0;
-    reinterpret_cast<int4*>(smem + kPipeProdOff)[1] = make_int4(0, 0, 0, 3);
+    reinterpret_cast<int4*>(smem + kPipeProdOff)[1] = make_int4(0, 0, 0, 0);
   }
   __syncthreads();
   int stage = 0, phase = 0;
-  if (warp == 0)
-    for (int s = 0; s < p.stages; ++s) {
-      produce<FULL, SB, 2>(p, smem, sbase, s, lane);
+  if (warp == 0) {
+    produce<FULL, SB, 2, true>(p, smem, sbase, 0, lane);
+    __syncwarp();
+    for (int s = 1; s < p.stages; ++s) {
+      produce<FULL, SB, 2, false>(p, smem, sbase, s, lane);
       __syncwarp();
     }
+  }
   {
 #ifdef PA_CHECK_BOUNDS
     const int slots_lo = (int)sbase + kPipeSlotOff;

@@ -184,7 +184,7 @@ struct BfParams {  // aligned as CUtensorMap requires
                                    // slot_pitch slots
   long long slot_pitch;
   int slot_margin;        // zero slots before a row's sample 0
-  int* counter;           // work counter (zeroed before launch)
+  int* counter;           // work counter (set before launch)
   int* err;               // error flags: 1, 2 index checks (checked builds), 8 a wait ran out
   int* timeouts;          // running count of blocks whose bounded TMA wait ran out
   int* host_flag;         // pinned host word set when one did (null before the
@@ -213,6 +213,7 @@ struct PrepParams {
   int mode, order;     // slot kind (PipeMode), order of its roots
   int* zero;           // words cleared before the fused kernel (work counter, maxima)
   int n_zero;
+  int counter0;        // what the work counter starts at: the fused kernel's blocks
 };
 void prep_spec(PrepParams* p, LaunchSpec* s);
 

@@ -1868,6 +1868,11 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
     const pa_status s = fused_params(P, f, rf_r, n, out + (size_t)f0 * planes * d.nx * d.nz, stages,
                                      scratch, &rd.b);
     if (s != PA_OK) return s;
+    Step sb;
+    sb.spec.func = f.func;
+    sb.spec.grid = dim3(std::max(1, std::min(rd.b.n_items, f.blocks_per_sm * P->num_sms)));
+    sb.spec.block = dim3(f.threads);
+    sb.spec.smem = f.smem;
     if (f.slots) {
       PrepParams& pp = rd.pp;
       pp.rf = rf_r;
@@ -1885,17 +1890,13 @@ pa_status prepare_chunk(pa_plan_s* P, const void* rf, int nf, float* out, uint32
       pp.order = P->K;
       pp.zero = c->zero;
       pp.n_zero = r == 0 ? c->zero_ints : 1;  // later rounds: the work counter only
+      pp.counter0 = (int)sb.spec.grid.x;
       Step sp;
       prep_spec(&pp, &sp.spec);
       sp.args[0] = &pp;
       sp.begin = 0;
       c->steps.push_back(sp);
     }
-    Step sb;
-    sb.spec.func = f.func;
-    sb.spec.grid = dim3(std::max(1, std::min(rd.b.n_items, f.blocks_per_sm * P->num_sms)));
-    sb.spec.block = dim3(f.threads);
-    sb.spec.smem = f.smem;
     sb.args[0] = &rd.b;
     // The kernel before lets its successor come up from its start on, and blocks
     // that are placed while it still runs are not spread evenly.  So a fused

@@ -7,7 +7,7 @@
 // record read as zero; the margins around the record and the row of zeros were
 // cleared when the plan was built; samples no window holds are left out.  The
 // partner of an odd launch's last frame is the frame itself (its results are not
-// stored).  The pass also clears the launch's work counter and maxima.
+// stored).  The pass also sets the launch's work counter and clears its maxima.
 //
 // Bound by the slot writes: 16 bytes per sample and frame pair against 8 read
 // (FP32); a thread takes slots a block's width apart, so that a warp's stores are
@@ -36,7 +36,7 @@ __global__ void __launch_bounds__(256) k_prep1(const PrepParams p) {
   launch_next();
   wait_previous();
   if (blockIdx.x == 0)
-    for (int i = threadIdx.x; i < p.n_zero; i += blockDim.x) p.zero[i] = 0;
+    for (int i = threadIdx.x; i < p.n_zero; i += blockDim.x) p.zero[i] = i ? 0 : p.counter0;
   const int row = blockIdx.x / p.blocks_per_row;  // frame * N + channel
   const int part = blockIdx.x - row * p.blocks_per_row;
   const size_t a0 = (size_t)row * (size_t)p.n_samples;
@@ -57,7 +57,7 @@ __global__ void __launch_bounds__(256) k_prep(const PrepParams p) {
   launch_next();
   wait_previous();
   if (blockIdx.x == 0)
-    for (int i = threadIdx.x; i < p.n_zero; i += blockDim.x) p.zero[i] = 0;
+    for (int i = threadIdx.x; i < p.n_zero; i += blockDim.x) p.zero[i] = i ? 0 : p.counter0;
   const int row = blockIdx.x / p.blocks_per_row;  // frame pair * N + channel
   const int part = blockIdx.x - row * p.blocks_per_row;
   const int fg = row / p.n_elem;
