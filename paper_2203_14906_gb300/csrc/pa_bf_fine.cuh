@@ -18,10 +18,9 @@
 // inner steps (the totals are touched every 64).  These variants still take
 // 0.65-0.9 of the one-frame form's time where pick_form sends them.
 // Measured on GB300 (RAW images, one-frame form -> this): one frame of 128 x 128,
-// 64 channels, k = 3 18.9 -> 14.8 us; one and two frames of 256 x 256, 64
-// channels, k = 2 BF16 + Kahan 16.7 -> 14.8 and 27.4 -> 18.9; one frame of 400 x
-// 512, full table 86.8 -> 57.4; one frame of 291 x 333, 97 channels of 1501
-// samples, k = 4 27.0 -> 20.9.  The lines are in pick_form.
+// 64 channels, k = 3 16.7 -> 14.6 us; one frame of 400 x 512, 128 channels, full
+// table 84.5 -> 67.4, with two pixels a thread 55.8; one frame of 291 x 333, 97
+// channels of 1501 samples, k = 4 25.0 -> 20.8.  The lines are in fine_pays.
 #pragma once
 
 #include "pa_bf_pipe.cuh"

@@ -1696,7 +1696,7 @@ bool encode_rf_map(pa_plan_s* P, const void* rf, int nf, CUtensorMap* map) {
 // Two pixels a thread, plain sums from 50 steps and from two items an SM on, up
 // to 2400 warps (at fewer items one pixel is the better one; Kahan sums, TMA and
 // vector loads 0.8-1.05):
-//   full table, orders up to 5: 1.1-1.45;
+//   full table, orders up to 5: 1.1-1.5;
 //   lattice, by samples: order 3 1.2-1.25 up to four items an SM, 4 and 5
 //     1.08-1.13 up to three, 0.95-1.05 elsewhere.
 bool fine_pays(const pa_plan_s* P, int px, int nf) {
