@@ -1,4 +1,5 @@
-"""Throughput benchmark of the HO-DMAS hot path (one JSON line on rank 0).
+"""Throughput benchmark of the HO-DMAS hot path (one short JSON line on rank 0;
+everything measured, the other legs included, as one line on stderr before it).
 
 Default workload (cfg2 geometry): 128-element linear array, 0.3 mm pitch,
 2048 samples at 40 MHz, 512 x 512 grid over 38.4 x 40 mm; DAS, DMAS and
@@ -119,6 +120,47 @@ def config_dict(args, wl, extra=None):
     if extra:
         d.update(extra)
     return d
+
+
+def rounded(x, digits=5):
+    """x with every float in it at `digits` significant digits."""
+    if isinstance(x, float):
+        return float(f"{x:.{digits}g}")
+    if isinstance(x, dict):
+        return {k: rounded(v, digits) for k, v in x.items()}
+    return [rounded(v, digits) for v in x] if isinstance(x, (list, tuple)) else x
+
+
+def pick(d, *keys):
+    return {k: d[k] for k in keys if k in d}
+
+
+def result_line(line, extras):
+    """The one line on stdout: the measurement itself whole, of the roofline and the
+    other legs their headline figures, short enough for a record that keeps the
+    last two kilobytes of output.  Everything measured goes to stderr, as one
+    line {"details": ...}."""
+    out = dict(line)
+    out.pop("graph_path", None)
+    out["roofline"] = rounded(pick(line["roofline"], "bound", "achieved", "peak", "unit", "frac",
+                                   "traffic", "kernel_ms_per_launch"))
+    out["ms_per_step_median"] = rounded(line["ms_per_step_median"])
+    legs = {n: rounded(extras[n]["value"]) for n in ("precision_form", "nearest_form", "off_lattice_form")
+            if "value" in extras.get(n, {})}
+    if "frames_per_s" in extras.get("throughput_batch", {}):
+        legs["throughput_batch_frames_per_s"] = rounded(extras["throughput_batch"]["frames_per_s"])
+    if legs:
+        out["other_legs"] = legs
+    if "cpu_baseline" in extras:
+        out["cpu_baseline"] = rounded(pick(extras["cpu_baseline"], "value", "unit", "cores", "kind"))
+    if "serving" in extras:
+        out["serving"] = {
+            form: rounded({"p50_ms": leg["offered"]["latency_ms_p50"]["median"],
+                           "p99_ms": leg["offered"]["latency_ms_p99"]["median"],
+                           "saturated_frames_per_s": leg["saturation"]["served_frames_per_s"]["median"]}, 4)
+            for form, leg in extras["serving"].items() if isinstance(leg, dict) and "saturation" in leg}
+    out["details"] = "stderr"
+    return out
 
 
 def dist_setup(args):
@@ -1131,8 +1173,8 @@ def run_ours(args):
             "config": config_dict(args, wl), "clocks": clocks, "e2e": e2e,
             "gpu_launches": launches, "roofline": roofline, "graph_path": graph_path,
         }
-        line.update(extras)
-        print(json.dumps(line), flush=True)
+        print(json.dumps({"details": dict(line, **extras)}), file=sys.stderr, flush=True)
+        print(json.dumps(result_line(line, extras)), flush=True)
     if pg is not None:
         pg.barrier()
         pg.destroy_process_group()
