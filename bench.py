@@ -158,7 +158,7 @@ def result_line(line, extras):
             form: rounded({"p50_ms": leg["offered"]["latency_ms_p50"]["median"],
                            "p99_ms": leg["offered"]["latency_ms_p99"]["median"],
                            "saturated_frames_per_s": leg["saturation"]["served_frames_per_s"]["median"]}, 4)
-            for form, leg in extras["serving"].items() if isinstance(leg, dict) and "saturation" in leg}
+            for form, leg in extras["serving"].items() if form in ("bf16_kahan", "fp32")}
     out["details"] = "stderr"
     return out
 

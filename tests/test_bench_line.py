@@ -35,7 +35,7 @@ def _leg(n):
 def test_the_line_is_short_and_keeps_the_measurement():
     line = _line()
     extras = {"serving": {"workload": "w" * 500, "bf16_kahan": _leg(2000), "fp32": _leg(2000),
-                          "paired": {"x": list(range(2000))}},
+                          "paired": {"saturation": {"pairs": 3}, "offered": {"pairs": list(range(2000))}}},
               "precision_form": {"value": 1630.12345678, "more": "m" * 500},
               "nearest_form": {"value": 2116.1}, "off_lattice_form": {"value": 1286.4},
               "throughput_batch": {"frames_per_s": 24246.81234, "kernels": list(range(500))},
