@@ -144,9 +144,9 @@ __host__ __device__ constexpr int packed_sums(int k, bool apod, bool comp, bool 
 // Blocks per SM.  Orders <= 2 have 24 sums a thread and run 24 warps a SM on 80
 // registers (16 warps: nearest k = 2 174 us instead of 153; 32 warps on 64
 // registers: 168), but for Kahan sums over the full aperture: their folds leave
-// room for one set of table entries only there, which takes 222 us instead of 230
-// in a full launch, but 33.0 instead of 31.9 in one of 200 blocks (six BF16 frames
-// of 256 x 256) and 289 instead of 285 with wide windows.  With the full table 80
+// room for one set of table entries only there, and over 350 plans of 2-48 frames
+// 24 warps take 1.04-1.18 of the time of 16, however the launch fills the GPU (one
+// full launch of 32 frames took 0.965).  With the full table 80
 // registers spill (entries and weights of three steps at once: up to 134 bytes) and
 // fewer loads are in flight; over 500 plans of 2-48 frames 24 warps take 1.17-1.20
 // of the time of 16 (apodised 1.26-1.37, with Kahan sums 1.16-1.26; nearest samples
